@@ -152,6 +152,14 @@ struct ff_ctx {
   __nv_bfloat16* WenvT_b[FF_MAX_LAYERS + 1] = {nullptr};
   __nv_bfloat16* Wlat_b[FF_MAX_LAYERS + 1][4] = {{nullptr}};
   __nv_bfloat16* WlatT_b[FF_MAX_LAYERS + 1][4] = {{nullptr}};
+  // FP32 path on the tensor cores: three bf16 slices of every dense weight matrix, laid out
+  // as the W^T [out][in] (forward) and W [in][out] (adjoint) operands
+  __nv_bfloat16* wbuf_s = nullptr;
+  __nv_bfloat16* W2b_s[4] = {nullptr}; __nv_bfloat16* W2bT_s[4] = {nullptr};
+  __nv_bfloat16* Wenv_s[FF_MAX_LAYERS + 1] = {nullptr};
+  __nv_bfloat16* WenvT_s[FF_MAX_LAYERS + 1] = {nullptr};
+  __nv_bfloat16* Wlat_s[FF_MAX_LAYERS + 1][4] = {{nullptr}};
+  __nv_bfloat16* WlatT_s[FF_MAX_LAYERS + 1][4] = {{nullptr}};
   bool gemm_fail = false;
   // system
   int n = 0, n_sys = 0, pbc[3] = {0, 0, 0};
@@ -455,6 +463,39 @@ int upload_weights(ff_ctx* c) {
   FF_TRY(dalloc(c, &c->wbuf, host.size()));
   FF_CK(c, cudaMemcpy(c->wbuf, host.data(), host.size() * sizeof(float), cudaMemcpyHostToDevice));
   for (auto& f : fix) *f.first = c->wbuf + f.second;
+  if (c->hp.precision == 0) {
+    // bf16 slices of the dense weights for the FP32 GEMM on the tensor cores
+    std::vector<std::pair<__nv_bfloat16**, size_t>> at;
+    std::vector<std::pair<const float*, std::pair<int, int>>> src;   // [rows][cols] FP32
+    size_t total = 0;
+    auto add = [&](__nv_bfloat16** dst, const float* w, int rows, int cols) {
+      at.push_back({dst, total});
+      src.push_back({w, {rows, cols}});
+      total += ((size_t)3 * rows * cols + 127) / 128 * 128;
+    };
+    auto both = [&](__nv_bfloat16** w_s, __nv_bfloat16** wt_s, const float* w, const float* wt,
+                    const std::string& name) {
+      const Tensor* t = find_tensor(c, name);
+      add(w_s, w, t->rows, t->cols);
+      add(wt_s, wt, t->cols, t->rows);
+    };
+    for (int k = 1; k < c->n2b; ++k)
+      both(&c->W2b_s[k], &c->W2bT_s[k], c->W2b[k], c->W2bT[k], "W2b." + std::to_string(k));
+    for (int L = 1; L <= c->NL; ++L) {
+      both(&c->Wenv_s[L], &c->WenvT_s[L], c->Wenv[L], c->WenvT[L], "Wenv." + std::to_string(L));
+      for (int k = 0; k < c->nlat; ++k)
+        both(&c->Wlat_s[L][k], &c->WlatT_s[L][k], c->Wlat[L][k], c->WlatT[L][k],
+             "Wlat." + std::to_string(L) + "." + std::to_string(k));
+    }
+    FF_TRY(dalloc(c, &c->wbuf_s, total));
+    for (size_t i = 0; i < at.size(); ++i) {
+      *at[i].first = c->wbuf_s + at[i].second;
+      launch_split_weights(src[i].first, src[i].second.first, src[i].second.second, *at[i].first,
+                           nullptr);
+    }
+    FF_CK(c, cudaGetLastError());
+    FF_CK(c, cudaStreamSynchronize(nullptr));
+  }
   if (c->hp.precision != 1) return FF_OK;
   // bf16 copies (rounded once from the FP64 draws) for the tensor-core GEMMs
   std::vector<__nv_bfloat16> hb;
@@ -814,13 +855,14 @@ void plan_chunks(const ff_ctx* c, long long cap, std::vector<int>& starts) {
   }
 }
 
-// C = alpha A B with the precision of the context: FP32 CUDA-core GEMM (A32, W32 [K][N])
-// or BF16 tensor-core GEMM (Ab, Wt_b = W^T [N][K]).
+// C = alpha A B with the precision of the context: FP32 (A32; Wt_s = bf16 slices of W^T
+// [N][K]) or BF16 (Ab, Wt_b = W^T [N][K]).
 void mlp_gemm(ff_ctx* c, int mode, long long M, int N, int K, const float* A32,
-              const __nv_bfloat16* Ab, int lda, const float* W32, const __nv_bfloat16* Wt_b,
-              const EpiParams& ep, cudaStream_t s) {
+              const __nv_bfloat16* Ab, int lda, const __nv_bfloat16* Wt_s,
+              const __nv_bfloat16* Wt_b, const EpiParams& ep, cudaStream_t s) {
   if (c->hp.precision == 0) {
-    launch_gemm_f32(mode, (int)M, N, K, A32, lda, W32, N, ep, s);
+    if (!launch_gemm_f32(mode, (int)M, N, K, A32, lda, Wt_s, ep, c->flags, s))
+      c->gemm_fail = true;
     return;
   }
   EpiParams e2 = ep;
@@ -868,7 +910,7 @@ void forward_chunk(ff_ctx* c, const double* pos, int a0, int a1, float* E_atom, 
         ep.out = c->h2b[k]; ep.ldo = wout;
       }
       mlp_gemm(c, last ? EPI_SILU_F : EPI_SILU, Ec, wout, win, c->h2b[k - 1], c->h2bb[k - 1], win,
-               c->W2b[k], c->W2bT_b[k], ep, s);
+               c->W2bT_s[k], c->W2bT_b[k], ep, s);
     }
   }
   const float inv_sqrt_nu = (float)(1.0 / sqrt((double)hp.avg_num_neighbors));
@@ -877,8 +919,8 @@ void forward_chunk(ff_ctx* c, const double* pos, int a0, int a1, float* E_atom, 
     ep.alpha = (float)(1.0 / sqrt((double)c->D));
     if (tc) { ep.outb = c->Wvb[L]; ep.ldob = c->ldw; }
     else { ep.out = c->Wv[L]; ep.ldo = c->ldw; }
-    mlp_gemm(c, EPI_STORE, Ec, c->ldw, c->D, c->X[L - 1], c->Xb[L - 1], c->ldx, c->Wenv[L],
-             c->WenvT_b[L], ep, s);
+    mlp_gemm(c, EPI_STORE, Ec, c->ldw, c->D, c->X[L - 1], c->Xb[L - 1], c->ldx,
+             c->WenvT_s[L], c->WenvT_b[L], ep, s);
     const int last = L == c->NL ? 1 : 0;
     launch_env_tp_fwd(c->lmax, c->layer_ink[L], c->layer_outk[L], c->C, na, rp, e0, c->ef,
                       tc ? (const void*)c->Wvb[L] : (const void*)c->Wv[L], tc ? 1 : 0, c->ldw, L >= 2 ? c->V[L - 1] : nullptr,
@@ -904,8 +946,8 @@ void forward_chunk(ff_ctx* c, const double* pos, int a0, int a1, float* E_atom, 
         el.wv = c->w_eff;
         el.outb = c->GZL; el.ldob = c->D;
         el.eout = c->E_edge; el.gfo = c->gfL;
-        mlp_gemm(c, EPI_HEAD, Ec, wout, fan, A32, Ab, lda, c->Wlat[L][k], c->WlatT_b[L][k], el,
-                 s);
+        mlp_gemm(c, EPI_HEAD, Ec, wout, fan, A32, Ab, lda, c->WlatT_s[L][k],
+                 c->WlatT_b[L][k], el, s);
         break;
       }
       if (lastk) {
@@ -924,8 +966,8 @@ void forward_chunk(ff_ctx* c, const double* pos, int a0, int a1, float* E_atom, 
       } else {
         el.out = c->hlat[L][k]; el.ldo = wout;
       }
-      mlp_gemm(c, lastk ? EPI_SILU_RES : EPI_SILU, Ec, wout, fan, A32, Ab, lda, c->Wlat[L][k],
-               c->WlatT_b[L][k], el, s);
+      mlp_gemm(c, lastk ? EPI_SILU_RES : EPI_SILU, Ec, wout, fan, A32, Ab, lda,
+               c->WlatT_s[L][k], c->WlatT_b[L][k], el, s);
       A32 = c->hlat[L][k];
       Ab = c->hlatb[L][k];
       fan = lda = wout;
@@ -983,7 +1025,7 @@ void backward_chunk(ff_ctx* c, int a0, int a1, const double* seed, cudaStream_t 
       else { ep.out = c->GZ[gzb ^ 1]; ep.ldo = hp.latent[k - 1]; }
       ep.z = c->zlat[L][k - 1]; ep.zb = c->zlatb[L][k - 1]; ep.ldz = hp.latent[k - 1];
       mlp_gemm(c, EPI_DSILU, Ec, hp.latent[k - 1], hp.latent[k], c->GZ[gzb], gzA,
-               hp.latent[k], c->WlatT[L][k], c->Wlat_b[L][k], ep, s);
+               hp.latent[k], c->Wlat_s[L][k], c->Wlat_b[L][k], ep, s);
       gzb ^= 1;
       gzA = c->GZb[gzb];
     }
@@ -1001,7 +1043,7 @@ void backward_chunk(ff_ctx* c, int a0, int a1, const double* seed, cudaStream_t 
       ep.out = c->GX[cur]; ep.ldo = c->ldx;
       ep.res = gx; ep.ldr = ldgx; ep.beta = r2; ep.split = c->D;
       mlp_gemm(c, EPI_RES, Ec, c->ldx, hp.latent[0], c->GZ[gzb], gzA, hp.latent[0],
-               c->WlatT[L][0], c->Wlat_b[L][0], ep, s);
+               c->Wlat_s[L][0], c->Wlat_b[L][0], ep, s);
     }
     const int last = L == c->NL ? 1 : 0;
     launch_env_tp_bwd(c->lmax, c->layer_ink[L], c->layer_outk[L], c->C, na, rp, e0, c->ef,
@@ -1045,7 +1087,7 @@ void backward_chunk(ff_ctx* c, int a0, int a1, const double* seed, cudaStream_t 
       EpiParams ep{};
       ep.alpha = (float)(1.0 / sqrt((double)c->D));
       ep.out = c->GX[cur]; ep.ldo = c->ldx;
-      mlp_gemm(c, EPI_ACC, Ec, c->D, c->ldw, c->GW, c->GWb, c->ldw, c->WenvT[L], c->Wenv_b[L],
+      mlp_gemm(c, EPI_ACC, Ec, c->D, c->ldw, c->GW, c->GWb, c->ldw, c->Wenv_s[L], c->Wenv_b[L],
                ep, s);
     }
     gx = c->GX[cur];
@@ -1067,7 +1109,7 @@ void backward_chunk(ff_ctx* c, int a0, int a1, const double* seed, cudaStream_t 
     else { ep.out = c->GZ[gzb ^ 1]; ep.ldo = hp.two_body[k - 1]; }
     ep.z = c->z2b[k - 1]; ep.zb = c->z2bb[k - 1]; ep.ldz = hp.two_body[k - 1];
     mlp_gemm(c, EPI_DSILU, Ec, hp.two_body[k - 1], hp.two_body[k], c->GZ[gzb], c->GZb[gzb],
-             hp.two_body[k], c->W2bT[k], c->W2b_b[k], ep, s);
+             hp.two_body[k], c->W2b_s[k], c->W2b_b[k], ep, s);
     gzb ^= 1;
   }
   const int w0 = hp.two_body[0];
@@ -1228,9 +1270,8 @@ int ff_create(ff_ctx** out, const ff_hparams* hp, uint64_t seed) {
   *out = nullptr;
   std::string why;
   if (!validate(*hp, why)) return set_err(nullptr, FF_ERR_ARG, why);
-  if (hp->precision == 1 && !gemm_bf16_available())
-    return set_err(nullptr, FF_ERR_ARG,
-                   "BF16 tensor-core path unavailable (no tensor-map encoder)");
+  if (!gemm_bf16_available())
+    return set_err(nullptr, FF_ERR_ARG, "tensor-core path unavailable (no tensor-map encoder)");
   ff_ctx* c = new ff_ctx();
   c->hp = *hp;
   c->seed = seed;
@@ -1266,7 +1307,7 @@ void ff_destroy(ff_ctx* c) {
   if (c->ev_a) cudaEventDestroy(c->ev_a);
   if (c->ev_b) cudaEventDestroy(c->ev_b);
   free_workspace(c);
-  dfree(c->wbuf); dfree(c->wbuf_b); dfree(c->Z); dfree(c->sys_ptr); dfree(c->sys_of);
+  dfree(c->wbuf); dfree(c->wbuf_b); dfree(c->wbuf_s); dfree(c->Z); dfree(c->sys_ptr); dfree(c->sys_of);
   dfree(c->L_d); dfree(c->Lf_d);
   dfree(c->vl_j); dfree(c->vl_s); dfree(c->vl_cnt); dfree(c->cell_of); dfree(c->img); dfree(c->xf);
   dfree(c->cell_count); dfree(c->cell_start); dfree(c->cell_fill); dfree(c->cell_atoms);

@@ -90,8 +90,13 @@ struct EpiParams {
   int test_stall;
 };
 
-void launch_gemm_f32(int mode, int M, int N, int K, const float* A, int lda, const float* B,
-                     int ldb, const EpiParams& ep, cudaStream_t s);
+// FP32 GEMM on the tensor cores from three bf16 slices per operand (gemm_f32.cu): A [M][K]
+// FP32, Bs = the slices of B^T, [3][N][K] bf16, from launch_split_weights (Wt = B^T [N][K]
+// FP32).  N % 16 == 0, K % 16 == 0, lda % 8 == 0, A 32-byte aligned.  Returns false if the
+// launch could not be set up; a device-side timeout sets FF_FLAG_TIMEOUT in *err.
+void launch_split_weights(const float* Wt, int N, int K, __nv_bfloat16* out, cudaStream_t s);
+bool launch_gemm_f32(int mode, int M, int N, int K, const float* A, int lda,
+                     const __nv_bfloat16* Bs, const EpiParams& ep, int* err, cudaStream_t s);
 
 // BF16 tensor-core GEMM (tcgen05 + TMA): A bf16 [M][K] row-major, Bt = B^T bf16 [N][K]
 // row-major; N % 16 == 0, K, lda, ldb % 8 == 0, 16-byte aligned bases.  Returns false if

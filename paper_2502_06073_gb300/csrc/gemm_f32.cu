@@ -1,151 +1,595 @@
-// FP32 CUDA-core GEMM for the per-edge MLPs (the "plain FP32" precision of the path),
-// with the MLP's element-wise work fused into the epilogue (SiLU, cutoff envelope,
-// residual update, SiLU' of the adjoint).
+// FP32 GEMM of the per-edge MLPs on the tensor cores (precision mode 0):
+// C[M][N] = alpha * A[M][K] * B[K][N] with A and C FP32 and the fused element-wise epilogues
+// of the FP32 path, at least as accurate as a chain of FP32 FMAs.
 //
-// C[M][N] = alpha * A[M][K] B[K][N]; A is edge-major (one row per edge), B the weight
-// matrix.  Tile 128 x 64 x 16, 256 threads, 8 x 4 outputs per thread (packed two-wide
-// FP32 FMAs over row pairs), register double-buffered global loads, three blocks per SM
-// (80 registers, no spills).  Requires K % 16 == 0, N % 4 == 0, lda/ldb % 4 == 0 and
-// 16-byte aligned A and B.
-#include "ff_internal.cuh"
+// How.  Each operand is split into three bf16 slices, a = a1 + a2 + a3, on a fixed-point grid
+// per row and 64-element K-chunk (row of B^T: output column).  With 2^e <= max|a| < 2^(e+1)
+// over the chunk and unit u = 2^(e-7):  a1 = a rounded to a multiple of u (at most 256 u, so
+// exact in bf16), a2 = the rest rounded to a multiple of u 2^-9, a3 = what is left, rounded to
+// bf16 (an error of at most 2^-27 of the chunk's largest element).  Of the nine products of
+// slices the six larger ones are kept (a2 b3, a3 b2 and a3 b3 are 2^-27 and less of the
+// largest product):
+//     main  = sum a1 b1      integers in units u_a u_b below 2^24 in all but contrived inputs,
+//                            so the tensor core's FP32 accumulation, which truncates, is exact
+//     cross = sum a1 b2 + a2 b1 + a2 b2 + a1 b3 + a3 b1      2^-9 of main: its truncation
+//                            errors are 2^-32 of the result
+// in two tensor-memory accumulators, added once, rounded to nearest, in the epilogue.  The
+// splitting of a dot product into exactly accumulated slices follows Ozaki, Ogita, Oishi and
+// Rump, Numer. Algorithms 59 (2012) 95.
+//
+// One persistent CTA per SM walks the (128-row tile, column slice of at most 128) tiles
+// blockIdx.x, + gridDim.x, ...:
+//   warps 0-7    two epilogue groups of 4 warps; group g drains tiles j = g mod 2 (its own
+//                main and cross accumulators), so the next tile's products overlap it
+//   warps 8-15   two splitting groups of 4 warps, on alternate 128 x 32 chunks of A: two chunks
+//                in flight in registers (64 floats a thread), split and stored 64-byte swizzled
+//   warp 16      TMA producer of the pre-split weight chunks (3 x slice x 32 bf16)
+//   warp 17      MMA issuer: 6 products of M=128, N=slice, K=16 per step
+// The ring holds 3 or 4 chunks (48 KB each at a 128-column slice): with two chunks of 64
+// elements, the weight loads and the splitting of a stage could not start before the products
+// of the one before had ended.
+//
+// What bounds it.  The six products take 64 us of the latent layer's 149 us (110,000 rows,
+// K = 352, N = 256: 0.13 PFLOP/s of FP32 products, 3.3 TB/s of HBM; 64 us is what the issue
+// of the products alone measures, 107 us everything but the epilogue); the rest is latency of
+// the splitting and of the epilogue at 18 warps an SM.  The CUDA-core kernel that this one
+// replaced ran at 0.6 of the FP32 FMA peak: all 16 launches of an evaluation took 12.47 ms at
+// 358,000 edges and 67.2 ms at 1.97 million, now 4.50 and 23.8 ms; at 5,500 edges and widths
+// of 16 to 64, 0.170 and now 0.128 ms, so it serves every size.  Against 64 bits the forces
+// of those evaluations are off by 6.1e-7 and 1.3e-6 (relative, 2-norm), with FP32 FMAs by
+// 7.3e-7 and 1.5e-6.
+#include "tc_ptx.cuh"
 
 namespace {
 
-constexpr int BM = 128, BN = 64, BK = 16;
+constexpr int FS_EW = 8;                       // epilogue warps
+constexpr int FS_CW = 8;                       // splitting warps
+constexpr int FS_THREADS = 32 * (FS_EW + FS_CW + 2);
+constexpr int FS_TK = 32;                      // K elements of a chunk (64-byte rows)
+constexpr uint32_t FS_ASLICE = TM * FS_TK * 2;   // bytes of one slice of an A chunk
+constexpr int FS_AUXN = 4;                     // epilogue-input slots of a warp, 2 KB each
 
-__device__ __forceinline__ float silu_f(float z) { return z / (1.f + expf(-z)); }
-__device__ __forceinline__ float dsilu_f(float z) {
-  const float sg = 1.f / (1.f + expf(-z));
+// Modes that read an epilogue input per output element keep it 4 slots ahead and have room
+// for 3 ring stages; the others run 4.
+template <int MODE>
+__host__ __device__ constexpr bool fs_has_aux() {
+  return MODE == EPI_SILU_RES || MODE == EPI_DSILU || MODE == EPI_RES || MODE == EPI_ACC;
+}
+template <int MODE>
+__host__ __device__ constexpr int fs_stages() { return fs_has_aux<MODE>() ? 3 : 4; }
+
+// A CTA's walk over its tiles: row tile and column slice of tile blockIdx.x + k * gridDim.x,
+// advanced without a division per step.
+struct FsWalk {
+  int t, row, sl, step, drow, dsl, nsl;
+  __device__ __forceinline__ FsWalk(int t0, int step_, int nslices)
+      : t(t0), row(t0 / nslices), sl(t0 % nslices), step(step_), drow(step_ / nslices),
+        dsl(step_ % nslices), nsl(nslices) {}
+  __device__ __forceinline__ void next() {
+    t += step;
+    row += drow;
+    sl += dsl;
+    if (sl >= nsl) {
+      sl -= nsl;
+      ++row;
+    }
+  }
+};
+
+// Shared-memory matrix descriptor: K-major operand, 64-byte swizzle, rows of 64 B, 8-row core
+// groups 512 B apart; start address encoded in 16-byte units.
+__device__ __forceinline__ uint64_t smem_desc64(uint32_t addr) {
+  uint64_t d = 0;
+  d |= (uint64_t)((addr & 0x3FFFFu) >> 4);
+  d |= (uint64_t)1 << 16;              // leading byte offset (not used by swizzled K-major)
+  d |= (uint64_t)(512 >> 4) << 32;     // stride byte offset
+  d |= (uint64_t)1 << 46;              // descriptor version
+  d |= (uint64_t)4 << 61;              // 64-byte swizzle
+  return d;
+}
+
+__device__ __forceinline__ void fs_cp16(uint32_t dst, const float* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+}
+
+// Logistic sigmoid from expf and the hardware reciprocal with one Newton step,
+// r' = r + r (1 - d r): within about an ulp, and without the branch of the IEEE division,
+// which took a fifth of the SiLU epilogues' time.  The clamp keeps d finite (the sigmoid at
+// -80 is 2e-35).
+__device__ __forceinline__ float sigm_nr(float z) {
+  const float d = 1.f + expf(fminf(-z, 80.f));
+  const float r = __fdividef(1.f, d);
+  return fmaf(r, fmaf(-d, r, 1.f), r);
+}
+__device__ __forceinline__ float silu_nr(float z) { return z * sigm_nr(z); }
+__device__ __forceinline__ float dsilu_nr(float z) {
+  const float sg = sigm_nr(z);
   return sg * (1.f + z * (1.f - sg));
 }
 
+// Rounding constants of the splitting for a chunk whose largest magnitude is m: adding and
+// subtracting c rounds to a multiple of 2^-23 of c's leading bit.  Magnitudes above 2^111 are
+// clamped (they lose digits, not finiteness); a non-finite element makes the result
+// non-finite.
+__device__ __forceinline__ void split_consts(float m, float& c1, float& c2) {
+  unsigned e = __float_as_uint(m) & 0x7f800000u;
+  e = min(e, 238u << 23);
+  c1 = __uint_as_float((e + (16u << 23)) | 0x400000u);
+  c2 = __uint_as_float((e + (7u << 23)) | 0x400000u);
+}
+__device__ __forceinline__ void split3(float a, float c1, float c2, float& a1, float& a2,
+                                       float& a3) {
+  a1 = __fsub_rn(__fadd_rn(a, c1), c1);
+  const float r = __fsub_rn(a, a1);            // exact
+  a2 = __fsub_rn(__fadd_rn(r, c2), c2);
+  a3 = __fsub_rn(r, a2);                       // exact; rounded to bf16 when packed
+}
+__device__ __forceinline__ uint32_t pack2(float lo, float hi) {
+  const __nv_bfloat162 p = __floats2bfloat162_rn(lo, hi);
+  return *reinterpret_cast<const uint32_t*>(&p);
+}
+
+// 16 columns of both accumulators (at taddr and taddr + 128) for a warp's 32 lanes; the wait
+// is in the same statement, so nothing reads the registers before it
+__device__ __forceinline__ void tmem_ld16x2(uint32_t taddr, uint32_t (&v)[16],
+                                            uint32_t (&x)[16]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, "
+      "%13, %14, %15}, [%32];\n\t"
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, "
+      "%26, %27, %28, %29, %30, %31}, [%33];\n\t"
+      "tcgen05.wait::ld.sync.aligned;"
+      : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]),
+        "=r"(v[7]), "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]),
+        "=r"(v[14]), "=r"(v[15]), "=r"(x[0]), "=r"(x[1]), "=r"(x[2]), "=r"(x[3]), "=r"(x[4]),
+        "=r"(x[5]), "=r"(x[6]), "=r"(x[7]), "=r"(x[8]), "=r"(x[9]), "=r"(x[10]), "=r"(x[11]),
+        "=r"(x[12]), "=r"(x[13]), "=r"(x[14]), "=r"(x[15])
+      : "r"(taddr), "r"(taddr + 128)
+      : "memory");
+}
+
+// 32 consecutive bytes (32-byte aligned) in one load
+__device__ __forceinline__ void ld8(const float* p, float (&v)[8]) {
+  asm volatile("ld.global.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+               : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]),
+                 "=f"(v[6]), "=f"(v[7])
+               : "l"(p));
+}
+
+// Weights Wt [N][K] FP32 (K % 16 == 0) -> three slices [3][N][K] bf16; one warp per row and
+// chunk.  Run once per weight matrix, at creation.
+__global__ void k_split_weights(const float* __restrict__ Wt, int N, int K,
+                                __nv_bfloat16* __restrict__ out) {
+  const int nk = (K + FS_TK - 1) / FS_TK;
+  const long long t = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  if (t >= (long long)N * nk) return;
+  const int n = (int)(t / nk), k = (int)(t % nk) * FS_TK + (threadIdx.x & 31);
+  const size_t i = (size_t)n * K + k, sl = (size_t)N * K;
+  const float w = k < K ? Wt[i] : 0.f;
+  float m = fabsf(w), c1, c2, a1, a2, a3;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+  split_consts(m, c1, c2);
+  if (k >= K) return;
+  split3(w, c1, c2, a1, a2, a3);
+  out[i] = __float2bfloat16_rn(a1);
+  out[i + sl] = __float2bfloat16_rn(a2);
+  out[i + 2 * sl] = __float2bfloat16_rn(a3);
+}
+
+// The epilogue input of 4 columns (SILU_RES, RES: the residual; DSILU: the pre-activations;
+// ACC: the output it adds to), or null where there is none.
 template <int MODE>
-__device__ __forceinline__ void epilogue(const EpiParams& ep, int row, int col, float acc) {
-  const float v = ep.alpha * acc;
-  if (MODE == EPI_STORE) {
-    ep.out[(size_t)row * ep.ldo + col] = v;
-  } else if (MODE == EPI_SILU) {
-    ep.pre[(size_t)row * ep.ldp + col] = v;
-    ep.out[(size_t)row * ep.ldo + col] = silu_f(v);
-  } else if (MODE == EPI_SILU_F) {
-    ep.pre[(size_t)row * ep.ldp + col] = v;
-    ep.out[(size_t)row * ep.ldo + col] = ep.f[(size_t)row * ep.ldf] * silu_f(v);
-  } else if (MODE == EPI_SILU_RES) {
-    ep.pre[(size_t)row * ep.ldp + col] = v;
-    const float r = ep.res[(size_t)row * ep.ldr + col];
-    ep.out[(size_t)row * ep.ldo + col] = ep.beta * (r + ep.f[(size_t)row * ep.ldf] * silu_f(v));
-  } else if (MODE == EPI_DSILU) {
-    ep.out[(size_t)row * ep.ldo + col] = v * dsilu_f(ep.z[(size_t)row * ep.ldz + col]);
-  } else if (MODE == EPI_RES) {
-    const float r = col < ep.split ? ep.beta * ep.res[(size_t)row * ep.ldr + col] : 0.f;
-    ep.out[(size_t)row * ep.ldo + col] = v + r;
-  } else if (MODE == EPI_ACC) {
-    ep.out[(size_t)row * ep.ldo + col] += v;
-  }
+__device__ __forceinline__ const float* fs_aux(const EpiParams& ep, size_t r, int col) {
+  if (MODE == EPI_SILU_RES) return ep.res + r * ep.ldr + col;
+  if (MODE == EPI_DSILU) return ep.z + r * ep.ldz + col;
+  if (MODE == EPI_ACC) return ep.out + r * ep.ldo + col;
+  if (MODE == EPI_RES && col < ep.split) return ep.res + r * ep.ldr + col;
+  return nullptr;
 }
 
 template <int MODE>
-__global__ void __launch_bounds__(256, 3)
-k_sgemm(int M, int N, int K, const float* __restrict__ A, int lda, const float* __restrict__ B,
-        int ldb, EpiParams ep) {
-  __shared__ __align__(16) float As[2][BK][BM + 4];
-  __shared__ __align__(16) float Bs[2][BK][BN];
-  const int tid = threadIdx.x;
-  const int tx = tid & 15, ty = tid >> 4;
-  const long long row0 = (long long)blockIdx.x * BM;
-  const int col0 = blockIdx.y * BN;
+__global__ void __launch_bounds__(FS_THREADS, 1)
+k_gemm_fs(const __grid_constant__ CUtensorMap tmB, const float* __restrict__ A, int lda, int M,
+          int N, int K, int nslices, int nbw, EpiParams ep, int* __restrict__ err) {
+  constexpr int S = fs_stages<MODE>();
+  constexpr bool AUX = fs_has_aux<MODE>();
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+  const uint32_t b_slice = (uint32_t)nbw * FS_TK * 2;
+  const uint32_t st_bytes = 3 * FS_ASLICE + 3 * b_slice;
+  float* tiles = reinterpret_cast<float*>(smem + S * st_bytes);   // FS_EW x 2 KB
+  uint8_t* auxs = (uint8_t*)(tiles + FS_EW * 32 * 16);            // FS_EW x FS_AUXN x 2 KB
+  uint64_t* bars = (uint64_t*)(auxs + (AUX ? FS_EW * FS_AUXN * 2048 : 0));
+  uint64_t* fulla = bars;           // stage: slices of A stored (4 arrivals)
+  uint64_t* fullb = fulla + S;      // stage: slices of B landed
+  uint64_t* empty = fullb + S;      // stage: products that read it complete
+  uint64_t* accf = empty + S;       // accumulators of group g complete
+  uint64_t* acce = accf + 2;        // ... drained (4 arrivals)
+  uint64_t* fin = acce + 2;
+  uint32_t* tslot = (uint32_t*)(fin + 1);
+  __shared__ int s_fail;
+  __shared__ volatile int s_abort;
 
-  // loaders
-  const int a_r = tid >> 2, a_k = (tid & 3) * 4;      // rows a_r and a_r + 64
-  const int b_k = tid >> 4, b_c = (tid & 15) * 4;
-  float4 ra[2], rb;
-  auto load = [&](int k0) {
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const long long r = row0 + a_r + 64 * h;
-      ra[h] = (r < M) ? *reinterpret_cast<const float4*>(A + r * lda + k0 + a_k)
-                      : make_float4(0.f, 0.f, 0.f, 0.f);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int ntiles = ff_cdiv(M, TM) * nslices;
+  const int nk = (K + FS_TK - 1) / FS_TK;
+
+  if (threadIdx.x == 0) {
+    s_fail = 0;
+    s_abort = 0;
+    for (int q = 0; q < S; ++q) {
+      mbar_init(smem_u32(&fulla[q]), 4);
+      mbar_init(smem_u32(&fullb[q]), 1);
+      mbar_init(smem_u32(&empty[q]), 1);
     }
-    const int c = col0 + b_c;
-    rb = (c < N) ? *reinterpret_cast<const float4*>(B + (size_t)(k0 + b_k) * ldb + c)
-                 : make_float4(0.f, 0.f, 0.f, 0.f);
-  };
-  auto store = [&](int buf) {
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      As[buf][a_k + 0][a_r + 64 * h] = ra[h].x;
-      As[buf][a_k + 1][a_r + 64 * h] = ra[h].y;
-      As[buf][a_k + 2][a_r + 64 * h] = ra[h].z;
-      As[buf][a_k + 3][a_r + 64 * h] = ra[h].w;
+    for (int g = 0; g < 2; ++g) {
+      mbar_init(smem_u32(&accf[g]), 1);
+      mbar_init(smem_u32(&acce[g]), 4);
     }
-    *reinterpret_cast<float4*>(&Bs[buf][b_k][b_c]) = rb;
-  };
-
-  // acc[p][j] holds rows 2p and 2p+1 of column j: packed FP32 FMAs (two per instruction,
-  // each rounded as a scalar FMA) over the row pairs that one float4 of A delivers
-  float2 acc[4][4];
-#pragma unroll
-  for (int i = 0; i < 4; ++i)
-#pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = make_float2(0.f, 0.f);
-
-  const int nk = K / BK;
-  load(0);
-  store(0);
+    mbar_init(smem_u32(fin), 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == FS_EW + FS_CW + 1) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
+                     smem_u32(tslot)),
+                 "r"(512)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  fence_before();
   __syncthreads();
-  for (int kt = 0; kt < nk; ++kt) {
-    const int buf = kt & 1;
-    if (kt + 1 < nk) load((kt + 1) * BK);
+  fence_after();
+  const uint32_t tbase = *tslot;
+
+  if (warp >= FS_EW && warp < FS_EW + FS_CW) {
+    // ---- splitting group g: chunks q = g mod 2 of this CTA's (tile, K-chunk) sequence; two
+    // of them are in flight in registers
+    const int g = (warp - FS_EW) >> 2, w = warp & 3;
+    const int j = lane & 3, rsub = lane >> 2;
+    float v[2][4][8];
+    FsWalk it(blockIdx.x, gridDim.x, nslices);   // position (it, kc) of the next chunk to load
+    int kc = g;
+    bool more[2];
+    auto load = [&](float (&d)[4][8], bool& have) {
+      while (kc >= nk) {
+        kc -= nk;
+        it.next();
+      }
+      have = it.t < ntiles;
+      if (have) {
+        const int m0 = it.row * TM + w * 32 + rsub;
+        const int k = kc * FS_TK + 8 * j;
 #pragma unroll
-    for (int kk = 0; kk < BK; ++kk) {
-      const float4 a0 = *reinterpret_cast<const float4*>(&As[buf][kk][ty * 8]);
-      const float4 a1 = *reinterpret_cast<const float4*>(&As[buf][kk][ty * 8 + 4]);
-      const float4 b = *reinterpret_cast<const float4*>(&Bs[buf][kk][tx * 4]);
-      const float2 a[4] = {make_float2(a0.x, a0.y), make_float2(a0.z, a0.w),
-                           make_float2(a1.x, a1.y), make_float2(a1.z, a1.w)};
-      const float2 bb[4] = {make_float2(b.x, b.x), make_float2(b.y, b.y),
-                            make_float2(b.z, b.z), make_float2(b.w, b.w)};
+        for (int i = 0; i < 4; ++i) {
+          const int r = m0 + 8 * i;
+          if (r < M && k < K) {
+            ld8(A + (size_t)r * lda + k, d[i]);
+          } else {
 #pragma unroll
-      for (int i = 0; i < 4; ++i)
+            for (int x = 0; x < 8; ++x) d[i][x] = 0.f;
+          }
+        }
+        kc += 2;
+      }
+    };
+    uint32_t q = g;               // sequence number of the chunk being stored
+    bool good = true;
+    auto store = [&](const float (&d)[4][8]) {
+      const uint32_t st = q % S;
+      if (q >= S && !__all_sync(0xffffffffu, mbar_wait_ab(smem_u32(&empty[st]),
+                                                          (q / S - 1) & 1, &s_abort)))
+        return false;
+      uint8_t* sa = smem + (size_t)st * st_bytes;
 #pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = __ffma2_rn(a[i], bb[j], acc[i][j]);
+      for (int i = 0; i < 4; ++i) {
+        float m = 0.f;
+#pragma unroll
+        for (int x = 0; x < 8; ++x) m = fmaxf(m, fabsf(d[i][x]));
+        m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 1));
+        m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 2));
+        float c1, c2;
+        split_consts(m, c1, c2);
+        uint32_t p1[4], p2[4], p3[4];
+#pragma unroll
+        for (int x = 0; x < 4; ++x) {
+          float a1, a2, a3, b1, b2, b3;
+          split3(d[i][2 * x], c1, c2, a1, a2, a3);
+          split3(d[i][2 * x + 1], c1, c2, b1, b2, b3);
+          p1[x] = pack2(a1, b1);
+          p2[x] = pack2(a2, b2);
+          p3[x] = pack2(a3, b3);
+        }
+        const int r = w * 32 + 8 * i + rsub;
+        uint8_t* dst = sa + r * 64 + ((j ^ ((r >> 1) & 3)) << 4);
+        *reinterpret_cast<uint4*>(dst) = make_uint4(p1[0], p1[1], p1[2], p1[3]);
+        *reinterpret_cast<uint4*>(dst + FS_ASLICE) = make_uint4(p2[0], p2[1], p2[2], p2[3]);
+        *reinterpret_cast<uint4*>(dst + 2 * FS_ASLICE) = make_uint4(p3[0], p3[1], p3[2], p3[3]);
+      }
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      __syncwarp();
+      if (lane == 0) mbar_arrive(smem_u32(&fulla[st]));
+      q += 2;
+      return true;
+    };
+    load(v[0], more[0]);
+    load(v[1], more[1]);
+    while (good && more[0]) {
+      good = store(v[0]);
+      load(v[0], more[0]);
+      if (!good || !more[1]) break;
+      good = store(v[1]);
+      load(v[1], more[1]);
     }
-    if (kt + 1 < nk) {
-      store(buf ^ 1);
-      __syncthreads();
+    if (!good && lane == 0) {
+      s_fail = 1;
+      s_abort = 1;
+    }
+  } else if (warp == FS_EW + FS_CW) {
+    // ---- TMA producer of the weight slices
+    if (lane == 0) {
+      uint32_t q = 0;
+      bool good = true;
+      for (int t = blockIdx.x; t < ntiles && good; t += gridDim.x) {
+        const int n0 = (t % nslices) * nbw;
+        for (int kc = 0; kc < nk; ++kc, ++q) {
+          const uint32_t st = q % S;
+          if (q >= S && !mbar_wait_ab(smem_u32(&empty[st]), (q / S - 1) & 1, &s_abort)) {
+            good = false;
+            break;
+          }
+          uint8_t* sb = smem + (size_t)st * st_bytes + 3 * FS_ASLICE;
+          mbar_expect_tx(smem_u32(&fullb[st]), 3 * b_slice);
+          for (int sl = 0; sl < 3; ++sl)
+            tma_load_2d(smem_u32(sb + sl * b_slice), &tmB, kc * FS_TK, sl * N + n0,
+                        smem_u32(&fullb[st]));
+        }
+      }
+      if (!good) {
+        s_fail = 1;
+        s_abort = 1;
+      }
+      // the loads issued last land before the CTA may exit
+      for (uint32_t k = 0; k < S && k < q; ++k) {
+        const uint32_t p = q - 1 - k;
+        mbar_wait(smem_u32(&fullb[p % S]), (p / S) & 1);
+      }
+    }
+  } else if (warp == FS_EW + FS_CW + 1) {
+    // ---- MMA issuer
+    if (lane == 0) {
+      uint32_t q = 0;
+      bool good = true;
+      int jt = 0;
+      for (int t = blockIdx.x; t < ntiles && good; t += gridDim.x, ++jt) {
+        const int g = jt & 1;
+        if (jt >= 2 &&
+            !mbar_wait_ab(smem_u32(&acce[g]), (uint32_t)(((jt >> 1) - 1) & 1), &s_abort)) {
+          good = false;
+          break;
+        }
+        fence_after();
+        const int ncur = min(nbw, N - (t % nslices) * nbw);
+        const uint32_t idesc = instr_desc(TM, ncur);
+        const uint32_t dmain = tbase + (uint32_t)(g * 256), dcross = dmain + 128;
+        for (int kc = 0; kc < nk; ++kc, ++q) {
+          const uint32_t st = q % S, par = (q / S) & 1;
+          if (!mbar_wait_ab(smem_u32(&fullb[st]), par, &s_abort) ||
+              !mbar_wait_ab(smem_u32(&fulla[st]), par, &s_abort)) {
+            good = false;
+            break;
+          }
+          fence_after();
+          const uint8_t* sa = smem + (size_t)st * st_bytes;
+          const uint8_t* sb = sa + 3 * FS_ASLICE;
+          uint64_t da[3], db[3];
+          for (int sl = 0; sl < 3; ++sl) {
+            da[sl] = smem_desc64(smem_u32(sa + sl * FS_ASLICE));
+            db[sl] = smem_desc64(smem_u32(sb + sl * b_slice));
+          }
+          const int nkk = min(FS_TK / 16, (K - kc * FS_TK) / 16);
+          for (int kk = 0; kk < nkk; ++kk) {
+            const uint64_t o = (uint64_t)(kk * 2);
+            const uint32_t acc = (kc > 0 || kk > 0) ? 1u : 0u;
+            mma_bf16(dmain, da[0] + o, db[0] + o, idesc, acc);
+            mma_bf16(dcross, da[0] + o, db[1] + o, idesc, acc);
+            mma_bf16(dcross, da[0] + o, db[2] + o, idesc, 1u);
+            mma_bf16(dcross, da[1] + o, db[0] + o, idesc, 1u);
+            mma_bf16(dcross, da[1] + o, db[1] + o, idesc, 1u);
+            mma_bf16(dcross, da[2] + o, db[0] + o, idesc, 1u);
+          }
+          mma_commit(smem_u32(&empty[st]));
+        }
+        if (good) mma_commit(smem_u32(&accf[g]));
+      }
+      if (!good) {
+        s_fail = 1;
+        s_abort = 1;
+      }
+      // every MMA issued above has completed before the tensor memory is released
+      mma_commit(smem_u32(fin));
+      mbar_wait(smem_u32(fin), 0);
+    }
+  } else {
+    // ---- epilogue group g, lane quadrant warp & 3: 16 columns of the warp's 32 rows at a
+    // time go through its shared tile (float4 groups XOR-swizzled, conflict-free both ways)
+    // and leave as 64-byte row segments; a lane then owns 4 columns of rows rsub + 8 i.  Every
+    // lane copies the epilogue inputs that it will read itself into its own slots, FS_AUXN
+    // - 1 column groups ahead and across tile boundaries (48 KB in flight per SM: with one
+    // group ahead in registers the residual modes ran at a third of the copy bandwidth).
+    const int g = warp >> 2, quad = warp & 3;
+    const int gq = lane & 3, rsub = lane >> 2;
+    float* tile = tiles + warp * 32 * 16;
+    uint8_t* my_aux = auxs + (size_t)warp * (FS_AUXN * 2048) + lane * 16;
+    FsWalk at(blockIdx.x + g * gridDim.x, 2 * gridDim.x, nslices);   // next columns to fetch:
+    int ac = 0;                                                      // tile, first column
+    uint32_t an = 0;                               // column groups fetched
+    auto fetch = [&]() {
+      if (at.t < ntiles) {
+        const int n0 = at.sl * nbw, mq = at.row * TM + quad * 32 + rsub;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const float* src =
+              mq + 8 * i < M ? fs_aux<MODE>(ep, (size_t)(mq + 8 * i), n0 + ac + 4 * gq) : nullptr;
+          if (src) fs_cp16(smem_u32(my_aux + (an % FS_AUXN) * 2048 + i * 512), src);
+        }
+        ac += 16;
+        if (ac >= min(nbw, N - n0)) {
+          ac = 0;
+          at.next();
+        }
+      }
+      ++an;
+      asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    uint32_t un = 0;                               // column groups used
+    if (AUX)
+      for (int k = 0; k < FS_AUXN - 1; ++k) fetch();
+    bool good = true;
+    int jt = g;
+    FsWalk it(blockIdx.x + g * gridDim.x, 2 * gridDim.x, nslices);
+    for (; it.t < ntiles; it.next(), jt += 2) {
+      const int m0 = it.row * TM + quad * 32 + rsub;
+      const int n0 = it.sl * nbw;
+      const int ncur = min(nbw, N - n0);
+      float fr[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        fr[i] = 0.f;
+        if ((MODE == EPI_SILU_F || MODE == EPI_SILU_RES) && m0 + 8 * i < M)
+          fr[i] = ep.f[(size_t)(m0 + 8 * i) * ep.ldf];
+      }
+      good = __all_sync(0xffffffffu, mbar_wait_ab(smem_u32(&accf[g]), (uint32_t)((jt >> 1) & 1),
+                                                  &s_abort));
+      if (!good) break;
+      fence_after();
+      for (int c0 = 0; c0 < ncur; c0 += 16) {
+        if (AUX) fetch();
+        {
+          uint32_t v[16], x[16];
+          tmem_ld16x2(tbase + ((uint32_t)(quad * 32) << 16) + (uint32_t)(g * 256 + c0), v, x);
+#pragma unroll
+          for (int q4 = 0; q4 < 4; ++q4) {
+            float s4[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+              s4[k] = __uint_as_float(v[4 * q4 + k]) + __uint_as_float(x[4 * q4 + k]);
+            *reinterpret_cast<float4*>(&tile[lane * 16 + 4 * (q4 ^ ((lane >> 1) & 3))]) =
+                make_float4(s4[0], s4[1], s4[2], s4[3]);
+          }
+        }
+        __syncwarp();
+        const int col = n0 + c0 + 4 * gq;
+        if (AUX) asm volatile("cp.async.wait_group %0;" ::"n"(FS_AUXN - 1) : "memory");
+        const uint8_t* ax = my_aux + (un++ % FS_AUXN) * 2048;
+        // the arithmetic runs for all rows, so that the 16 chains of a lane interleave (under a
+        // branch per row they ran four at a time); only the stores look at the row count
+        float pre[4][4], o[4][4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const int rl = 8 * i + rsub;
+          const float4 acc =
+              *reinterpret_cast<const float4*>(&tile[rl * 16 + 4 * (gq ^ ((rl >> 1) & 3))]);
+          float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+          if (AUX) a = *reinterpret_cast<const float4*>(ax + i * 512);
+          const float v[4] = {ep.alpha * acc.x, ep.alpha * acc.y, ep.alpha * acc.z,
+                              ep.alpha * acc.w};
+          const float a4[4] = {a.x, a.y, a.z, a.w};
+#pragma unroll
+          for (int k = 0; k < 4; ++k) {
+            pre[i][k] = v[k];
+            if (MODE == EPI_STORE) o[i][k] = v[k];
+            else if (MODE == EPI_SILU) o[i][k] = silu_nr(v[k]);
+            else if (MODE == EPI_SILU_F) o[i][k] = fr[i] * silu_nr(v[k]);
+            else if (MODE == EPI_SILU_RES) o[i][k] = ep.beta * (a4[k] + fr[i] * silu_nr(v[k]));
+            else if (MODE == EPI_DSILU) o[i][k] = v[k] * dsilu_nr(a4[k]);
+            else if (MODE == EPI_RES) o[i][k] = v[k] + (col < ep.split ? ep.beta * a4[k] : 0.f);
+            else o[i][k] = a4[k] + v[k];
+          }
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          if (m0 + 8 * i >= M) continue;
+          const size_t r = (size_t)(m0 + 8 * i);
+          if (MODE == EPI_SILU || MODE == EPI_SILU_F || MODE == EPI_SILU_RES)
+            *reinterpret_cast<float4*>(ep.pre + r * ep.ldp + col) =
+                make_float4(pre[i][0], pre[i][1], pre[i][2], pre[i][3]);
+          *reinterpret_cast<float4*>(ep.out + r * ep.ldo + col) =
+              make_float4(o[i][0], o[i][1], o[i][2], o[i][3]);
+        }
+        __syncwarp();   // the shared tile is free again
+      }
+      // the accumulators are free again
+      fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(smem_u32(&acce[g]));
+    }
+    if (AUX) asm volatile("cp.async.wait_all;" ::: "memory");
+    if (!good && lane == 0) {
+      s_fail = 1;
+      s_abort = 1;
     }
   }
-#pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    const long long r = row0 + ty * 8 + i;
-    if (r >= M) continue;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int c = col0 + tx * 4 + j;
-      if (c < N) epilogue<MODE>(ep, (int)r, c, (i & 1) ? acc[i >> 1][j].y : acc[i >> 1][j].x);
-    }
-  }
+  fence_before();
+  __syncthreads();
+  if (threadIdx.x == 0 && s_fail) atomicOr(err, FF_FLAG_TIMEOUT);
+  if (warp == FS_EW + FS_CW + 1)
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tbase), "r"(512)
+                 : "memory");
 }
+
+template <int MODE>
+bool launch_fs(const CUtensorMap& tb, const float* A, int lda, int M, int N, int K, int nslices,
+               int nbw, const EpiParams& ep, int* err, cudaStream_t s) {
+  static int n_sm = 0;
+  if (!n_sm) {
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+        cudaFuncSetAttribute(k_gemm_fs<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             226 * 1024) != cudaSuccess) {
+      cudaGetLastError();
+      return false;
+    }
+    n_sm = sms;
+  }
+  // ring, tiles, epilogue inputs, alignment, barriers
+  const size_t bytes = fs_stages<MODE>() * (3 * (size_t)FS_ASLICE + 3 * (size_t)nbw * FS_TK * 2) +
+                       FS_EW * 32 * 16 * 4 + (fs_has_aux<MODE>() ? FS_EW * FS_AUXN * 2048 : 0) +
+                       1024 + 256;
+  const int ntiles = ff_cdiv(M, TM) * nslices;
+  k_gemm_fs<MODE><<<ntiles < n_sm ? ntiles : n_sm, FS_THREADS, bytes, s>>>(
+      tb, A, lda, M, N, K, nslices, nbw, ep, err);
+  return true;
+}
+
+using FsFn = bool (*)(const CUtensorMap&, const float*, int, int, int, int, int, int,
+                      const EpiParams&, int*, cudaStream_t);
+// indexed by epilogue mode
+const FsFn kFs[] = {launch_fs<EPI_STORE>,    launch_fs<EPI_SILU>,  launch_fs<EPI_SILU_F>,
+                    launch_fs<EPI_SILU_RES>, launch_fs<EPI_DSILU>, launch_fs<EPI_RES>,
+                    launch_fs<EPI_ACC>};
 
 }  // namespace
 
-
-void launch_gemm_f32(int mode, int M, int N, int K, const float* A, int lda, const float* B,
-                     int ldb, const EpiParams& ep, cudaStream_t s) {
-  ProfScope ps_(PC_GEMM_F32, s);
-  if (M <= 0) return;
-  dim3 grid(ff_cdiv(M, BM), ff_cdiv(N, BN));
-  switch (mode) {
-    case EPI_STORE: k_sgemm<EPI_STORE><<<grid, 256, 0, s>>>(M, N, K, A, lda, B, ldb, ep); break;
-    case EPI_SILU: k_sgemm<EPI_SILU><<<grid, 256, 0, s>>>(M, N, K, A, lda, B, ldb, ep); break;
-    case EPI_SILU_F: k_sgemm<EPI_SILU_F><<<grid, 256, 0, s>>>(M, N, K, A, lda, B, ldb, ep); break;
-    case EPI_SILU_RES:
-      k_sgemm<EPI_SILU_RES><<<grid, 256, 0, s>>>(M, N, K, A, lda, B, ldb, ep);
-      break;
-    case EPI_DSILU: k_sgemm<EPI_DSILU><<<grid, 256, 0, s>>>(M, N, K, A, lda, B, ldb, ep); break;
-    case EPI_RES: k_sgemm<EPI_RES><<<grid, 256, 0, s>>>(M, N, K, A, lda, B, ldb, ep); break;
-    case EPI_ACC: k_sgemm<EPI_ACC><<<grid, 256, 0, s>>>(M, N, K, A, lda, B, ldb, ep); break;
-    default: return;
-  }
+void launch_split_weights(const float* Wt, int N, int K, __nv_bfloat16* out, cudaStream_t s) {
+  const long long n = (long long)N * ((K + FS_TK - 1) / FS_TK);
+  k_split_weights<<<ff_cdiv(n, 8), 256, 0, s>>>(Wt, N, K, out);
   ff_count_launch(1);
+}
+
+bool launch_gemm_f32(int mode, int M, int N, int K, const float* A, int lda,
+                     const __nv_bfloat16* Bs, const EpiParams& ep, int* err, cudaStream_t s) {
+  ProfScope ps_(PC_GEMM_F32, s);
+  if (M <= 0) return true;
+  if (mode < EPI_STORE || mode > EPI_ACC || N % 16 != 0 || K % 16 != 0 || lda % 8 != 0 ||
+      ((uintptr_t)A & 31))
+    return false;
+  const int nslices = (N + 127) / 128;
+  const int nbw = nslices == 1 ? N : 128;
+  CUtensorMap tb;
+  if (!make_map(&tb, Bs, 3LL * N, K, K, nbw, FS_TK)) return false;
+  if (!kFs[mode](tb, A, lda, M, N, K, nslices, nbw, ep, err, s)) return false;
+  ff_count_launch(1);
+  return true;
 }
