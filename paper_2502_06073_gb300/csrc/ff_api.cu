@@ -1069,6 +1069,9 @@ void backward_chunk(ff_ctx* c, int a0, int a1, const double* seed, cudaStream_t 
       int mode = EPI_RES;
       if (fuse_here) {
         mode = EPI_RES_DS;
+        // below the first layer nothing reads dE/dx itself, only the dE/dz of this epilogue
+        // (1 KB per edge of writes at D = 256)
+        if (below_2b) ep.out = nullptr;
         ep.zs = below_2b ? c->z2bb[kb] : c->zlatb[L - 1][kl];
         ep.ldzs = c->D;
         ep.alpha2 = below_2b ? 1.f : r2;
