@@ -153,10 +153,14 @@ struct ff_ctx {
   __nv_bfloat16* Wlat_b[FF_MAX_LAYERS + 1][4] = {{nullptr}};
   __nv_bfloat16* WlatT_b[FF_MAX_LAYERS + 1][4] = {{nullptr}};
   // FP32 path on the tensor cores: three bf16 slices of every dense weight matrix, laid out
-  // as the W^T [out][in] (forward) and W [in][out] (adjoint) operands
+  // as the W^T [out][in] (forward) and W [in][out] (adjoint) operands; of the first latent
+  // matrix's adjoint operand Wlat_s[L][0] holds the scalar rows D.., Bcat_s the others
+  // (concatenated with the env weights as in Bcat_b: Bcat [D][bcat_ldf] FP32)
   __nv_bfloat16* wbuf_s = nullptr;
   __nv_bfloat16* W2b_s[4] = {nullptr}; __nv_bfloat16* W2bT_s[4] = {nullptr};
-  __nv_bfloat16* Wenv_s[FF_MAX_LAYERS + 1] = {nullptr};
+  float* Bcat[FF_MAX_LAYERS + 1] = {nullptr};
+  int bcat_ldf = 0;
+  __nv_bfloat16* Bcat_s[FF_MAX_LAYERS + 1] = {nullptr};
   __nv_bfloat16* WenvT_s[FF_MAX_LAYERS + 1] = {nullptr};
   __nv_bfloat16* Wlat_s[FF_MAX_LAYERS + 1][4] = {{nullptr}};
   __nv_bfloat16* WlatT_s[FF_MAX_LAYERS + 1][4] = {{nullptr}};
@@ -214,13 +218,15 @@ struct ff_ctx {
   __nv_bfloat16* Xb[FF_MAX_LAYERS + 1] = {nullptr};
   __nv_bfloat16* GZb[2] = {nullptr};
   __nv_bfloat16* GWb = nullptr;
-  // fused readout of the tensor-core path (last latent GEMM + edge-energy head): dE_e/dz
-  // of the last latent layer, per-edge energies and the envelope-gradient seed
+  // fused readout (last latent GEMM + edge-energy head; BF16 path: D <= 256): dE_e/dz of the
+  // last latent layer, per-edge energies and the envelope-gradient seed.  FP32 path: the sums
+  // per 128-column slice, E_edge[slice][wcap] and the first slots of gfp
   bool head = false;
   __nv_bfloat16* GZL = nullptr;
+  float* GZLf = nullptr;
   float* E_edge = nullptr; float* gfL = nullptr;
   // envelope-gradient partials written by the fused RES + SiLU-adjoint GEMMs: one slot per
-  // (fused launch, 128-column slice), ecap floats each
+  // (fused launch, 128-column slice), wcap floats each
   float* gfp = nullptr; int gfp_slots = 0;
   // FF_TEST_STALL_ONCE set at creation: the next tensor-core GEMM launch withholds a
   // completion signal so that a bounded device wait runs out (tests of the timeout path)
@@ -343,7 +349,7 @@ void build_structure(ff_ctx* c) {
   c->ldx = c->D + c->ns * c->C;
   c->ldw = (hp.lmax + 1) * c->C;
   c->cgroups = c->C > 32 ? c->C / 32 : 1;
-  c->head = hp.precision == 1 && c->D <= 256 && hp.latent[hp.n_latent - 1] == c->D;
+  c->head = hp.precision == 0 || c->D <= 256;   // (the last latent width is D)
   c->maxw = c->ldx;
   for (int k = 0; k < hp.n_two_body; ++k) c->maxw = std::max(c->maxw, hp.two_body[k]);
   for (int k = 0; k < hp.n_latent; ++k) c->maxw = std::max(c->maxw, hp.latent[k]);
@@ -460,6 +466,28 @@ int upload_weights(ff_ctx* c) {
     for (size_t d = 0; d < u.size(); ++d) host[base + d] = (float)u[d];
     fix.push_back({&c->w_eff, base});
   }
+  // adjoint of the latent input and the env weights in one FP32 GEMM over [GZ | GW]: per layer
+  // Bcat [D][ld] = [Wlat[:D] | 0 | (a_env / a_lat) Wenv] with a_lat = ldx^-1/2, a_env = D^-1/2
+  // (the two fan-in scales), the first part padded to a multiple of 32
+  if (c->hp.precision == 0) {
+    const int k1p = (c->hp.latent[0] + 31) / 32 * 32;
+    c->bcat_ldf = k1p + c->ldw;
+    const double ratio = sqrt((double)c->ldx) / sqrt((double)c->D);
+    for (int L = 1; L <= c->NL; ++L) {
+      const Tensor* tl = find_tensor(c, "Wlat." + std::to_string(L) + ".0");   // [ldx][latent0]
+      const Tensor* te = find_tensor(c, "Wenv." + std::to_string(L));          // [D][ldw]
+      const size_t base = host.size();
+      host.resize(base + (size_t)c->D * c->bcat_ldf, 0.f);
+      for (int r = 0; r < c->D; ++r) {
+        float* row = host.data() + base + (size_t)r * c->bcat_ldf;
+        for (int q = 0; q < tl->cols; ++q)
+          row[q] = (float)c->params[tl->off + (size_t)r * tl->cols + q];
+        for (int q = 0; q < te->cols; ++q)
+          row[k1p + q] = (float)(ratio * c->params[te->off + (size_t)r * te->cols + q]);
+      }
+      fix.push_back({&c->Bcat[L], base});
+    }
+  }
   FF_TRY(dalloc(c, &c->wbuf, host.size()));
   FF_CK(c, cudaMemcpy(c->wbuf, host.data(), host.size() * sizeof(float), cudaMemcpyHostToDevice));
   for (auto& f : fix) *f.first = c->wbuf + f.second;
@@ -482,8 +510,12 @@ int upload_weights(ff_ctx* c) {
     for (int k = 1; k < c->n2b; ++k)
       both(&c->W2b_s[k], &c->W2bT_s[k], c->W2b[k], c->W2bT[k], "W2b." + std::to_string(k));
     for (int L = 1; L <= c->NL; ++L) {
-      both(&c->Wenv_s[L], &c->WenvT_s[L], c->Wenv[L], c->WenvT[L], "Wenv." + std::to_string(L));
-      for (int k = 0; k < c->nlat; ++k)
+      const int lat0 = c->hp.latent[0];
+      add(&c->WenvT_s[L], c->WenvT[L], c->ldw, c->D);
+      add(&c->WlatT_s[L][0], c->WlatT[L][0], lat0, c->ldx);
+      add(&c->Wlat_s[L][0], c->Wlat[L][0] + (size_t)c->D * lat0, c->ldx - c->D, lat0);
+      add(&c->Bcat_s[L], c->Bcat[L], c->D, c->bcat_ldf);
+      for (int k = 1; k < c->nlat; ++k)
         both(&c->Wlat_s[L][k], &c->WlatT_s[L][k], c->Wlat[L][k], c->WlatT[L][k],
              "Wlat." + std::to_string(L) + "." + std::to_string(k));
     }
@@ -570,17 +602,13 @@ void free_workspace(ff_ctx* c) {
 // environment adjoint, plus one per channel group for the layer-1 term of V^0 = w (x) Y.
 int gy_slices(const ff_ctx* c) { return (c->NL + 1) * c->cgroups; }
 
-// Carve every per-chunk buffer from one allocation sized for `ecap` edges / `acap` atoms.
-int ensure_workspace(ff_ctx* c, long long ecap, int acap, long long budget_edges) {
-  if (ecap <= c->wcap && acap <= c->acap) return FF_OK;
-  // grow with headroom (edge counts drift from step to step in MD, and every regrowth is
-  // a free + malloc of the whole workspace), but never beyond the chunk budget
-  ecap = std::max(std::min(ecap + ecap / 8 + 4096, std::max(budget_edges, ecap)), c->wcap);
-  acap = std::max(acap + acap / 16 + 64, c->acap);
-  free_workspace(c);
+// Every per-chunk buffer for `ecap` edges and `acap` atoms: (pointer, bytes).
+using Plan = std::vector<std::pair<void**, size_t>>;
+Plan workspace_plan(ff_ctx* c, long long ecap, long long acap) {
   const ff_hparams& hp = c->hp;
-  std::vector<std::pair<void**, size_t>> plan;   // (pointer, bytes)
+  Plan plan;
   const bool tc = hp.precision == 1;
+  const int nsl = (c->D + 127) / 128;
   auto f32 = [&](float** p, long long count) { plan.push_back({(void**)p, (size_t)count * 4}); };
   auto b16 = [&](__nv_bfloat16** p, long long count) {
     plan.push_back({(void**)p, (size_t)count * 2});
@@ -596,16 +624,18 @@ int ensure_workspace(ff_ctx* c, long long ecap, int acap, long long budget_edges
       else f32(&c->h2b[k], ecap * hp.two_body[k]);
     }
   }
-  // the tensor-core path keeps the residual stream in bf16 (its GEMM operand) and needs
-  // an FP32 copy only of x^N when the readout is not fused
+  // the tensor-core path keeps the residual stream in bf16 (its GEMM operand); x^N is stored,
+  // in FP32, only when the readout is not fused
   for (int L = 0; L <= c->NL; ++L) {
-    if (!tc || (L == c->NL && !c->head)) f32(&c->X[L], ecap * c->ldx);
+    if (L == c->NL ? !c->head : !tc) f32(&c->X[L], ecap * c->ldx);
     if (tc) b16(&c->Xb[L], ecap * c->ldx);
   }
   for (int L = 1; L <= c->NL; ++L) {
     for (int k = 0; k < c->nlat; ++k) {
-      if (tc) b16(&c->zlatb[L][k], ecap * hp.latent[k]);
-      else f32(&c->zlat[L][k], ecap * hp.latent[k]);
+      if (!(c->head && L == c->NL && k == c->nlat - 1)) {   // (the fused readout keeps none)
+        if (tc) b16(&c->zlatb[L][k], ecap * hp.latent[k]);
+        else f32(&c->zlat[L][k], ecap * hp.latent[k]);
+      }
       if (k < c->nlat - 1) {
         if (tc) b16(&c->hlatb[L][k], ecap * hp.latent[k]);
         else f32(&c->hlat[L][k], ecap * hp.latent[k]);
@@ -614,7 +644,7 @@ int ensure_workspace(ff_ctx* c, long long ecap, int acap, long long budget_edges
     if (tc) b16(&c->Wvb[L], ecap * c->ldw);
     else f32(&c->Wv[L], ecap * c->ldw);
     if (L < c->NL) f32(&c->V[L], ecap * (long long)c->layer_dout[L] * c->C);
-    f32(&c->Gam[L], (long long)acap * 9 * c->C);
+    f32(&c->Gam[L], acap * 9 * c->C);
   }
   for (int b = 0; b < 2; ++b) {
     f32(&c->GX[b], ecap * c->ldx);
@@ -623,21 +653,32 @@ int ensure_workspace(ff_ctx* c, long long ecap, int acap, long long budget_edges
   }
   f32(&c->GW, ecap * c->ldw);
   f32(&c->gY, ecap * 9 * gy_slices(c));
-  f32(&c->gf, ecap);
   if (tc) {
+    f32(&c->gf, ecap);
     b16(&c->GZb[0], ecap * c->maxw);
     b16(&c->GZb[1], ecap * c->maxw);
     b16(&c->GWb, ecap * c->ldw);
   }
   if (c->head) {
-    b16(&c->GZL, ecap * c->D);
-    f32(&c->E_edge, ecap);
-    f32(&c->gfL, ecap);
+    if (tc) b16(&c->GZL, ecap * c->D);
+    else f32(&c->GZLf, ecap * c->D);
+    f32(&c->E_edge, ecap * (tc ? 1 : nsl));
+    if (tc) f32(&c->gfL, ecap);
   }
-  if (tc) {
-    c->gfp_slots = c->NL * ((c->D + 127) / 128);
-    f32(&c->gfp, ecap * c->gfp_slots);
-  }
+  c->gfp_slots = (c->NL + (tc ? 0 : 1)) * nsl;
+  f32(&c->gfp, ecap * c->gfp_slots);
+  return plan;
+}
+
+// Carve every per-chunk buffer from one allocation sized for `ecap` edges / `acap` atoms.
+int ensure_workspace(ff_ctx* c, long long ecap, int acap, long long budget_edges) {
+  if (ecap <= c->wcap && acap <= c->acap) return FF_OK;
+  // grow with headroom (edge counts drift from step to step in MD, and every regrowth is
+  // a free + malloc of the whole workspace), but never beyond the chunk budget
+  ecap = std::max(std::min(ecap + ecap / 8 + 4096, std::max(budget_edges, ecap)), c->wcap);
+  acap = std::max(acap + acap / 16 + 64, c->acap);
+  free_workspace(c);
+  const Plan plan = workspace_plan(c, ecap, acap);
   size_t total = 0;
   for (auto& p : plan) total += (p.second + 255) & ~(size_t)255;
   void* base = nullptr;
@@ -659,28 +700,16 @@ int ensure_workspace(ff_ctx* c, long long ecap, int acap, long long budget_edges
   return FF_OK;
 }
 
-size_t bytes_per_edge(const ff_ctx* c) {
-  const ff_hparams& hp = c->hp;
-  size_t b = FF_EF_STRIDE * 4 + 8 + 4;
-  for (int k = 0; k < c->n2b; ++k) b += (size_t)hp.two_body[k] * 4 * (k < c->n2b - 1 ? 2 : 1);
-  b += (size_t)(c->NL + 1) * c->ldx * 4;
-  for (int L = 1; L <= c->NL; ++L) {
-    for (int k = 0; k < c->nlat; ++k) b += (size_t)hp.latent[k] * 4 * (k < c->nlat - 1 ? 2 : 1);
-    b += (size_t)c->ldw * (hp.precision == 1 ? 2 : 4);
-    if (L < c->NL) b += (size_t)c->layer_dout[L] * c->C * 4;
-  }
-  b += 2 * ((size_t)c->ldx + c->maxw + (size_t)c->maxdim * c->C) * 4;
-  b += (size_t)c->ldw * 4 + 9 * 4 * (size_t)gy_slices(c) + 4;
-  if (hp.precision == 1)   // bf16 operands (the fp32 hidden activations are not kept)
-    b += (size_t)(c->NL + 1) * c->ldx * 2 + 2 * (size_t)c->maxw * 2 + (size_t)c->ldw * 2;
-  if (c->head) b += (size_t)c->D * 2 + 8;
+size_t bytes_per_edge(ff_ctx* c) {
+  size_t b = 0;
+  for (auto& p : workspace_plan(c, 1, 0)) b += p.second;
   return b;
 }
 
 // Edges per chunk: 120 GB (or FF_WORKSPACE_MB) of workspace, at most 60 % of the device
 // memory that is free or already held by this context's workspace.  Independent of the
 // current capacity, so the plan cannot feed back into the allocation.
-long long chunk_edge_budget(const ff_ctx* c) {
+long long chunk_edge_budget(ff_ctx* c) {
   size_t budget = (size_t)120 << 30;
   if (const char* s = getenv("FF_WORKSPACE_MB")) budget = (size_t)atoll(s) << 20;
   size_t fr = 0, tot = 0;
@@ -861,7 +890,7 @@ void mlp_gemm(ff_ctx* c, int mode, long long M, int N, int K, const float* A32,
               const __nv_bfloat16* Ab, int lda, const __nv_bfloat16* Wt_s,
               const __nv_bfloat16* Wt_b, const EpiParams& ep, cudaStream_t s) {
   if (c->hp.precision == 0) {
-    if (!launch_gemm_f32(mode, (int)M, N, K, A32, lda, Wt_s, ep, c->flags, s))
+    if (!launch_gemm_f32(mode, (int)M, N, K, A32, lda, Wt_s, K, ep, c->flags, s))
       c->gemm_fail = true;
     return;
   }
@@ -940,12 +969,14 @@ void forward_chunk(ff_ctx* c, const double* pos, int a0, int a1, float* E_atom, 
         // last latent layer + edge-energy head in one epilogue: per-edge energies, the
         // envelope-gradient seed and dE/dz of this layer; x^N itself is never stored
         el.pre = nullptr; el.preb = nullptr;
-        el.resb = c->Xb[L - 1]; el.ldr = c->ldx;
+        el.resb = c->Xb[L - 1]; el.res = c->X[L - 1]; el.ldr = c->ldx;
         el.f = fptr; el.ldf = 1;
         el.beta = (float)(1.0 / sqrt(2.0));
         el.wv = c->w_eff;
         el.outb = c->GZL; el.ldob = c->D;
+        el.out = c->GZLf; el.ldo = c->D;
         el.eout = c->E_edge; el.gfo = c->gfL;
+        el.gfp = c->gfp; el.gfp_ld = c->wcap;
         mlp_gemm(c, EPI_HEAD, Ec, wout, fan, A32, Ab, lda, c->WlatT_s[L][k],
                  c->WlatT_b[L][k], el, s);
         break;
@@ -973,7 +1004,8 @@ void forward_chunk(ff_ctx* c, const double* pos, int a0, int a1, float* E_atom, 
       fan = lda = wout;
     }
   }
-  if (c->head) launch_energy_sum(na, rp, e0, c->E_edge, E_atom + a0, s);
+  if (c->head)
+    launch_energy_sum(na, rp, e0, c->E_edge, tc ? 1 : (c->D + 127) / 128, c->wcap, E_atom + a0, s);
   else launch_energy(na, rp, e0, c->X[c->NL], c->ldx, c->D, c->w_eff, E_atom + a0, s);
 }
 
@@ -985,125 +1017,123 @@ void backward_chunk(ff_ctx* c, int a0, int a1, const double* seed, cudaStream_t 
   if (Ec <= 0) return;
   const int* rp = c->row_ptr + a0;
   const int na = a1 - a0;
-  if (c->head)   // the forward readout seeded the envelope gradient of the last layer
-    cudaMemcpyAsync(c->gf, c->gfL, (size_t)Ec * sizeof(float), cudaMemcpyDeviceToDevice, s);
-  else
-    cudaMemsetAsync(c->gf, 0, (size_t)Ec * sizeof(float), s);
   const float* gx = c->w_eff;
   int ldgx = 0;
   int cur = 0, gvb = 0;
   const float inv_sqrt_nu = (float)(1.0 / sqrt((double)hp.avg_num_neighbors));
   const float r2 = (float)(1.0 / sqrt(2.0));
-  // with the persistent tensor-core GEMM, each layer's dE/dx GEMM also applies the SiLU
-  // adjoint of the layer below (its row reduction): bf16 dE/dz out, envelope-gradient
-  // partials per 128-column slice into their own slots (summed in order by the geometric
-  // adjoint)
-  const int kb = c->n2b - 1;
-  const bool rr_fuse = tc && c->tune_stages == 0 && c->tune_slice == 128;
+  // with the persistent GEMMs, each layer's dE/dx GEMM also applies the SiLU adjoint of the
+  // layer below (its row reduction): dE/dz out, envelope-gradient partials per 128-column
+  // slice into their own slots (summed in order by the geometric adjoint); BF16 path: when
+  // that dE/dz is bf16, i.e. not below a two-body MLP of a single layer
+  const int kb = c->n2b - 1, kl = c->nlat - 1;
+  const bool rr_fuse = !tc || (c->tune_stages == 0 && c->tune_slice == 128);
   const int nsl = (c->D + 127) / 128;
-  int n_gfp = 0;
+  int n_gfp = tc ? 0 : nsl;   // (FP32: the first slots came from the readout)
+  // the envelope gradient outside the slots: BF16 path, from the readout, and from the row
+  // reductions where those run
+  const float* gf = nullptr;
+  if (tc) {
+    if (c->head && rr_fuse && kb >= 1) {
+      gf = c->gfL;
+    } else {
+      if (c->head)
+        cudaMemcpyAsync(c->gf, c->gfL, (size_t)Ec * sizeof(float), cudaMemcpyDeviceToDevice, s);
+      else
+        cudaMemsetAsync(c->gf, 0, (size_t)Ec * sizeof(float), s);
+      gf = c->gf;
+    }
+  }
   bool rr_done = false;   // dE/dz of the next layer down was produced by the last GEMM
   int zb0 = 0;            // which of the ping-pong dE/dz buffers holds this layer's
   for (int L = c->NL; L >= 1; --L) {
-    const int kl = c->nlat - 1;
     // dE/dz of this layer came from the readout or from the previous layer's GEMM
     const bool from_head = c->head && L == c->NL;
     const bool fused = from_head || rr_done;
     rr_done = false;
-    if (!fused) {
+    if (!fused) {   // BF16 path only
       zb0 = 0;
-      launch_rowred_bwd(Ec, hp.latent[kl], gx, ldgx, c->zlat[L][kl], c->zlatb[L][kl],
-                        hp.latent[kl], c->ef, r2, tc ? nullptr : c->GZ[0], hp.latent[kl],
-                        tc ? c->GZb[0] : nullptr, c->gf, s);
+      launch_rowred_bwd(Ec, hp.latent[kl], gx, ldgx, c->zlatb[L][kl], hp.latent[kl], c->ef, r2,
+                        nullptr, hp.latent[kl], c->GZb[0], c->gf, s);
     }
     int gzb = from_head ? 0 : zb0;
     const __nv_bfloat16* gzA = from_head ? c->GZL : c->GZb[gzb];
+    const float* gzF = from_head ? c->GZLf : c->GZ[gzb];
     for (int k = kl; k >= 1; --k) {
       EpiParams ep{};
       ep.alpha = (float)(1.0 / sqrt((double)hp.latent[k - 1]));
       if (tc) { ep.outb = c->GZb[gzb ^ 1]; ep.ldob = hp.latent[k - 1]; }
       else { ep.out = c->GZ[gzb ^ 1]; ep.ldo = hp.latent[k - 1]; }
       ep.z = c->zlat[L][k - 1]; ep.zb = c->zlatb[L][k - 1]; ep.ldz = hp.latent[k - 1];
-      mlp_gemm(c, EPI_DSILU, Ec, hp.latent[k - 1], hp.latent[k], c->GZ[gzb], gzA,
-               hp.latent[k], c->Wlat_s[L][k], c->Wlat_b[L][k], ep, s);
+      mlp_gemm(c, EPI_DSILU, Ec, hp.latent[k - 1], hp.latent[k], gzF, gzA, hp.latent[k],
+               c->Wlat_s[L][k], c->Wlat_b[L][k], ep, s);
       gzb ^= 1;
       gzA = c->GZb[gzb];
+      gzF = c->GZ[gzb];
     }
-    if (tc) {
+    {
       // gradients of the tensor-product scalars only (GX columns D..): the TP adjoint needs
       // them; the first D columns come after it, together with the env-weight term
       EpiParams ep{};
       ep.alpha = (float)(1.0 / sqrt((double)c->ldx));
       ep.out = c->GX[cur] + c->D; ep.ldo = c->ldx;
-      mlp_gemm(c, EPI_STORE, Ec, c->ldx - c->D, hp.latent[0], nullptr, gzA, hp.latent[0],
-               nullptr, c->Wlat_b[L][0] + (size_t)c->D * hp.latent[0], ep, s);
-    } else {
-      EpiParams ep{};
-      ep.alpha = (float)(1.0 / sqrt((double)c->ldx));
-      ep.out = c->GX[cur]; ep.ldo = c->ldx;
-      ep.res = gx; ep.ldr = ldgx; ep.beta = r2; ep.split = c->D;
-      mlp_gemm(c, EPI_RES, Ec, c->ldx, hp.latent[0], c->GZ[gzb], gzA, hp.latent[0],
-               c->Wlat_s[L][0], c->Wlat_b[L][0], ep, s);
+      mlp_gemm(c, EPI_STORE, Ec, c->ldx - c->D, hp.latent[0], gzF, gzA, hp.latent[0],
+               c->Wlat_s[L][0], tc ? c->Wlat_b[L][0] + (size_t)c->D * hp.latent[0] : nullptr, ep,
+               s);
     }
     const int last = L == c->NL ? 1 : 0;
     launch_env_tp_bwd(c->lmax, c->layer_ink[L], c->layer_outk[L], c->C, na, rp, e0, c->ef,
-                      tc ? (const void*)c->Wvb[L] : (const void*)c->Wv[L], tc ? 1 : 0, c->ldw, L >= 2 ? c->V[L - 1] : nullptr,
-                      last ? nullptr : c->theta[L], c->GX[cur], c->ldx, c->D,
-                      last ? nullptr : c->gV[gvb],
+                      tc ? (const void*)c->Wvb[L] : (const void*)c->Wv[L], tc ? 1 : 0, c->ldw,
+                      L >= 2 ? c->V[L - 1] : nullptr, last ? nullptr : c->theta[L], c->GX[cur],
+                      c->ldx, c->D, last ? nullptr : c->gV[gvb],
                       L >= 2 ? c->gV[gvb ^ 1] : nullptr, c->GW, tc ? c->GWb : nullptr,
                       c->gY + (size_t)c->NL * c->cgroups * 9,
                       c->gY + (size_t)(L - 1) * c->cgroups * 9, 9 * gy_slices(c), c->Gam[L],
                       inv_sqrt_nu, s);
-    if (tc) {
-      // dE/dx^(L-1) = a_lat GZ Wlat[:D]^T + a_env GW Wenv^T + gx / sqrt(2): one GEMM over the
-      // concatenated K of [GZ | GW] (the env part of Bcat carries a_env / a_lat)
-      EpiParams ep{};
-      ep.alpha = (float)(1.0 / sqrt((double)c->ldx));
-      ep.out = c->GX[cur]; ep.ldo = c->ldx;
-      ep.res = gx; ep.ldr = ldgx; ep.beta = r2; ep.split = c->D;
-      // the layer below: latent layer L-1 (scale 1/sqrt2) or the two-body MLP (scale 1; its
-      // dE/dz must be bf16, i.e. it has a hidden layer before the last)
-      const bool below_2b = L == 1;
-      const bool fuse_here = rr_fuse && (!below_2b || kb >= 1) &&
-                             (below_2b ? hp.two_body[kb] : hp.latent[kl]) == c->D;
-      int mode = EPI_RES;
-      if (fuse_here) {
-        mode = EPI_RES_DS;
-        // below the first layer nothing reads dE/dx itself, only the dE/dz of this epilogue
-        // (1 KB per edge of writes at D = 256)
-        if (below_2b) ep.out = nullptr;
-        ep.zs = below_2b ? c->z2bb[kb] : c->zlatb[L - 1][kl];
-        ep.ldzs = c->D;
-        ep.alpha2 = below_2b ? 1.f : r2;
-        ep.gzo = c->GZb[gzb ^ 1]; ep.ldgzo = c->D;   // not this GEMM's own operand
-        zb0 = gzb ^ 1;
-        ep.f = c->fenv; ep.ldf = 1;
-        ep.gfp = c->gfp + (size_t)n_gfp * c->wcap; ep.gfp_ld = c->wcap;
-        n_gfp += nsl;
-        rr_done = true;
-      }
-      if (!launch_gemm_bf16(mode, (int)Ec, c->D, hp.latent[0], gzA, hp.latent[0],
-                            c->Bcat_b[L], c->bcat_ld, ep, c->flags, s, c->tune_slice,
-                            c->tune_stages, c->GWb, c->ldw, c->ldw))
-        c->gemm_fail = true;
-    } else {
-      EpiParams ep{};
-      ep.alpha = (float)(1.0 / sqrt((double)c->D));
-      ep.out = c->GX[cur]; ep.ldo = c->ldx;
-      mlp_gemm(c, EPI_ACC, Ec, c->D, c->ldw, c->GW, c->GWb, c->ldw, c->Wenv_s[L], c->Wenv_b[L],
-               ep, s);
+    // dE/dx^(L-1) = a_lat GZ Wlat[:D]^T + a_env GW Wenv^T + gx / sqrt(2): one GEMM over the
+    // concatenated K of [GZ | GW] (the env part of Bcat carries a_env / a_lat)
+    EpiParams ep{};
+    ep.alpha = (float)(1.0 / sqrt((double)c->ldx));
+    ep.out = c->GX[cur]; ep.ldo = c->ldx;
+    ep.res = gx; ep.ldr = ldgx; ep.beta = r2; ep.split = c->D;
+    // the layer below: latent layer L-1 (scale 1/sqrt2) or the two-body MLP (scale 1)
+    const bool below_2b = L == 1;
+    int mode = EPI_RES;
+    if (rr_fuse && !(tc && below_2b && kb < 1)) {
+      mode = EPI_RES_DS;
+      ep.zs = below_2b ? c->z2bb[kb] : c->zlatb[L - 1][kl];
+      ep.z = below_2b ? c->z2b[kb] : c->zlat[L - 1][kl];
+      ep.ldzs = ep.ldz = c->D;
+      // below the first layer nothing reads dE/dx itself, only the dE/dz of this epilogue
+      // (1 KB per edge of writes at D = 256)
+      if (below_2b) ep.out = nullptr;
+      ep.alpha2 = below_2b ? 1.f : r2;
+      zb0 = gzb ^ 1;   // not this GEMM's own operand
+      ep.gzo = c->GZb[zb0]; ep.ldgzo = c->D;
+      ep.pre = c->GZ[zb0]; ep.ldp = c->D;
+      ep.f = c->fenv; ep.ldf = 1;
+      ep.gfp = c->gfp + (size_t)n_gfp * c->wcap; ep.gfp_ld = c->wcap;
+      n_gfp += nsl;
+      rr_done = true;
     }
+    const bool ok =
+        tc ? launch_gemm_bf16(mode, (int)Ec, c->D, hp.latent[0], gzA, hp.latent[0], c->Bcat_b[L],
+                              c->bcat_ld, ep, c->flags, s, c->tune_slice, c->tune_stages, c->GWb,
+                              c->ldw, c->ldw)
+           : launch_gemm_f32(mode, (int)Ec, c->D, hp.latent[0], gzF, hp.latent[0], c->Bcat_s[L],
+                             c->bcat_ldf, ep, c->flags, s, c->GW, c->ldw, c->ldw);
+    if (!ok) c->gemm_fail = true;
     gx = c->GX[cur];
     ldgx = c->ldx;
     cur ^= 1;
     gvb ^= 1;
   }
   // two-body MLP: x^0 = f * silu(z_last); the last gradient (dE/dz_0) stays FP32
-  const bool b16_first = tc && kb >= 1;
-  if (!rr_done)
-    launch_rowred_bwd(Ec, hp.two_body[kb], gx, ldgx, c->z2b[kb], c->z2bb[kb],
-                      hp.two_body[kb], c->ef, 1.f, b16_first ? nullptr : c->GZ[0],
-                      hp.two_body[kb], b16_first ? c->GZb[0] : nullptr, c->gf, s);
+  const bool b16_first = kb >= 1;
+  if (!rr_done)   // BF16 path only
+    launch_rowred_bwd(Ec, hp.two_body[kb], gx, ldgx, c->z2bb[kb], hp.two_body[kb], c->ef, 1.f,
+                      b16_first ? nullptr : c->GZ[0], hp.two_body[kb],
+                      b16_first ? c->GZb[0] : nullptr, c->gf, s);
   int gzb = rr_done ? zb0 : 0;
   for (int k = kb; k >= 1; --k) {
     EpiParams ep{};
@@ -1118,7 +1148,7 @@ void backward_chunk(ff_ctx* c, int a0, int a1, const double* seed, cudaStream_t 
   const int w0 = hp.two_body[0];
   const float a0f = (float)(1.0 / sqrt((double)(2 * FF_N_SPECIES + hp.n_basis)));
   launch_edge_grad(Ec, w0, hp.n_basis, hp.rc, hp.poly_p, c->lmax, c->ef, c->GZ[gzb], w0,
-                   c->W2b[0] + (size_t)2 * FF_N_SPECIES * w0, a0f, c->gf, c->gfp, n_gfp,
+                   c->W2b[0] + (size_t)2 * FF_N_SPECIES * w0, a0f, gf, c->gfp, n_gfp,
                    c->wcap, c->gY, gy_slices(c), c->src + e0, c->sys_of, seed, c->g + e0, s);
 }
 

@@ -47,7 +47,7 @@ __host__ __device__ inline void ff_unpack_shift(int p, int& a, int& b, int& c) {
   c = (int)(signed char)((p >> 16) & 0xff);
 }
 
-// Epilogue modes of the FP32 GEMM (C = alpha * A B with A [M][K] row-major, B [K][N]).
+// Epilogue modes of the GEMMs (C = alpha * A B with A [M][K] row-major, B [K][N]).
 enum EpiMode {
   EPI_STORE = 0,     // out = alpha acc
   EPI_SILU = 1,      // pre = alpha acc; out = silu(pre)
@@ -55,16 +55,18 @@ enum EpiMode {
   EPI_SILU_RES = 3,  // pre = alpha acc; out = beta (res[row, col] + f[row] silu(pre))
   EPI_DSILU = 4,     // out = alpha acc silu'(z[row, col])
   EPI_RES = 5,       // out = alpha acc + (col < split ? beta res[row * ldr + col] : 0)
-  EPI_ACC = 6,       // out += alpha acc
   // last latent layer with the edge-energy head (tensor-core GEMM, whole rows per CTA):
   // z = alpha acc, s = silu(z), x = beta (res + f s);  eout[row] = sum_col wv x,
   // gfo[row] = beta sum_col wv s,  outb = beta f silu'(z) wv  (dE_ij/dz, bf16)
-  EPI_HEAD = 7,
+  // (the FP32 GEMM: dE/dz FP32 in out, the sums per 128-column slice in eout and gfp, slices
+  // gfp_ld apart)
+  EPI_HEAD = 6,
   // tensor-core GEMM, persistent kernel only: EPI_RES, fused with the SiLU adjoint of the
   // layer below that the row reduction would otherwise do: with o the RES output and z the
   // layer's stored pre-activation (zs), gzo = alpha2 f o silu'(z) (bf16) and, per column
   // slice, gfp[slice * gfp_ld + row] = alpha2 sum_col o silu(z) (the envelope gradient)
-  EPI_RES_DS = 8
+  // (the FP32 GEMM: z and dE/dz are FP32, in z and pre)
+  EPI_RES_DS = 7
 };
 
 struct EpiParams {
@@ -91,12 +93,15 @@ struct EpiParams {
 };
 
 // FP32 GEMM on the tensor cores from three bf16 slices per operand (gemm_f32.cu): A [M][K]
-// FP32, Bs = the slices of B^T, [3][N][K] bf16, from launch_split_weights (Wt = B^T [N][K]
-// FP32).  N % 16 == 0, K % 16 == 0, lda % 8 == 0, A 32-byte aligned.  Returns false if the
-// launch could not be set up; a device-side timeout sets FF_FLAG_TIMEOUT in *err.
+// FP32, Bs = the slices of B^T, [3][N][ldb] bf16, from launch_split_weights (Wt = B^T [N][ldb]
+// FP32).  N, K % 16 == 0, lda, ldb % 8 == 0, A 32-byte aligned.  With A2 (FP32 [M][K2]) the
+// product is [A | A2] B over a concatenated K: A's columns rounded up to a multiple of 32
+// (zero-filled), then A2's; B^T has zeros in the padding.  Returns false if the launch could
+// not be set up; a device-side timeout sets FF_FLAG_TIMEOUT in *err.
 void launch_split_weights(const float* Wt, int N, int K, __nv_bfloat16* out, cudaStream_t s);
 bool launch_gemm_f32(int mode, int M, int N, int K, const float* A, int lda,
-                     const __nv_bfloat16* Bs, const EpiParams& ep, int* err, cudaStream_t s);
+                     const __nv_bfloat16* Bs, int ldb, const EpiParams& ep, int* err,
+                     cudaStream_t s, const float* A2 = nullptr, int K2 = 0, int lda2 = 0);
 
 // BF16 tensor-core GEMM (tcgen05 + TMA): A bf16 [M][K] row-major, Bt = B^T bf16 [N][K]
 // row-major; N % 16 == 0, K, lda, ldb % 8 == 0, 16-byte aligned bases.  Returns false if
@@ -172,15 +177,15 @@ void launch_env_tp_bwd(int lmax, int in_kind, int out_kind, int C, int n_atoms,
                        float inv_sqrt_nu, cudaStream_t s);
 void launch_energy(int n_atoms, const int* row_ptr, int e0, const float* X, int ldx, int D,
                    const float* w_eff, float* E_atom, cudaStream_t s);
-void launch_energy_sum(int n_atoms, const int* row_ptr, int e0, const float* E_edge,
-                       float* E_atom, cudaStream_t s);
-void launch_rowred_bwd(long long E, int N, const float* gx, int ldgx, const float* z,
-                       const __nv_bfloat16* zb, int ldz, const float* ef, float alpha,
-                       float* gz, int ldgz, __nv_bfloat16* gzb, float* gf, cudaStream_t s);
+void launch_energy_sum(int n_atoms, const int* row_ptr, int e0, const float* E_edge, int nsl,
+                       long long ld, float* E_atom, cudaStream_t s);
+void launch_rowred_bwd(long long E, int N, const float* gx, int ldgx, const __nv_bfloat16* zb,
+                       int ldz, const float* ef, float alpha, float* gz, int ldgz,
+                       __nv_bfloat16* gzb, float* gf, cudaStream_t s);
 void launch_cvt_bf16(const float* src, int lds, __nv_bfloat16* dst, int ldd, long long rows,
                      int col0, int ncols, cudaStream_t s);
-// gf: envelope gradient per edge; gfp: n_gfp further partial sums per edge (rows gfp_ld
-// apart), added to gf in order
+// gf: envelope gradient per edge or null (zero); gfp: n_gfp further partial sums per edge
+// (rows gfp_ld apart), added to it in order
 void launch_edge_grad(long long E, int w0, int n_basis, float rc, int p, int lmax,
                       const float* ef, const float* gz0, int ldg, const float* WB,
                       float alpha0, const float* gf, const float* gfp, int n_gfp,

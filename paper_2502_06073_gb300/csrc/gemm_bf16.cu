@@ -31,12 +31,12 @@ __device__ __forceinline__ float dsilu_f(float z) {
 
 // Element type of the epilogue input a mode reads per output element (0: none, 1: bf16,
 // 2: fp32): the bf16 residual stream (SILU_RES, HEAD), the bf16 pre-activations (DSILU),
-// the FP32 residual (RES) or the FP32 output it accumulates into (ACC).
+// or the FP32 residual (RES).
 template <int MODE>
 __host__ __device__ constexpr int aux_kind() {
   return (MODE == EPI_SILU_RES || MODE == EPI_HEAD || MODE == EPI_DSILU)  ? 1
-         : (MODE == EPI_RES || MODE == EPI_ACC || MODE == EPI_RES_DS) ? 2
-                                                                        : 0;
+         : (MODE == EPI_RES || MODE == EPI_RES_DS) ? 2
+                                                    : 0;
 }
 // Bytes of one warp's epilogue-input tile (32 rows x 32 columns); EPI_RES_DS adds the bf16
 // pre-activation tile of the layer below behind its FP32 residual tile.
@@ -122,9 +122,7 @@ __device__ __forceinline__ void epi_batch(const EpiParams& ep, const float4 (&ac
         else if (MODE == EPI_SILU_F) o[j] = fr[i] * silu_f(v[j]);
         else if (MODE == EPI_SILU_RES) o[j] = ep.beta * (a4[j] + fr[i] * silu_f(v[j]));
         else if (MODE == EPI_DSILU) o[j] = v[j] * dsilu_f(a4[j]);
-        else if (MODE == EPI_RES || MODE == EPI_RES_DS)
-          o[j] = v[j] + (col < ep.split ? ep.beta * a4[j] : 0.f);
-        else o[j] = a4[j] + v[j];
+        else o[j] = v[j] + (col < ep.split ? ep.beta * a4[j] : 0.f);   // RES, RES_DS
       }
       if (MODE == EPI_RES_DS) {
         // SiLU adjoint of the layer below (as its row reduction computes it)
@@ -259,8 +257,6 @@ __device__ __forceinline__ bool epi_chunk(const EpiParams& ep, uint32_t taddr, f
         const size_t r = (size_t)rows[i];
         if (MODE == EPI_RES && col < ep.split)
           aux[ii] = *reinterpret_cast<const float4*>(ep.res + r * ep.ldr + col);
-        if (MODE == EPI_ACC)
-          aux[ii] = *reinterpret_cast<const float4*>(ep.out + r * ep.ldo + col);
         if (MODE == EPI_SILU_RES || MODE == EPI_HEAD || MODE == EPI_DSILU) {
           const __nv_bfloat16* src =
               (MODE == EPI_DSILU) ? ep.zb + r * ep.ldz + col : ep.resb + r * ep.ldr + col;
@@ -801,8 +797,6 @@ int aux_map(CUtensorMap* tx, const EpiParams& ep, int M, int N) {
   } else if constexpr (MODE == EPI_RES || MODE == EPI_RES_DS) {
     return ep.ldr > 0 && ep.split > 0 &&
            make_aux_map(tx, ep.res, M, ep.split < N ? ep.split : N, (size_t)ep.ldr * 4, 4);
-  } else if constexpr (MODE == EPI_ACC) {
-    return make_aux_map(tx, ep.out, M, N, (size_t)ep.ldo * 4, 4);
   }
   return 0;
 }
@@ -904,8 +898,7 @@ using LaunchFn = bool (*)(const CUtensorMap&, const CUtensorMap&, const CUtensor
 const LaunchFn kLaunch[] = {launch_mode<EPI_STORE>, launch_mode<EPI_SILU>,
                             launch_mode<EPI_SILU_F>, launch_mode<EPI_SILU_RES>,
                             launch_mode<EPI_DSILU>, launch_mode<EPI_RES>,
-                            launch_mode<EPI_ACC>, launch_mode<EPI_HEAD>,
-                            launch_mode<EPI_RES_DS>};
+                            launch_mode<EPI_HEAD>, launch_mode<EPI_RES_DS>};
 
 }  // namespace
 

@@ -47,16 +47,21 @@ constexpr int FS_CW = 8;                       // splitting warps
 constexpr int FS_THREADS = 32 * (FS_EW + FS_CW + 2);
 constexpr int FS_TK = 32;                      // K elements of a chunk (64-byte rows)
 constexpr uint32_t FS_ASLICE = TM * FS_TK * 2;   // bytes of one slice of an A chunk
-constexpr int FS_AUXN = 4;                     // epilogue-input slots of a warp, 2 KB each
 
-// Modes that read an epilogue input per output element keep it 4 slots ahead and have room
-// for 3 ring stages; the others run 4.
+// Epilogue-input streams of a mode: the residual (SILU_RES, HEAD), the pre-activations (DSILU),
+// or both the residual gradient and the pre-activations of the layer below (RES_DS).
 template <int MODE>
-__host__ __device__ constexpr bool fs_has_aux() {
-  return MODE == EPI_SILU_RES || MODE == EPI_DSILU || MODE == EPI_RES || MODE == EPI_ACC;
+__host__ __device__ constexpr int fs_naux() {
+  return MODE == EPI_RES_DS                                                   ? 2
+         : (MODE == EPI_SILU_RES || MODE == EPI_HEAD || MODE == EPI_DSILU) ? 1
+                                                                              : 0;
 }
+// Column groups of input a warp has room for (2 KB each and stream), and ring stages, within
+// the 227 KB of a CTA.
 template <int MODE>
-__host__ __device__ constexpr int fs_stages() { return fs_has_aux<MODE>() ? 3 : 4; }
+__host__ __device__ constexpr int fs_auxn() { return MODE == EPI_RES_DS ? 2 : 4; }
+template <int MODE>
+__host__ __device__ constexpr int fs_stages() { return fs_naux<MODE>() ? 3 : 4; }
 
 // A CTA's walk over its tiles: row tile and column slice of tile blockIdx.x + k * gridDim.x,
 // advanced without a division per step.
@@ -177,30 +182,30 @@ __global__ void k_split_weights(const float* __restrict__ Wt, int N, int K,
   out[i + 2 * sl] = __float2bfloat16_rn(a3);
 }
 
-// The epilogue input of 4 columns (SILU_RES, RES: the residual; DSILU: the pre-activations;
-// ACC: the output it adds to), or null where there is none.
+// Stream u of a mode's epilogue inputs at row r, column col.
 template <int MODE>
-__device__ __forceinline__ const float* fs_aux(const EpiParams& ep, size_t r, int col) {
-  if (MODE == EPI_SILU_RES) return ep.res + r * ep.ldr + col;
+__device__ __forceinline__ const float* fs_aux(const EpiParams& ep, int u, size_t r, int col) {
   if (MODE == EPI_DSILU) return ep.z + r * ep.ldz + col;
-  if (MODE == EPI_ACC) return ep.out + r * ep.ldo + col;
-  if (MODE == EPI_RES && col < ep.split) return ep.res + r * ep.ldr + col;
-  return nullptr;
+  if (u == 1) return ep.z + r * ep.ldz + col;
+  return ep.res + r * ep.ldr + col;
 }
 
 template <int MODE>
 __global__ void __launch_bounds__(FS_THREADS, 1)
-k_gemm_fs(const __grid_constant__ CUtensorMap tmB, const float* __restrict__ A, int lda, int M,
-          int N, int K, int nslices, int nbw, EpiParams ep, int* __restrict__ err) {
+k_gemm_fs(const __grid_constant__ CUtensorMap tmB, const float* __restrict__ A, int lda,
+          const float* __restrict__ A2, int lda2, int M, int N, int K1, int K2, int nslices,
+          int nbw, EpiParams ep, int* __restrict__ err) {
   constexpr int S = fs_stages<MODE>();
-  constexpr bool AUX = fs_has_aux<MODE>();
+  constexpr int NAUX = fs_naux<MODE>(), AUXN = fs_auxn<MODE>();
+  constexpr int SLOT = NAUX * 2048;                               // bytes of a column group
+  constexpr bool AUX = NAUX > 0;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   const uint32_t b_slice = (uint32_t)nbw * FS_TK * 2;
   const uint32_t st_bytes = 3 * FS_ASLICE + 3 * b_slice;
   float* tiles = reinterpret_cast<float*>(smem + S * st_bytes);   // FS_EW x 2 KB
-  uint8_t* auxs = (uint8_t*)(tiles + FS_EW * 32 * 16);            // FS_EW x FS_AUXN x 2 KB
-  uint64_t* bars = (uint64_t*)(auxs + (AUX ? FS_EW * FS_AUXN * 2048 : 0));
+  uint8_t* auxs = (uint8_t*)(tiles + FS_EW * 32 * 16);            // FS_EW x AUXN x SLOT
+  uint64_t* bars = (uint64_t*)(auxs + FS_EW * AUXN * SLOT);
   uint64_t* fulla = bars;           // stage: slices of A stored (4 arrivals)
   uint64_t* fullb = fulla + S;      // stage: slices of B landed
   uint64_t* empty = fullb + S;      // stage: products that read it complete
@@ -213,7 +218,8 @@ k_gemm_fs(const __grid_constant__ CUtensorMap tmB, const float* __restrict__ A, 
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int ntiles = ff_cdiv(M, TM) * nslices;
-  const int nk = (K + FS_TK - 1) / FS_TK;
+  // K-chunks of A, then those of A2 (K2 = 0: none)
+  const int k1c = (K1 + FS_TK - 1) / FS_TK, nk = k1c + (K2 + FS_TK - 1) / FS_TK;
 
   if (threadIdx.x == 0) {
     s_fail = 0;
@@ -259,12 +265,16 @@ k_gemm_fs(const __grid_constant__ CUtensorMap tmB, const float* __restrict__ A, 
       have = it.t < ntiles;
       if (have) {
         const int m0 = it.row * TM + w * 32 + rsub;
-        const int k = kc * FS_TK + 8 * j;
+        const bool second = kc >= k1c;
+        const int k = (second ? kc - k1c : kc) * FS_TK + 8 * j;
+        const bool kok = k < (second ? K2 : K1);
+        const float* src = second ? A2 : A;
+        const int ld = second ? lda2 : lda;
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
           const int r = m0 + 8 * i;
-          if (r < M && k < K) {
-            ld8(A + (size_t)r * lda + k, d[i]);
+          if (r < M && kok) {
+            ld8(src + (size_t)r * ld + k, d[i]);
           } else {
 #pragma unroll
             for (int x = 0; x < 8; ++x) d[i][x] = 0.f;
@@ -387,7 +397,8 @@ k_gemm_fs(const __grid_constant__ CUtensorMap tmB, const float* __restrict__ A, 
             da[sl] = smem_desc64(smem_u32(sa + sl * FS_ASLICE));
             db[sl] = smem_desc64(smem_u32(sb + sl * b_slice));
           }
-          const int nkk = min(FS_TK / 16, (K - kc * FS_TK) / 16);
+          const int nkk =
+              min(FS_TK / 16, (kc < k1c ? K1 - kc * FS_TK : K2 - (kc - k1c) * FS_TK) / 16);
           for (int kk = 0; kk < nkk; ++kk) {
             const uint64_t o = (uint64_t)(kk * 2);
             const uint32_t acc = (kc > 0 || kk > 0) ? 1u : 0u;
@@ -414,25 +425,26 @@ k_gemm_fs(const __grid_constant__ CUtensorMap tmB, const float* __restrict__ A, 
     // ---- epilogue group g, lane quadrant warp & 3: 16 columns of the warp's 32 rows at a
     // time go through its shared tile (float4 groups XOR-swizzled, conflict-free both ways)
     // and leave as 64-byte row segments; a lane then owns 4 columns of rows rsub + 8 i.  Every
-    // lane copies the epilogue inputs that it will read itself into its own slots, FS_AUXN
-    // - 1 column groups ahead and across tile boundaries (48 KB in flight per SM: with one
+    // lane copies the epilogue inputs that it will read itself into its own slots, AUXN - 1
+    // column groups ahead and across tile boundaries (48 KB in flight per SM: with one
     // group ahead in registers the residual modes ran at a third of the copy bandwidth).
     const int g = warp >> 2, quad = warp & 3;
     const int gq = lane & 3, rsub = lane >> 2;
     float* tile = tiles + warp * 32 * 16;
-    uint8_t* my_aux = auxs + (size_t)warp * (FS_AUXN * 2048) + lane * 16;
+    uint8_t* my_aux = auxs + (size_t)warp * (AUXN * SLOT) + lane * 16;
     FsWalk at(blockIdx.x + g * gridDim.x, 2 * gridDim.x, nslices);   // next columns to fetch:
     int ac = 0;                                                      // tile, first column
-    uint32_t an = 0;                               // column groups fetched
+    uint32_t an = 0;                                                 // column groups fetched
     auto fetch = [&]() {
       if (at.t < ntiles) {
         const int n0 = at.sl * nbw, mq = at.row * TM + quad * 32 + rsub;
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          const float* src =
-              mq + 8 * i < M ? fs_aux<MODE>(ep, (size_t)(mq + 8 * i), n0 + ac + 4 * gq) : nullptr;
-          if (src) fs_cp16(smem_u32(my_aux + (an % FS_AUXN) * 2048 + i * 512), src);
-        }
+        for (int u = 0; u < NAUX; ++u)
+#pragma unroll
+          for (int i = 0; i < 4; ++i)
+            if (mq + 8 * i < M)
+              fs_cp16(smem_u32(my_aux + (an % AUXN) * SLOT + u * 2048 + i * 512),
+                      fs_aux<MODE>(ep, u, (size_t)(mq + 8 * i), n0 + ac + 4 * gq));
         ac += 16;
         if (ac >= min(nbw, N - n0)) {
           ac = 0;
@@ -444,7 +456,7 @@ k_gemm_fs(const __grid_constant__ CUtensorMap tmB, const float* __restrict__ A, 
     };
     uint32_t un = 0;                               // column groups used
     if (AUX)
-      for (int k = 0; k < FS_AUXN - 1; ++k) fetch();
+      for (int k = 0; k < AUXN - 1; ++k) fetch();
     bool good = true;
     int jt = g;
     FsWalk it(blockIdx.x + g * gridDim.x, 2 * gridDim.x, nslices);
@@ -456,13 +468,17 @@ k_gemm_fs(const __grid_constant__ CUtensorMap tmB, const float* __restrict__ A, 
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
         fr[i] = 0.f;
-        if ((MODE == EPI_SILU_F || MODE == EPI_SILU_RES) && m0 + 8 * i < M)
+        if ((MODE == EPI_SILU_F || MODE == EPI_SILU_RES || MODE == EPI_HEAD ||
+             MODE == EPI_RES_DS) && m0 + 8 * i < M)
           fr[i] = ep.f[(size_t)(m0 + 8 * i) * ep.ldf];
       }
       good = __all_sync(0xffffffffu, mbar_wait_ab(smem_u32(&accf[g]), (uint32_t)((jt >> 1) & 1),
                                                   &s_abort));
       if (!good) break;
       fence_after();
+      float racc[4][2];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) racc[i][0] = racc[i][1] = 0.f;
       for (int c0 = 0; c0 < ncur; c0 += 16) {
         if (AUX) fetch();
         {
@@ -480,44 +496,85 @@ k_gemm_fs(const __grid_constant__ CUtensorMap tmB, const float* __restrict__ A, 
         }
         __syncwarp();
         const int col = n0 + c0 + 4 * gq;
-        if (AUX) asm volatile("cp.async.wait_group %0;" ::"n"(FS_AUXN - 1) : "memory");
-        const uint8_t* ax = my_aux + (un++ % FS_AUXN) * 2048;
+        if (AUX) asm volatile("cp.async.wait_group %0;" ::"n"(AUXN - 1) : "memory");
+        const uint8_t* ax = my_aux + (un++ % AUXN) * SLOT;
+        float4 w4 = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (MODE == EPI_HEAD) w4 = *reinterpret_cast<const float4*>(ep.wv + col);
+        const float wv[4] = {w4.x, w4.y, w4.z, w4.w};
         // the arithmetic runs for all rows, so that the 16 chains of a lane interleave (under a
         // branch per row they ran four at a time); only the stores look at the row count
-        float pre[4][4], o[4][4];
+        float pre[4][4], o[4][4];   // RES_DS: pre = dE/dz of the layer below
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
           const int rl = 8 * i + rsub;
           const float4 acc =
               *reinterpret_cast<const float4*>(&tile[rl * 16 + 4 * (gq ^ ((rl >> 1) & 3))]);
-          float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+          float4 a = make_float4(0.f, 0.f, 0.f, 0.f), z = a;
           if (AUX) a = *reinterpret_cast<const float4*>(ax + i * 512);
+          if (NAUX == 2) z = *reinterpret_cast<const float4*>(ax + 2048 + i * 512);
           const float v[4] = {ep.alpha * acc.x, ep.alpha * acc.y, ep.alpha * acc.z,
                               ep.alpha * acc.w};
-          const float a4[4] = {a.x, a.y, a.z, a.w};
+          const float a4[4] = {a.x, a.y, a.z, a.w}, z4[4] = {z.x, z.y, z.z, z.w};
 #pragma unroll
           for (int k = 0; k < 4; ++k) {
             pre[i][k] = v[k];
+            if (MODE == EPI_HEAD || MODE == EPI_RES_DS) {
+              // HEAD: sums of w a and w silu(v), dE/dz = beta f w silu'(v).  RES_DS: dE/dx, its
+              // sum with silu(z), and dE/dz of the layer below.
+              const float zk = MODE == EPI_HEAD ? v[k] : z4[k];
+              const float sg = sigm_nr(zk), sv = zk * sg;
+              const float ds = sg + sv * (1.f - sg);
+              if (MODE == EPI_HEAD) {
+                racc[i][0] += wv[k] * a4[k];
+                racc[i][1] += wv[k] * sv;
+                o[i][k] = ep.beta * fr[i] * wv[k] * ds;
+              } else {
+                o[i][k] = v[k] + ep.beta * a4[k];
+                racc[i][0] += o[i][k] * sv;
+                pre[i][k] = ep.alpha2 * fr[i] * o[i][k] * ds;
+              }
+              continue;
+            }
             if (MODE == EPI_STORE) o[i][k] = v[k];
             else if (MODE == EPI_SILU) o[i][k] = silu_nr(v[k]);
             else if (MODE == EPI_SILU_F) o[i][k] = fr[i] * silu_nr(v[k]);
             else if (MODE == EPI_SILU_RES) o[i][k] = ep.beta * (a4[k] + fr[i] * silu_nr(v[k]));
-            else if (MODE == EPI_DSILU) o[i][k] = v[k] * dsilu_nr(a4[k]);
-            else if (MODE == EPI_RES) o[i][k] = v[k] + (col < ep.split ? ep.beta * a4[k] : 0.f);
-            else o[i][k] = a4[k] + v[k];
+            else o[i][k] = v[k] * dsilu_nr(a4[k]);   // DSILU
           }
         }
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
           if (m0 + 8 * i >= M) continue;
           const size_t r = (size_t)(m0 + 8 * i);
-          if (MODE == EPI_SILU || MODE == EPI_SILU_F || MODE == EPI_SILU_RES)
+          if (MODE == EPI_SILU || MODE == EPI_SILU_F || MODE == EPI_SILU_RES ||
+              MODE == EPI_RES_DS)
             *reinterpret_cast<float4*>(ep.pre + r * ep.ldp + col) =
                 make_float4(pre[i][0], pre[i][1], pre[i][2], pre[i][3]);
-          *reinterpret_cast<float4*>(ep.out + r * ep.ldo + col) =
-              make_float4(o[i][0], o[i][1], o[i][2], o[i][3]);
+          if (MODE != EPI_RES_DS || ep.out)
+            *reinterpret_cast<float4*>(ep.out + r * ep.ldo + col) =
+                make_float4(o[i][0], o[i][1], o[i][2], o[i][3]);
         }
         __syncwarp();   // the shared tile is free again
+      }
+      if (MODE == EPI_HEAD || MODE == EPI_RES_DS) {
+        // row sums over this slice's columns (the 4 lanes of a row), into the slice's own slot
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+#pragma unroll
+          for (int q = 0; q < (MODE == EPI_HEAD ? 2 : 1); ++q) {
+            racc[i][q] += __shfl_xor_sync(0xffffffffu, racc[i][q], 1);
+            racc[i][q] += __shfl_xor_sync(0xffffffffu, racc[i][q], 2);
+          }
+          if (gq == 0 && m0 + 8 * i < M) {
+            const size_t at_ = (size_t)it.sl * ep.gfp_ld + m0 + 8 * i;
+            if (MODE == EPI_HEAD) {
+              ep.eout[at_] = ep.beta * (racc[i][0] + fr[i] * racc[i][1]);
+              ep.gfp[at_] = ep.beta * racc[i][1];
+            } else {
+              ep.gfp[at_] = ep.alpha2 * racc[i][0];
+            }
+          }
+        }
       }
       // the accumulators are free again
       fence_before();
@@ -539,8 +596,9 @@ k_gemm_fs(const __grid_constant__ CUtensorMap tmB, const float* __restrict__ A, 
 }
 
 template <int MODE>
-bool launch_fs(const CUtensorMap& tb, const float* A, int lda, int M, int N, int K, int nslices,
-               int nbw, const EpiParams& ep, int* err, cudaStream_t s) {
+bool launch_fs(const CUtensorMap& tb, const float* A, int lda, const float* A2, int lda2, int M,
+               int N, int K1, int K2, int nslices, int nbw, const EpiParams& ep, int* err,
+               cudaStream_t s) {
   static int n_sm = 0;
   if (!n_sm) {
     int dev = 0, sms = 0;
@@ -555,20 +613,20 @@ bool launch_fs(const CUtensorMap& tb, const float* A, int lda, int M, int N, int
   }
   // ring, tiles, epilogue inputs, alignment, barriers
   const size_t bytes = fs_stages<MODE>() * (3 * (size_t)FS_ASLICE + 3 * (size_t)nbw * FS_TK * 2) +
-                       FS_EW * 32 * 16 * 4 + (fs_has_aux<MODE>() ? FS_EW * FS_AUXN * 2048 : 0) +
+                       FS_EW * 32 * 16 * 4 + FS_EW * fs_auxn<MODE>() * fs_naux<MODE>() * 2048 +
                        1024 + 256;
   const int ntiles = ff_cdiv(M, TM) * nslices;
   k_gemm_fs<MODE><<<ntiles < n_sm ? ntiles : n_sm, FS_THREADS, bytes, s>>>(
-      tb, A, lda, M, N, K, nslices, nbw, ep, err);
+      tb, A, lda, A2, lda2, M, N, K1, K2, nslices, nbw, ep, err);
   return true;
 }
 
-using FsFn = bool (*)(const CUtensorMap&, const float*, int, int, int, int, int, int,
-                      const EpiParams&, int*, cudaStream_t);
+using FsFn = bool (*)(const CUtensorMap&, const float*, int, const float*, int, int, int, int, int,
+                      int, int, const EpiParams&, int*, cudaStream_t);
 // indexed by epilogue mode
 const FsFn kFs[] = {launch_fs<EPI_STORE>,    launch_fs<EPI_SILU>,  launch_fs<EPI_SILU_F>,
-                    launch_fs<EPI_SILU_RES>, launch_fs<EPI_DSILU>, launch_fs<EPI_RES>,
-                    launch_fs<EPI_ACC>};
+                    launch_fs<EPI_SILU_RES>, launch_fs<EPI_DSILU>, nullptr,   // (no EPI_RES)
+                    launch_fs<EPI_HEAD>,     launch_fs<EPI_RES_DS>};
 
 }  // namespace
 
@@ -579,17 +637,21 @@ void launch_split_weights(const float* Wt, int N, int K, __nv_bfloat16* out, cud
 }
 
 bool launch_gemm_f32(int mode, int M, int N, int K, const float* A, int lda,
-                     const __nv_bfloat16* Bs, const EpiParams& ep, int* err, cudaStream_t s) {
+                     const __nv_bfloat16* Bs, int ldb, const EpiParams& ep, int* err,
+                     cudaStream_t s, const float* A2, int K2, int lda2) {
   ProfScope ps_(PC_GEMM_F32, s);
   if (M <= 0) return true;
-  if (mode < EPI_STORE || mode > EPI_ACC || N % 16 != 0 || K % 16 != 0 || lda % 8 != 0 ||
-      ((uintptr_t)A & 31))
-    return false;
+  if (mode < EPI_STORE || mode > EPI_RES_DS || !kFs[mode]) return false;
+  if (N % 16 != 0 || K % 16 != 0 || lda % 8 != 0 || ((uintptr_t)A & 31)) return false;
+  if (A2 && (K2 <= 0 || K2 % 16 != 0 || lda2 % 8 != 0 || ((uintptr_t)A2 & 31))) return false;
+  const int ktot = A2 ? (K + FS_TK - 1) / FS_TK * FS_TK + K2 : K;
+  if (ldb < ktot || ldb % 8 != 0) return false;
   const int nslices = (N + 127) / 128;
   const int nbw = nslices == 1 ? N : 128;
   CUtensorMap tb;
-  if (!make_map(&tb, Bs, 3LL * N, K, K, nbw, FS_TK)) return false;
-  if (!kFs[mode](tb, A, lda, M, N, K, nslices, nbw, ep, err, s)) return false;
+  if (!make_map(&tb, Bs, 3LL * N, ktot, ldb, nbw, FS_TK)) return false;
+  if (!kFs[mode](tb, A, lda, A2, lda2, M, N, K, A2 ? K2 : 0, nslices, nbw, ep, err, s))
+    return false;
   ff_count_launch(1);
   return true;
 }

@@ -21,7 +21,6 @@ constexpr float kS5 = 2.23606797749979f;
 constexpr float kS15 = 3.872983346207417f;
 
 __device__ __forceinline__ float silu_f(float z) { return z / (1.f + expf(-z)); }
-__device__ __forceinline__ float sigm_f(float z) { return 1.f / (1.f + expf(-z)); }
 
 __device__ __forceinline__ float warp_sum(float v) {
 #pragma unroll
@@ -151,7 +150,10 @@ __global__ void k_twobody_in(long long E, int width, int n_basis, const float* _
 }
 
 // E_i = sum over the edges of i of x^N_ij . w_eff (the linear edge-energy MLP folded into
-// one vector).  One warp per atom; fixed summation order.
+// one vector; D <= 512).  One warp per atom, lane l owns columns l + 32 k; the sums run edge
+// by edge in order, the rows of four edges are loaded before them (a row at a time, the loads'
+// latency made 512 atoms of 55 edges take 155 us; now 14).
+constexpr int kEnergyCols = 16, kEnergyRows = 4;
 __global__ void k_energy(int n_atoms, const int* __restrict__ row_ptr, int e0,
                          const float* __restrict__ X, int ldx, int D,
                          const float* __restrict__ w_eff, float* __restrict__ E_atom) {
@@ -159,38 +161,59 @@ __global__ void k_energy(int n_atoms, const int* __restrict__ row_ptr, int e0,
   const int lane = threadIdx.x & 31;
   if (a >= n_atoms) return;
   const int eb = row_ptr[a] - e0, ee = row_ptr[a + 1] - e0;
+  float w[kEnergyCols];
+#pragma unroll
+  for (int k = 0; k < kEnergyCols; ++k) w[k] = lane + 32 * k < D ? w_eff[lane + 32 * k] : 0.f;
   float acc = 0.f;
-  for (int e = eb; e < ee; ++e)
-    for (int d = lane; d < D; d += 32) acc += X[(size_t)e * ldx + d] * w_eff[d];
+  for (int e = eb; e < ee; e += kEnergyRows) {
+    float x[kEnergyRows][kEnergyCols];
+#pragma unroll
+    for (int u = 0; u < kEnergyRows; ++u)
+#pragma unroll
+      for (int k = 0; k < kEnergyCols; ++k)
+        x[u][k] = e + u < ee && lane + 32 * k < D ? X[(size_t)(e + u) * ldx + lane + 32 * k] : 0.f;
+#pragma unroll
+    for (int u = 0; u < kEnergyRows; ++u) {
+      if (e + u >= ee) break;
+#pragma unroll
+      for (int k = 0; k < kEnergyCols; ++k)
+        if (lane + 32 * k < D) acc += x[u][k] * w[k];
+    }
+  }
   acc = warp_sum(acc);
   if (lane == 0) E_atom[a] = acc;
 }
 
-// E_i = sum_{e in seg(i)} E_e for per-edge energies from the fused readout; one warp per
-// atom, lanes stride the segment, fixed-order warp sum.
+// E_i = sum_{e in seg(i)} E_e for per-edge energies from the fused readout (nsl partial sums
+// per edge, ld apart, added in order); one warp per atom, lanes stride the segment,
+// fixed-order warp sum.
 __global__ void k_energy_sum(int n_atoms, const int* __restrict__ row_ptr, int e0,
-                             const float* __restrict__ E_edge, float* __restrict__ E_atom) {
+                             const float* __restrict__ E_edge, int nsl, long long ld,
+                             float* __restrict__ E_atom) {
   const int a = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (a >= n_atoms) return;
   const int eb = row_ptr[a] - e0, ee = row_ptr[a + 1] - e0;
   float acc = 0.f;
-  for (int e = eb + lane; e < ee; e += 32) acc += E_edge[e];
+  for (int e = eb + lane; e < ee; e += 32) {
+    float x = E_edge[e];
+    for (int k = 1; k < nsl; ++k) x += E_edge[k * ld + e];
+    acc += x;
+  }
   acc = warp_sum(acc);
   if (lane == 0) E_atom[a] = acc;
 }
 
-// Adjoint of out = f * silu(z) (scaled by alpha):  gz = alpha f silu'(z) gx,
-// gf += alpha sum_d gx silu(z).  One warp per EPW edges; lane l owns the float4 column
-// groups l, l + 32, ... (NGL of them: N <= 128 NGL) of each row; all loads of the rows are
-// issued first.  ldgx == 0: gx is one broadcast row.  gz (FP32) and/or gzb (BF16) receive
-// the result.  ZB: the pre-activations are bf16 (tensor-core path).
-template <bool ZB, int NGL, int EPW>
+// Adjoint of out = f * silu(z) (scaled by alpha), z bf16 (tensor-core path):
+// gz = alpha f silu'(z) gx, gf += alpha sum_d gx silu(z).  One warp per EPW edges; lane l owns
+// the float4 column groups l, l + 32, ... (NGL of them: N <= 128 NGL) of each row; all loads
+// of the rows are issued first.  ldgx == 0: gx is one broadcast row.  gz (FP32) or gzb (BF16)
+// receives the result.
+template <int NGL, int EPW>
 __global__ void k_rowred_bwd(long long E, int N, const float* __restrict__ gx, int ldgx,
-                             const float* __restrict__ z, const __nv_bfloat16* __restrict__ zb,
-                             int ldz, const float* __restrict__ ef, float alpha,
-                             float* __restrict__ gz, int ldgz, __nv_bfloat16* __restrict__ gzb,
-                             float* __restrict__ gf) {
+                             const __nv_bfloat16* __restrict__ zb, int ldz,
+                             const float* __restrict__ ef, float alpha, float* __restrict__ gz,
+                             int ldgz, __nv_bfloat16* __restrict__ gzb, float* __restrict__ gf) {
   const long long eb = ((long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * EPW;
   const int lane = threadIdx.x & 31;
   if (eb >= E) return;
@@ -207,14 +230,10 @@ __global__ void k_rowred_bwd(long long E, int N, const float* __restrict__ gx, i
       const int gi = lane + 32 * k;
       if (e < E && gi < ng) {
         g4[u][k] = *reinterpret_cast<const float4*>(gx + (size_t)e * ldgx + 4 * gi);
-        if (ZB) {
-          const uint2 pk = *reinterpret_cast<const uint2*>(zb + (size_t)e * ldz + 4 * gi);
-          const float2 lo = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&pk.x));
-          const float2 hi = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&pk.y));
-          z4[u][k] = make_float4(lo.x, lo.y, hi.x, hi.y);
-        } else {
-          z4[u][k] = *reinterpret_cast<const float4*>(z + (size_t)e * ldz + 4 * gi);
-        }
+        const uint2 pk = *reinterpret_cast<const uint2*>(zb + (size_t)e * ldz + 4 * gi);
+        const float2 lo = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&pk.x));
+        const float2 hi = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&pk.y));
+        z4[u][k] = make_float4(lo.x, lo.y, hi.x, hi.y);
       }
     }
   }
@@ -232,8 +251,8 @@ __global__ void k_rowred_bwd(long long E, int N, const float* __restrict__ gx, i
       float o[4];
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
-        // the bf16 path takes the hardware exponential and fast division, as its GEMMs do
-        const float sg = ZB ? __fdividef(1.f, 1.f + __expf(-zv[j])) : sigm_f(zv[j]);
+        // the hardware exponential and fast division, as in the GEMMs of this path
+        const float sg = __fdividef(1.f, 1.f + __expf(-zv[j]));
         o[j] = alpha * f[u] * gv[j] * (sg * (1.f + zv[j] * (1.f - sg)));
         acc += gv[j] * zv[j] * sg;
       }
@@ -253,12 +272,12 @@ __global__ void k_rowred_bwd(long long E, int N, const float* __restrict__ gx, i
   }
 }
 
-template <bool ZB, int NGL, int EPW>
-void rowred_one(long long E, int N, const float* gx, int ldgx, const float* z,
-                const __nv_bfloat16* zb, int ldz, const float* ef, float alpha, float* gz,
-                int ldgz, __nv_bfloat16* gzb, float* gf, cudaStream_t s) {
-  k_rowred_bwd<ZB, NGL, EPW><<<ff_cdiv(E, 8 * EPW), 256, 0, s>>>(E, N, gx, ldgx, z, zb, ldz, ef,
-                                                               alpha, gz, ldgz, gzb, gf);
+template <int NGL, int EPW>
+void rowred_one(long long E, int N, const float* gx, int ldgx, const __nv_bfloat16* zb, int ldz,
+                const float* ef, float alpha, float* gz, int ldgz, __nv_bfloat16* gzb, float* gf,
+                cudaStream_t s) {
+  k_rowred_bwd<NGL, EPW><<<ff_cdiv(E, 8 * EPW), 256, 0, s>>>(E, N, gx, ldgx, zb, ldz, ef, alpha,
+                                                             gz, ldgz, gzb, gf);
 }
 
 // dE/dr_e from the radial-basis gradient (via the first two-body layer), the envelope
@@ -301,7 +320,7 @@ __global__ void k_edge_grad(long long E, int w0, int n_basis, float rc, int p, i
     sincosf(a * r, &sn, &cs);
     gr += alpha0 * gB[n - 1] * pref * (a * cs * r - sn) / (r * r);
   }
-  float gfe = gf[e];
+  float gfe = gf ? gf[e] : 0.f;
   for (int k = 0; k < n_gfp; ++k) gfe += gfp[(size_t)k * gfp_ld + e];
   gr += gfe * envelope_df(r / rc, p, rc);
   // harmonic gradients: partial sums of the channel groups, added in a fixed order
@@ -548,30 +567,24 @@ void launch_energy(int n_atoms, const int* row_ptr, int e0, const float* X, int 
   ff_count_launch(1);
 }
 
-void launch_energy_sum(int n_atoms, const int* row_ptr, int e0, const float* E_edge,
-                       float* E_atom, cudaStream_t s) {
+void launch_energy_sum(int n_atoms, const int* row_ptr, int e0, const float* E_edge, int nsl,
+                       long long ld, float* E_atom, cudaStream_t s) {
   ProfScope ps_(PC_ENERGY, s);
   if (n_atoms <= 0) return;
-  k_energy_sum<<<ff_cdiv(n_atoms, 8), 256, 0, s>>>(n_atoms, row_ptr, e0, E_edge, E_atom);
+  k_energy_sum<<<ff_cdiv(n_atoms, 8), 256, 0, s>>>(n_atoms, row_ptr, e0, E_edge, nsl, ld,
+                                                   E_atom);
   ff_count_launch(1);
 }
 
-void launch_rowred_bwd(long long E, int N, const float* gx, int ldgx, const float* z,
-                       const __nv_bfloat16* zb, int ldz, const float* ef, float alpha,
-                       float* gz, int ldgz, __nv_bfloat16* gzb, float* gf, cudaStream_t s) {
+void launch_rowred_bwd(long long E, int N, const float* gx, int ldgx, const __nv_bfloat16* zb,
+                       int ldz, const float* ef, float alpha, float* gz, int ldgz,
+                       __nv_bfloat16* gzb, float* gf, cudaStream_t s) {
   ProfScope ps_(PC_ROWRED, s);
   if (E <= 0) return;
   // registers sized to the row: NGL float4 groups per lane, two rows per warp up to N = 256
-  if (N <= 128) {
-    if (zb) rowred_one<true, 1, 2>(E, N, gx, ldgx, z, zb, ldz, ef, alpha, gz, ldgz, gzb, gf, s);
-    else rowred_one<false, 1, 2>(E, N, gx, ldgx, z, zb, ldz, ef, alpha, gz, ldgz, gzb, gf, s);
-  } else if (N <= 256) {
-    if (zb) rowred_one<true, 2, 2>(E, N, gx, ldgx, z, zb, ldz, ef, alpha, gz, ldgz, gzb, gf, s);
-    else rowred_one<false, 2, 2>(E, N, gx, ldgx, z, zb, ldz, ef, alpha, gz, ldgz, gzb, gf, s);
-  } else {
-    if (zb) rowred_one<true, 4, 1>(E, N, gx, ldgx, z, zb, ldz, ef, alpha, gz, ldgz, gzb, gf, s);
-    else rowred_one<false, 4, 1>(E, N, gx, ldgx, z, zb, ldz, ef, alpha, gz, ldgz, gzb, gf, s);
-  }
+  if (N <= 128) rowred_one<1, 2>(E, N, gx, ldgx, zb, ldz, ef, alpha, gz, ldgz, gzb, gf, s);
+  else if (N <= 256) rowred_one<2, 2>(E, N, gx, ldgx, zb, ldz, ef, alpha, gz, ldgz, gzb, gf, s);
+  else rowred_one<4, 1>(E, N, gx, ldgx, zb, ldz, ef, alpha, gz, ldgz, gzb, gf, s);
   ff_count_launch(1);
 }
 
