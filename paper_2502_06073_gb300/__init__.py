@@ -120,11 +120,17 @@ def hparams_struct(hp: dict, precision: int = 0) -> HParams:
     return h
 
 
+_torch_mod = None
+
+
 def _torch():
-    import torch
-    if not torch.cuda.is_available():
-        raise FFError("a CUDA device is required (this library has no CPU path)")
-    return torch
+    global _torch_mod
+    if _torch_mod is None:      # a device that was there once is not asked for again
+        import torch
+        if not torch.cuda.is_available():
+            raise FFError("a CUDA device is required (this library has no CPU path)")
+        _torch_mod = torch
+    return _torch_mod
 
 
 def _stream(torch):

@@ -174,6 +174,9 @@ struct ff_ctx {
   int vmax = 0;
   int ncells = 0;
   std::vector<int> sys_ptr_h;
+  // elements of the buffers that a rebind keeps when they fit (dalloc_keep)
+  size_t cap_sys_ptr = 0, cap_esys = 0, cap_ccount = 0, cap_cstart = 0, cap_cfill = 0;
+  size_t cap_vlj = 0, cap_vls = 0;
   int* Z = nullptr; int* sys_ptr = nullptr; int* sys_of = nullptr;
   double* L_d = nullptr; float* Lf_d = nullptr;
   int* vl_j = nullptr; int* vl_s = nullptr; int* vl_cnt = nullptr;
@@ -184,9 +187,10 @@ struct ff_ctx {
   int* cnt = nullptr; int* row_ptr = nullptr;
   int* col = nullptr; int* shift = nullptr; int* src = nullptr; int* rev = nullptr;
   long long ecap = 0, E = 0;
-  std::vector<int> row_ptr_h;
+  std::vector<int> row_ptr_h;   // [0] and [n] always; all of it when row_ptr_full
+  bool row_ptr_full = false;
   int* scan_tmp = nullptr;
-  int* flags = nullptr;       // [0] error bits, [1] displacement flag
+  int* flags = nullptr;       // [0] error bits, [1] displacement flag, [2] edges counted
   int* flags_h = nullptr;     // pinned mirror
   float4* g = nullptr;
   float* E_atom = nullptr;
@@ -291,6 +295,18 @@ int dalloc(ff_ctx* c, T** p, size_t count) {
                                       " bytes failed: " + cudaGetErrorString(e));
   }
   return FF_OK;
+}
+
+// dalloc for a buffer whose capacity is remembered: kept while it fits and is at most four
+// times what is asked for (a free and an allocation cost more than a small system's whole
+// neighbour build), given back and allocated anew otherwise.
+template <typename T>
+int dalloc_keep(ff_ctx* c, T** p, size_t* cap, size_t count) {
+  if (*p && count <= *cap && *cap <= 4 * count + 4096) return FF_OK;
+  *cap = 0;
+  const int r = dalloc(c, p, count);
+  if (r == FF_OK) *cap = count;
+  return r;
 }
 
 template <typename T>
@@ -722,13 +738,14 @@ long long chunk_edge_budget(ff_ctx* c) {
 }
 
 int read_flags(ff_ctx* c, cudaStream_t s) {
-  FF_CK(c, cudaMemcpyAsync(c->flags_h, c->flags, 2 * sizeof(int), cudaMemcpyDeviceToHost, s));
+  FF_CK(c, cudaMemcpyAsync(c->flags_h, c->flags, 3 * sizeof(int), cudaMemcpyDeviceToHost, s));
   FF_CK(c, cudaStreamSynchronize(s));
   const int e = c->flags_h[0];
   if (e) {
     FF_CK(c, cudaMemsetAsync(c->flags, 0, sizeof(int), s));
     const char* what = nullptr;
-    const int st = ff_flags_status(e, &what);
+    // a list that must grow is rebuilt, which would lose the timeout of work enqueued earlier
+    const int st = ff_flags_status(e & FF_FLAG_TIMEOUT ? e & ~FF_FLAG_CAPACITY : e, &what);
     if (st != FF_OK) return set_err(c, st, what);
   }
   return FF_OK;
@@ -765,60 +782,72 @@ void setup_grid(ff_ctx* c) {
   c->ncells = (int)total;
 }
 
-int build_verlet(ff_ctx* c, const double* pos, cudaStream_t s) {
-  // positions are binned only once they are known to be finite
+// Enqueue the Verlet list at rc + skin.  A non-finite coordinate sets its error bit; it bins
+// into some cell (the index is clamped) and no pair passes the distance test with it.
+void enqueue_build(ff_ctx* c, const double* pos, cudaStream_t s) {
   launch_check_pos(pos, c->n, c->flags, s);
-  FF_TRY(read_flags(c, s));
+  if (c->allpairs) {
+    launch_pos_to_f32(pos, c->n, c->xf, s);
+    launch_verlet_allpairs(c->n, c->sys_of, c->sys_ptr, c->xf, c->rl2, c->vmax, c->vl_j, c->vl_s,
+                           c->vl_cnt, c->flags, s);
+    return;
+  }
+  cudaMemsetAsync(c->cell_count, 0, (size_t)c->ncells * sizeof(int), s);
+  launch_bin_atoms(pos, c->n, c->grid, c->cell_of, c->img, c->xf, c->cell_count, s);
+  launch_scan_i32(c->cell_count, c->cell_start, c->ncells, c->scan_tmp, nullptr, s);
+  cudaMemsetAsync(c->cell_fill, 0, (size_t)c->ncells * sizeof(int), s);
+  launch_cell_scatter(c->cell_of, c->n, c->cell_start, c->cell_fill, c->cell_atoms, s);
+  launch_verlet_cells(c->n, c->grid, c->cell_of, c->img, c->xf, c->cell_start, c->cell_atoms,
+                      c->rl2, c->vmax, c->vl_j, c->vl_s, c->vl_cnt, c->flags, s);
+}
+
+// Grow the per-atom capacity to the largest count of the list just built.
+int grow_verlet(ff_ctx* c) {
+  std::vector<int> cnt(c->n);
+  FF_CK(c, cudaMemcpy(cnt.data(), c->vl_cnt, (size_t)c->n * sizeof(int), cudaMemcpyDeviceToHost));
+  const int mx = *std::max_element(cnt.begin(), cnt.end());
+  if (mx > FF_MAX_NEIGHBORS)
+    return set_err(c, FF_ERR_CAPACITY, "an atom has " + std::to_string(mx) +
+                                           " neighbours within rc + skin (limit " +
+                                           std::to_string(FF_MAX_NEIGHBORS) + ")");
+  c->vmax = std::min(FF_MAX_NEIGHBORS, ((mx * 5 / 4) + 31) / 32 * 32);
+  FF_TRY(dalloc_keep(c, &c->vl_j, &c->cap_vlj, (size_t)c->n * c->vmax));
+  return dalloc_keep(c, &c->vl_s, &c->cap_vls, (size_t)c->n * c->vmax);
+}
+
+int built_ok(ff_ctx* c, const double* pos, cudaStream_t s) {
+  if (pos != c->xref)
+    FF_CK(c, cudaMemcpyAsync(c->xref, pos, (size_t)c->n * 3 * sizeof(double),
+                             cudaMemcpyDeviceToDevice, s));
+  c->built = true;
+  c->list_gen++;
+  return FF_OK;
+}
+
+int build_verlet(ff_ctx* c, const double* pos, cudaStream_t s) {
+  c->built = false;
   for (int attempt = 0; attempt < 3; ++attempt) {
-    if (c->allpairs) {
-      launch_pos_to_f32(pos, c->n, c->xf, s);
-      launch_verlet_allpairs(c->n, c->sys_of, c->sys_ptr, c->xf, c->rl2, c->vmax, c->vl_j,
-                             c->vl_s, c->vl_cnt, c->flags, s);
-    } else {
-      FF_CK(c, cudaMemsetAsync(c->cell_count, 0, (size_t)c->ncells * sizeof(int), s));
-      launch_bin_atoms(pos, c->n, c->grid, c->cell_of, c->img, c->xf, c->cell_count, s);
-      launch_scan_i32(c->cell_count, c->cell_start, c->ncells, c->scan_tmp, s);
-      FF_CK(c, cudaMemsetAsync(c->cell_fill, 0, (size_t)c->ncells * sizeof(int), s));
-      launch_cell_scatter(c->cell_of, c->n, c->cell_start, c->cell_fill, c->cell_atoms, s);
-      launch_verlet_cells(c->n, c->grid, c->cell_of, c->img, c->xf, c->cell_start,
-                          c->cell_atoms, c->rl2, c->vmax, c->vl_j, c->vl_s, c->vl_cnt, c->flags,
-                          s);
-    }
+    enqueue_build(c, pos, s);
     FF_CK(c, cudaGetLastError());
     const int r = read_flags(c, s);
-    if (r != FF_ERR_CAPACITY) {
-      if (r != FF_OK) return r;
-      FF_CK(c, cudaMemcpyAsync(c->xref, pos, (size_t)c->n * 3 * sizeof(double),
-                               cudaMemcpyDeviceToDevice, s));
-      c->built = true;
-      c->list_gen++;
-      return FF_OK;
-    }
-    // grow the per-atom capacity to the largest count seen and rebuild
-    std::vector<int> cnt(c->n);
-    FF_CK(c, cudaMemcpy(cnt.data(), c->vl_cnt, (size_t)c->n * sizeof(int), cudaMemcpyDeviceToHost));
-    const int mx = *std::max_element(cnt.begin(), cnt.end());
-    if (mx > FF_MAX_NEIGHBORS)
-      return set_err(c, FF_ERR_CAPACITY, "an atom has " + std::to_string(mx) +
-                                             " neighbours within rc + skin (limit " +
-                                             std::to_string(FF_MAX_NEIGHBORS) + ")");
-    c->vmax = std::min(FF_MAX_NEIGHBORS, ((mx * 5 / 4) + 31) / 32 * 32);
-    FF_TRY(dalloc(c, &c->vl_j, (size_t)c->n * c->vmax));
-    FF_TRY(dalloc(c, &c->vl_s, (size_t)c->n * c->vmax));
+    if (r == FF_OK) return built_ok(c, pos, s);
+    if (r != FF_ERR_CAPACITY) return r;
+    FF_TRY(grow_verlet(c));
   }
   return set_err(c, FF_ERR_CAPACITY, "neighbour capacity could not be established");
 }
 
-int filter_edges(ff_ctx* c, const double* pos, cudaStream_t s, float r2cut) {
-  launch_pos_to_f32(pos, c->n, c->xf, s);
+// Edges per atom at distance below the cutoff, their CSR offsets and their number (flags[2]).
+void enqueue_count(ff_ctx* c, const double* pos, cudaStream_t s, float r2cut, bool have_xf) {
+  if (!have_xf) launch_pos_to_f32(pos, c->n, c->xf, s);
   launch_filter(0, c->n, c->xf, c->Lf_d, r2cut, c->vmax, c->vl_j, c->vl_s, c->vl_cnt, c->cnt,
                 nullptr, nullptr, nullptr, nullptr, s);
-  launch_scan_i32(c->cnt, c->row_ptr, c->n, c->scan_tmp, s);
-  FF_CK(c, cudaGetLastError());
-  c->row_ptr_h.resize(c->n + 1);
-  FF_CK(c, cudaMemcpyAsync(c->row_ptr_h.data(), c->row_ptr, (size_t)(c->n + 1) * sizeof(int),
-                           cudaMemcpyDeviceToHost, s));
-  FF_CK(c, cudaStreamSynchronize(s));
+  launch_scan_i32(c->cnt, c->row_ptr, c->n, c->scan_tmp, c->flags + 2, s);
+}
+
+// The model list from the counts read back (c->flags_h[2] edges).  The host keeps all CSR
+// offsets only when the list may need several chunks (fill_row_ptr).
+int fill_edges(ff_ctx* c, cudaStream_t s, float r2cut) {
   if ((long long)c->n * c->vmax > INT32_MAX) {
     // the int32 CSR offsets wrap beyond 2^31 - 1 edges: count the edges in 64 bits first
     std::vector<int> cnt_h(c->n);
@@ -830,7 +859,11 @@ int filter_edges(ff_ctx* c, const double* pos, cudaStream_t s, float r2cut) {
       return set_err(c, FF_ERR_CAPACITY, "the model list has " + std::to_string(tot) +
                                              " edges (limit 2^31 - 1)");
   }
-  c->E = c->row_ptr_h[c->n];
+  c->E = c->flags_h[2];
+  c->row_ptr_full = false;
+  c->row_ptr_h.resize(c->n + 1);
+  c->row_ptr_h[0] = 0;
+  c->row_ptr_h[c->n] = (int)c->E;
   if (c->E > c->ecap) {
     const long long cap = std::max(c->E + c->E / 8 + 1024, 2 * c->ecap);
     FF_TRY(dalloc(c, &c->col, cap));
@@ -847,22 +880,54 @@ int filter_edges(ff_ctx* c, const double* pos, cudaStream_t s, float r2cut) {
   return FF_OK;
 }
 
-int update_neighbors(ff_ctx* c, const double* pos, cudaStream_t s) {
-  bool rebuild = !c->built || c->hp.skin <= 0.f;
-  if (!rebuild) {
+// The model list at `r2cut` for positions `pos`, from the standing Verlet list or (build) from
+// a new one.  One read-back and wait in the usual case: the error word, the displacement flag
+// and the edge count together.  check_disp: also rebuild when an atom has moved more than
+// skin/2; the count made on the old list is then thrown away.
+int make_list(ff_ctx* c, const double* pos, cudaStream_t s, float r2cut, bool build,
+              bool check_disp) {
+  if (check_disp && !build) {
     const double lim = 0.5 * (double)c->hp.skin;
     launch_disp_check(pos, c->xref, c->n, lim * lim, c->flags + 1, s);
-    // one read of both words: the displacement flag and the error word of the work
-    // enqueued before it
-    FF_TRY(read_flags(c, s));
-    if (c->flags_h[1]) {
-      rebuild = true;
-      FF_CK(c, cudaMemsetAsync(c->flags + 1, 0, sizeof(int), s));
-    }
   }
-  if (rebuild) FF_TRY(build_verlet(c, pos, s));
+  for (int attempt = 0; attempt < 4; ++attempt) {
+    if (build) {
+      c->built = false;
+      enqueue_build(c, pos, s);
+    }
+    enqueue_count(c, pos, s, r2cut, build);
+    FF_CK(c, cudaGetLastError());
+    const int r = read_flags(c, s);
+    if (build && r == FF_ERR_CAPACITY) {
+      FF_TRY(grow_verlet(c));
+      continue;
+    }
+    if (r != FF_OK) return r;
+    if (!build && check_disp && c->flags_h[1]) {
+      FF_CK(c, cudaMemsetAsync(c->flags + 1, 0, sizeof(int), s));
+      build = true;
+      continue;
+    }
+    if (build) FF_TRY(built_ok(c, pos, s));
+    return fill_edges(c, s, r2cut);
+  }
+  return set_err(c, FF_ERR_CAPACITY, "neighbour capacity could not be established");
+}
+
+int update_neighbors(ff_ctx* c, const double* pos, cudaStream_t s) {
+  FF_TRY(make_list(c, pos, s, c->rc2, !c->built || c->hp.skin <= 0.f, true));
   c->list_fixed = false;
-  return filter_edges(c, pos, s, c->rc2);
+  return FF_OK;
+}
+
+// every CSR offset on the host
+int fill_row_ptr(ff_ctx* c, cudaStream_t s) {
+  if (c->row_ptr_full) return FF_OK;
+  FF_CK(c, cudaMemcpyAsync(c->row_ptr_h.data(), c->row_ptr, (size_t)(c->n + 1) * sizeof(int),
+                           cudaMemcpyDeviceToHost, s));
+  FF_CK(c, cudaStreamSynchronize(s));
+  c->row_ptr_full = true;
+  return FF_OK;
 }
 
 // chunks of consecutive centre atoms with at most `cap` edges each
@@ -870,6 +935,10 @@ void plan_chunks(const ff_ctx* c, long long cap, std::vector<int>& starts) {
   starts.clear();
   int a = 0;
   starts.push_back(0);
+  if (c->E <= cap) {   // one chunk (the host may not have the offsets in between)
+    starts.push_back(c->n);
+    return;
+  }
   while (a < c->n) {
     int b = a + 1;
     // binary search the last atom boundary within the capacity
@@ -1153,8 +1222,15 @@ void backward_chunk(ff_ctx* c, int a0, int a1, const double* seed, cudaStream_t 
 }
 
 // chunk plan for the current model list, workspace sized for it
-int plan_and_reserve(ff_ctx* c, std::vector<int>& starts) {
+int plan_and_reserve(ff_ctx* c, std::vector<int>& starts, cudaStream_t s) {
+  // a list that fits the workspace at hand is one chunk (asking the driver for the free memory
+  // takes longer than several kernels of a small system)
+  if (c->E <= c->wcap && c->n <= c->acap && !getenv("FF_WORKSPACE_MB")) {
+    starts = {0, c->n};
+    return FF_OK;
+  }
   const long long budget = chunk_edge_budget(c);
+  if (c->E > budget) FF_TRY(fill_row_ptr(c, s));
   plan_chunks(c, budget, starts);
   long long maxc = 0;
   int maxa = 0;
@@ -1193,7 +1269,7 @@ int evaluate(ff_ctx* c, const double* pos, double* E_sys, float* E_atom, float* 
              const double* seed, bool forces, cudaStream_t s, bool check_err = true) {
   FF_TRY(update_neighbors(c, pos, s));
   std::vector<int> starts;
-  FF_TRY(plan_and_reserve(c, starts));
+  FF_TRY(plan_and_reserve(c, starts, s));
   FF_TRY(run_model(c, pos, E_sys, E_atom, F, seed, forces, starts, s));
   // the error word of this evaluation (a tensor-core pipeline timeout) is reported by it
   if (check_err) FF_TRY(read_flags(c, s));
@@ -1216,9 +1292,8 @@ void graph_reset(ff_ctx* c) {
 // list: edges beyond rc contribute exactly zero (the envelope and its derivative vanish),
 // so it stays valid while every atom is within skin/2 of its reference position.
 int prepare_fixed(ff_ctx* c, cudaStream_t s) {
-  if (!c->built) FF_TRY(build_verlet(c, c->xref, s));
-  FF_TRY(filter_edges(c, c->xref, s, c->rl2));
-  FF_TRY(plan_and_reserve(c, c->fixed_starts));
+  FF_TRY(make_list(c, c->xref, s, c->rl2, !c->built, false));
+  FF_TRY(plan_and_reserve(c, c->fixed_starts, s));
   c->list_fixed = true;
   c->fixed_gen = c->list_gen;
   graph_reset(c);
@@ -1394,11 +1469,11 @@ int ff_neighbors(ff_ctx* c, const double* pos, const int32_t* Z, int n_atoms, co
     FF_TRY(dalloc(c, &c->E_atom, n_atoms));
     FF_TRY(dalloc(c, &c->F_int, (size_t)n_atoms * 3));
   }
-  FF_TRY(dalloc(c, &c->sys_ptr, n_sys + 1));
-  FF_TRY(dalloc(c, &c->esys_tmp, n_sys));
-  FF_TRY(dalloc(c, &c->cell_count, c->ncells));
-  FF_TRY(dalloc(c, &c->cell_start, c->ncells + 1));
-  FF_TRY(dalloc(c, &c->cell_fill, c->ncells));
+  FF_TRY(dalloc_keep(c, &c->sys_ptr, &c->cap_sys_ptr, n_sys + 1));
+  FF_TRY(dalloc_keep(c, &c->esys_tmp, &c->cap_esys, n_sys));
+  FF_TRY(dalloc_keep(c, &c->cell_count, &c->cap_ccount, c->ncells));
+  FF_TRY(dalloc_keep(c, &c->cell_start, &c->cap_cstart, c->ncells + 1));
+  FF_TRY(dalloc_keep(c, &c->cell_fill, &c->cap_cfill, c->ncells));
   // initial per-atom capacity from the density (grown on overflow)
   int vm;
   if (c->allpairs) {
@@ -1412,29 +1487,35 @@ int ff_neighbors(ff_ctx* c, const double* pos, const int32_t* Z, int n_atoms, co
   }
   vm = std::min(FF_MAX_NEIGHBORS, std::max(32, (vm + 31) / 32 * 32));
   c->vmax = vm;
-  FF_TRY(dalloc(c, &c->vl_j, (size_t)n_atoms * vm));
-  FF_TRY(dalloc(c, &c->vl_s, (size_t)n_atoms * vm));
-  std::vector<int> sof(n_atoms);
-  for (int k = 0; k < n_sys; ++k)
-    for (int i = sp[k]; i < sp[k + 1]; ++i) sof[i] = k;
+  FF_TRY(dalloc_keep(c, &c->vl_j, &c->cap_vlj, (size_t)n_atoms * vm));
+  FF_TRY(dalloc_keep(c, &c->vl_s, &c->cap_vls, (size_t)n_atoms * vm));
+  // (host arrays of this call: copies from pageable memory have been staged on return)
   FF_CK(c, cudaMemcpyAsync(c->Z, Z, (size_t)n_atoms * sizeof(int), cudaMemcpyDeviceToDevice, s));
-  FF_CK(c, cudaMemcpy(c->sys_of, sof.data(), (size_t)n_atoms * sizeof(int),
-                      cudaMemcpyHostToDevice));
-  FF_CK(c, cudaMemcpy(c->sys_ptr, sp.data(), (size_t)(n_sys + 1) * sizeof(int),
-                      cudaMemcpyHostToDevice));
+  if (n_sys == 1) {
+    FF_CK(c, cudaMemsetAsync(c->sys_of, 0, (size_t)n_atoms * sizeof(int), s));
+  } else {
+    std::vector<int> sof(n_atoms);
+    for (int k = 0; k < n_sys; ++k)
+      for (int i = sp[k]; i < sp[k + 1]; ++i) sof[i] = k;
+    FF_CK(c, cudaMemcpyAsync(c->sys_of, sof.data(), (size_t)n_atoms * sizeof(int),
+                             cudaMemcpyHostToDevice, s));
+  }
+  FF_CK(c, cudaMemcpyAsync(c->sys_ptr, sp.data(), (size_t)(n_sys + 1) * sizeof(int),
+                           cudaMemcpyHostToDevice, s));
   const float Lf[3] = {(float)box[0], (float)box[1], (float)box[2]};
-  FF_CK(c, cudaMemcpy(c->L_d, box, 3 * sizeof(double), cudaMemcpyHostToDevice));
-  FF_CK(c, cudaMemcpy(c->Lf_d, Lf, 3 * sizeof(float), cudaMemcpyHostToDevice));
+  FF_CK(c, cudaMemcpyAsync(c->L_d, box, 3 * sizeof(double), cudaMemcpyHostToDevice, s));
+  FF_CK(c, cudaMemcpyAsync(c->Lf_d, Lf, 3 * sizeof(float), cudaMemcpyHostToDevice, s));
   launch_check_species(c->Z, n_atoms, c->flags, s);
-  FF_TRY(read_flags(c, s));
+  const bool was_bound = c->bound;
   c->bound = true;
   c->built = false;
   c->state_valid = false;
   c->g_pos = nullptr;
   c->md_force_pos = nullptr;
-  FF_TRY(build_verlet(c, pos, s));
   c->list_fixed = false;
-  return filter_edges(c, pos, s, c->rc2);
+  const int r = make_list(c, pos, s, c->rc2, true, false);
+  if (r == FF_ERR_SPECIES) c->bound = was_bound;
+  return r;
 }
 
 int ff_energy_forces(ff_ctx* c, const double* pos, double* E_sys, float* E_atom, float* F,
@@ -1566,7 +1647,7 @@ int ff_autotune(ff_ctx* c, const double* pos, int* slice, int* stages, double* m
         // neighbour work and host synchronisation stay outside the timed region
         FF_TRY(update_neighbors(c, pos, s));
         std::vector<int> starts;
-        FF_TRY(plan_and_reserve(c, starts));
+        FF_TRY(plan_and_reserve(c, starts, s));
         FF_CK(c, cudaEventRecord(e0, s));
         FF_TRY(run_model(c, pos, nullptr, nullptr, c->F_int, nullptr, true, starts, s));
         FF_CK(c, cudaEventRecord(e1, s));

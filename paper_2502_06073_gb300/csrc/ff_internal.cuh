@@ -126,7 +126,9 @@ struct NbrGrid {
   float Lf[3];        // float32 box used by the membership test
 };
 
-void launch_scan_i32(const int* in, int* out, int n, int* block_sums, cudaStream_t s);
+// exclusive sums out[0..n], out[n] = the total, which also goes to *total unless it is null
+void launch_scan_i32(const int* in, int* out, int n, int* block_sums, int* total,
+                     cudaStream_t s);
 void launch_bin_atoms(const double* pos, int n, NbrGrid g, int* cell_of, int4* img,
                       float4* xf, int* cell_count, cudaStream_t s);
 void launch_cell_scatter(const int* cell_of, int n, const int* cell_start, int* cell_fill,

@@ -81,15 +81,45 @@ __global__ void __launch_bounds__(1024) k_scan_block(const int* __restrict__ in,
   if (threadIdx.x == 0) bsum[blockIdx.x] = total;
 }
 
+// Up to FF_SCAN_BLOCK elements in one block: offsets, out[n] and the total.
+__global__ void __launch_bounds__(1024) k_scan_one(const int* __restrict__ in,
+                                                   int* __restrict__ out, int n,
+                                                   int* __restrict__ total_out) {
+  __shared__ int sh[96];
+  const int base = threadIdx.x * 4;
+  int v[4], s = 0;
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    v[k] = (base + k < n) ? in[base + k] : 0;
+    s += v[k];
+  }
+  int total;
+  int run = block_exclusive_scan(s, sh, total);
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    if (base + k < n) out[base + k] = run;
+    run += v[k];
+  }
+  if (threadIdx.x == 0) {
+    out[n] = total;
+    if (total_out) *total_out = total;
+  }
+}
+
 __global__ void __launch_bounds__(1024) k_scan_add(int* __restrict__ out, int n,
                                                    const int* __restrict__ bex,
-                                                   const int* __restrict__ bsum, int nb) {
+                                                   const int* __restrict__ bsum, int nb,
+                                                   int* __restrict__ total) {
   const long long base = (long long)blockIdx.x * FF_SCAN_BLOCK + threadIdx.x * 4;
   const int add = bex[blockIdx.x];
 #pragma unroll
   for (int k = 0; k < 4; ++k)
     if (base + k < n) out[base + k] += add;
-  if (blockIdx.x == 0 && threadIdx.x == 0) out[n] = bex[nb - 1] + bsum[nb - 1];
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    const int t = bex[nb - 1] + bsum[nb - 1];
+    out[n] = t;
+    if (total) *total = t;
+  }
 }
 
 // ------------------------------------------------------------------ binning
@@ -336,15 +366,21 @@ __global__ void k_check_species(const int* __restrict__ Z, int n, int* __restric
 }  // namespace
 
 
-void launch_scan_i32(const int* in, int* out, int n, int* block_sums, cudaStream_t s) {
+void launch_scan_i32(const int* in, int* out, int n, int* block_sums, int* total,
+                     cudaStream_t s) {
   ProfScope ps_(PC_NEIGHBOR, s);
   const int nb = n > 0 ? ff_cdiv(n, FF_SCAN_BLOCK) : 1;
+  if (nb == 1) {   // one block scans it all and writes the total: one launch instead of three
+    k_scan_one<<<1, 1024, 0, s>>>(in, out, n, total);
+    ff_count_launch(1);
+    return;
+  }
   int* bsum = block_sums;
   int* bex = block_sums + FF_SCAN_BLOCK;
   int* tmp = block_sums + 2 * FF_SCAN_BLOCK;
   k_scan_block<<<nb, 1024, 0, s>>>(in, out, n, bsum);
   k_scan_block<<<1, 1024, 0, s>>>(bsum, bex, nb, tmp);
-  k_scan_add<<<nb, 1024, 0, s>>>(out, n, bex, bsum, nb);
+  k_scan_add<<<nb, 1024, 0, s>>>(out, n, bex, bsum, nb, total);
   ff_count_launch(3);
 }
 

@@ -149,13 +149,13 @@ extern "C" int ff_neighbors_noalloc(const double* pos, int n_atoms, const double
   // (clamped into a valid cell) but the call then reports it instead of a list
   launch_check_pos(pos, n_atoms, flags, s);
   launch_bin_atoms(pos, n_atoms, g, cell_of, img, xf, cell_count, s);
-  launch_scan_i32(cell_count, cell_start, ncells, scan_tmp, s);
+  launch_scan_i32(cell_count, cell_start, ncells, scan_tmp, nullptr, s);
   launch_cell_scatter(cell_of, n_atoms, cell_start, cell_fill, cell_atoms, s);
   launch_verlet_cells(n_atoms, g, cell_of, img, xf, cell_start, cell_atoms, rc2, kMaxNbr, vl_j,
                       vl_s, vl_cnt, flags, s);
   launch_filter(0, n_atoms, xf, Lf_dev, rc2, kMaxNbr, vl_j, vl_s, vl_cnt, cnt, nullptr, nullptr,
                 nullptr, nullptr, s);
-  launch_scan_i32(cnt, row_ptr, n_atoms, scan_tmp, s);
+  launch_scan_i32(cnt, row_ptr, n_atoms, scan_tmp, nullptr, s);
   int host[2] = {0, 0};
   if (cudaMemcpyAsync(&host[0], flags, sizeof(int), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
       cudaMemcpyAsync(&host[1], row_ptr + n_atoms, sizeof(int), cudaMemcpyDeviceToHost, s) !=
