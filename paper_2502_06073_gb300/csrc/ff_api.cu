@@ -154,12 +154,10 @@ struct ff_ctx {
   __nv_bfloat16* WlatT_b[FF_MAX_LAYERS + 1][4] = {{nullptr}};
   // FP32 path on the tensor cores: three bf16 slices of every dense weight matrix, laid out
   // as the W^T [out][in] (forward) and W [in][out] (adjoint) operands; of the first latent
-  // matrix's adjoint operand Wlat_s[L][0] holds the scalar rows D.., Bcat_s the others
-  // (concatenated with the env weights as in Bcat_b: Bcat [D][bcat_ldf] FP32)
+  // matrix's adjoint operand Wlat_s[L][0] holds the scalar rows D.., Bcat_s the others,
+  // concatenated with the env weights as in Bcat_b
   __nv_bfloat16* wbuf_s = nullptr;
   __nv_bfloat16* W2b_s[4] = {nullptr}; __nv_bfloat16* W2bT_s[4] = {nullptr};
-  float* Bcat[FF_MAX_LAYERS + 1] = {nullptr};
-  int bcat_ldf = 0;
   __nv_bfloat16* Bcat_s[FF_MAX_LAYERS + 1] = {nullptr};
   __nv_bfloat16* WenvT_s[FF_MAX_LAYERS + 1] = {nullptr};
   __nv_bfloat16* Wlat_s[FF_MAX_LAYERS + 1][4] = {{nullptr}};
@@ -223,8 +221,9 @@ struct ff_ctx {
   __nv_bfloat16* GZb[2] = {nullptr};
   __nv_bfloat16* GWb = nullptr;
   // fused readout (last latent GEMM + edge-energy head; BF16 path: D <= 256): dE_e/dz of the
-  // last latent layer, per-edge energies and the envelope-gradient seed.  FP32 path: the sums
-  // per 128-column slice, E_edge[slice][wcap] and the first slots of gfp
+  // last latent layer, per-edge energies and the envelope-gradient seed, as sums per 128-column
+  // slice: E_edge[slice][wcap] and the first slots of gfp (the one-tile GEMM: whole rows,
+  // E_edge[0] and gfL)
   bool head = false;
   __nv_bfloat16* GZL = nullptr;
   float* GZLf = nullptr;
@@ -482,64 +481,47 @@ int upload_weights(ff_ctx* c) {
     for (size_t d = 0; d < u.size(); ++d) host[base + d] = (float)u[d];
     fix.push_back({&c->w_eff, base});
   }
-  // adjoint of the latent input and the env weights in one FP32 GEMM over [GZ | GW]: per layer
-  // Bcat [D][ld] = [Wlat[:D] | 0 | (a_env / a_lat) Wenv] with a_lat = ldx^-1/2, a_env = D^-1/2
-  // (the two fan-in scales), the first part padded to a multiple of 32
-  if (c->hp.precision == 0) {
-    const int k1p = (c->hp.latent[0] + 31) / 32 * 32;
-    c->bcat_ldf = k1p + c->ldw;
-    const double ratio = sqrt((double)c->ldx) / sqrt((double)c->D);
-    for (int L = 1; L <= c->NL; ++L) {
-      const Tensor* tl = find_tensor(c, "Wlat." + std::to_string(L) + ".0");   // [ldx][latent0]
-      const Tensor* te = find_tensor(c, "Wenv." + std::to_string(L));          // [D][ldw]
-      const size_t base = host.size();
-      host.resize(base + (size_t)c->D * c->bcat_ldf, 0.f);
-      for (int r = 0; r < c->D; ++r) {
-        float* row = host.data() + base + (size_t)r * c->bcat_ldf;
-        for (int q = 0; q < tl->cols; ++q)
-          row[q] = (float)c->params[tl->off + (size_t)r * tl->cols + q];
-        for (int q = 0; q < te->cols; ++q)
-          row[k1p + q] = (float)(ratio * c->params[te->off + (size_t)r * te->cols + q]);
-      }
-      fix.push_back({&c->Bcat[L], base});
-    }
-  }
   FF_TRY(dalloc(c, &c->wbuf, host.size()));
   FF_CK(c, cudaMemcpy(c->wbuf, host.data(), host.size() * sizeof(float), cudaMemcpyHostToDevice));
   for (auto& f : fix) *f.first = c->wbuf + f.second;
   if (c->hp.precision == 0) {
     // bf16 slices of the dense weights for the FP32 GEMM on the tensor cores
-    std::vector<std::pair<__nv_bfloat16**, size_t>> at;
-    std::vector<std::pair<const float*, std::pair<int, int>>> src;   // [rows][cols] FP32
-    size_t total = 0;
+    struct Src { __nv_bfloat16** dst; const float* w1; const float* w2; int n, k1, k2; };
+    std::vector<Src> src;
     auto add = [&](__nv_bfloat16** dst, const float* w, int rows, int cols) {
-      at.push_back({dst, total});
-      src.push_back({w, {rows, cols}});
-      total += ((size_t)3 * rows * cols + 127) / 128 * 128;
+      src.push_back({dst, w, nullptr, rows, cols, 0});
     };
     auto both = [&](__nv_bfloat16** w_s, __nv_bfloat16** wt_s, const float* w, const float* wt,
-                    const std::string& name) {
-      const Tensor* t = find_tensor(c, name);
-      add(w_s, w, t->rows, t->cols);
-      add(wt_s, wt, t->cols, t->rows);
+                    int rows, int cols) {
+      add(w_s, w, rows, cols);
+      add(wt_s, wt, cols, rows);
     };
+    const ff_hparams& hp = c->hp;
     for (int k = 1; k < c->n2b; ++k)
-      both(&c->W2b_s[k], &c->W2bT_s[k], c->W2b[k], c->W2bT[k], "W2b." + std::to_string(k));
+      both(&c->W2b_s[k], &c->W2bT_s[k], c->W2b[k], c->W2bT[k], hp.two_body[k - 1], hp.two_body[k]);
     for (int L = 1; L <= c->NL; ++L) {
-      const int lat0 = c->hp.latent[0];
+      const int lat0 = hp.latent[0];
       add(&c->WenvT_s[L], c->WenvT[L], c->ldw, c->D);
       add(&c->WlatT_s[L][0], c->WlatT[L][0], lat0, c->ldx);
       add(&c->Wlat_s[L][0], c->Wlat[L][0] + (size_t)c->D * lat0, c->ldx - c->D, lat0);
-      add(&c->Bcat_s[L], c->Bcat[L], c->D, c->bcat_ldf);
+      // [Wlat[:D] | (a_env / a_lat) Wenv], a_lat = ldx^-1/2, a_env = D^-1/2 the fan-in scales
+      src.push_back({&c->Bcat_s[L], c->Wlat[L][0], c->Wenv[L], c->D, lat0, c->ldw});
       for (int k = 1; k < c->nlat; ++k)
         both(&c->Wlat_s[L][k], &c->WlatT_s[L][k], c->Wlat[L][k], c->WlatT[L][k],
-             "Wlat." + std::to_string(L) + "." + std::to_string(k));
+             hp.latent[k - 1], hp.latent[k]);
+    }
+    std::vector<size_t> off;
+    size_t total = 0;
+    for (const Src& t : src) {
+      off.push_back(total);
+      total += ((size_t)3 * t.n * split_ld(t.k1, t.k2) + 127) / 128 * 128;
     }
     FF_TRY(dalloc(c, &c->wbuf_s, total));
-    for (size_t i = 0; i < at.size(); ++i) {
-      *at[i].first = c->wbuf_s + at[i].second;
-      launch_split_weights(src[i].first, src[i].second.first, src[i].second.second, *at[i].first,
-                           nullptr);
+    const double ratio = sqrt((double)c->ldx) / sqrt((double)c->D);
+    for (size_t i = 0; i < src.size(); ++i) {
+      const Src& t = src[i];
+      *t.dst = c->wbuf_s + off[i];
+      launch_split_weights(t.w1, t.n, t.k1, t.w2, t.k2, ratio, *t.dst, nullptr);
     }
     FF_CK(c, cudaGetLastError());
     FF_CK(c, cudaStreamSynchronize(nullptr));
@@ -678,10 +660,10 @@ Plan workspace_plan(ff_ctx* c, long long ecap, long long acap) {
   if (c->head) {
     if (tc) b16(&c->GZL, ecap * c->D);
     else f32(&c->GZLf, ecap * c->D);
-    f32(&c->E_edge, ecap * (tc ? 1 : nsl));
+    f32(&c->E_edge, ecap * nsl);
     if (tc) f32(&c->gfL, ecap);
   }
-  c->gfp_slots = (c->NL + (tc ? 0 : 1)) * nsl;
+  c->gfp_slots = (c->NL + 1) * nsl;
   f32(&c->gfp, ecap * c->gfp_slots);
   return plan;
 }
@@ -973,6 +955,11 @@ void mlp_gemm(ff_ctx* c, int mode, long long M, int N, int K, const float* A32,
     c->gemm_fail = true;
 }
 
+// Whether the GEMMs are the persistent ones, which write row sums per 128-column slice.
+bool slice_sums(const ff_ctx* c) {
+  return c->hp.precision == 0 || (c->tune_stages == 0 && c->tune_slice == 128);
+}
+
 void forward_chunk(ff_ctx* c, const double* pos, int a0, int a1, float* E_atom, cudaStream_t s) {
   const ff_hparams& hp = c->hp;
   const bool tc = hp.precision == 1;
@@ -1074,7 +1061,8 @@ void forward_chunk(ff_ctx* c, const double* pos, int a0, int a1, float* E_atom, 
     }
   }
   if (c->head)
-    launch_energy_sum(na, rp, e0, c->E_edge, tc ? 1 : (c->D + 127) / 128, c->wcap, E_atom + a0, s);
+    launch_energy_sum(na, rp, e0, c->E_edge, slice_sums(c) ? (c->D + 127) / 128 : 1, c->wcap,
+                      E_atom + a0, s);
   else launch_energy(na, rp, e0, c->X[c->NL], c->ldx, c->D, c->w_eff, E_atom + a0, s);
 }
 
@@ -1096,22 +1084,18 @@ void backward_chunk(ff_ctx* c, int a0, int a1, const double* seed, cudaStream_t 
   // slice into their own slots (summed in order by the geometric adjoint); BF16 path: when
   // that dE/dz is bf16, i.e. not below a two-body MLP of a single layer
   const int kb = c->n2b - 1, kl = c->nlat - 1;
-  const bool rr_fuse = !tc || (c->tune_stages == 0 && c->tune_slice == 128);
+  const bool rr_fuse = slice_sums(c);
   const int nsl = (c->D + 127) / 128;
-  int n_gfp = tc ? 0 : nsl;   // (FP32: the first slots came from the readout)
-  // the envelope gradient outside the slots: BF16 path, from the readout, and from the row
-  // reductions where those run
+  int n_gfp = c->head && rr_fuse ? nsl : 0;   // the first slots came from the readout
+  // the envelope gradient outside the slots, where a row reduction adds to it (BF16 path: above
+  // an unfused readout or a two-body MLP of one layer, or with the one-tile GEMMs)
   const float* gf = nullptr;
-  if (tc) {
-    if (c->head && rr_fuse && kb >= 1) {
-      gf = c->gfL;
-    } else {
-      if (c->head)
-        cudaMemcpyAsync(c->gf, c->gfL, (size_t)Ec * sizeof(float), cudaMemcpyDeviceToDevice, s);
-      else
-        cudaMemsetAsync(c->gf, 0, (size_t)Ec * sizeof(float), s);
-      gf = c->gf;
-    }
+  if (tc && !(c->head && rr_fuse && kb >= 1)) {
+    if (c->head && !rr_fuse)
+      cudaMemcpyAsync(c->gf, c->gfL, (size_t)Ec * sizeof(float), cudaMemcpyDeviceToDevice, s);
+    else
+      cudaMemsetAsync(c->gf, 0, (size_t)Ec * sizeof(float), s);
+    gf = c->gf;
   }
   bool rr_done = false;   // dE/dz of the next layer down was produced by the last GEMM
   int zb0 = 0;            // which of the ping-pong dE/dz buffers holds this layer's
@@ -1190,7 +1174,7 @@ void backward_chunk(ff_ctx* c, int a0, int a1, const double* seed, cudaStream_t 
                               c->bcat_ld, ep, c->flags, s, c->tune_slice, c->tune_stages, c->GWb,
                               c->ldw, c->ldw)
            : launch_gemm_f32(mode, (int)Ec, c->D, hp.latent[0], gzF, hp.latent[0], c->Bcat_s[L],
-                             c->bcat_ldf, ep, c->flags, s, c->GW, c->ldw, c->ldw);
+                             split_ld(hp.latent[0], c->ldw), ep, c->flags, s, c->GW, c->ldw, c->ldw);
     if (!ok) c->gemm_fail = true;
     gx = c->GX[cur];
     ldgx = c->ldx;

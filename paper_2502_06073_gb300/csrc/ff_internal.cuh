@@ -58,8 +58,8 @@ enum EpiMode {
   // last latent layer with the edge-energy head (tensor-core GEMM, whole rows per CTA):
   // z = alpha acc, s = silu(z), x = beta (res + f s);  eout[row] = sum_col wv x,
   // gfo[row] = beta sum_col wv s,  outb = beta f silu'(z) wv  (dE_ij/dz, bf16)
-  // (the FP32 GEMM: dE/dz FP32 in out, the sums per 128-column slice in eout and gfp, slices
-  // gfp_ld apart)
+  // (the persistent kernels: the sums per 128-column slice in eout and gfp, slices gfp_ld
+  // apart; the FP32 GEMM: dE/dz FP32 in out)
   EPI_HEAD = 6,
   // tensor-core GEMM, persistent kernel only: EPI_RES, fused with the SiLU adjoint of the
   // layer below that the row reduction would otherwise do: with o the RES output and z the
@@ -93,12 +93,16 @@ struct EpiParams {
 };
 
 // FP32 GEMM on the tensor cores from three bf16 slices per operand (gemm_f32.cu): A [M][K]
-// FP32, Bs = the slices of B^T, [3][N][ldb] bf16, from launch_split_weights (Wt = B^T [N][ldb]
-// FP32).  N, K % 16 == 0, lda, ldb % 8 == 0, A 32-byte aligned.  With A2 (FP32 [M][K2]) the
-// product is [A | A2] B over a concatenated K: A's columns rounded up to a multiple of 32
-// (zero-filled), then A2's; B^T has zeros in the padding.  Returns false if the launch could
-// not be set up; a device-side timeout sets FF_FLAG_TIMEOUT in *err.
-void launch_split_weights(const float* Wt, int N, int K, __nv_bfloat16* out, cudaStream_t s);
+// FP32, Bs = the slices of B^T, [3][N][ldb] bf16, from launch_split_weights.  N, K % 16 == 0,
+// lda, ldb % 8 == 0, A 32-byte aligned.  With A2 (FP32 [M][K2]) the product is [A | A2] B over
+// a concatenated K: A's columns rounded up to a multiple of 32 (zero-filled), then A2's.
+// Returns false if the launch could not be set up; a device-side timeout sets FF_FLAG_TIMEOUT
+// in *err.
+// Slices of B^T = [W1 | 0 | scale W2], W1 [N][K1], W2 [N][K2] FP32 (K2 = 0: W1 alone); a row
+// has split_ld(K1, K2) elements.
+int split_ld(int K1, int K2);
+void launch_split_weights(const float* W1, int N, int K1, const float* W2, int K2, double scale,
+                          __nv_bfloat16* out, cudaStream_t s);
 bool launch_gemm_f32(int mode, int M, int N, int K, const float* A, int lda,
                      const __nv_bfloat16* Bs, int ldb, const EpiParams& ep, int* err,
                      cudaStream_t s, const float* A2 = nullptr, int K2 = 0, int lda2 = 0);

@@ -489,7 +489,7 @@ k_gemm_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUten
 }
 
 // ---------------------------------------------------------------------------------------
-// Persistent variant for output slices of at most 128 columns (every mode but the readout):
+// Persistent variant for output slices of at most 128 columns:
 // one CTA per SM walks the (row tile, column slice) tiles blockIdx.x, + gridDim.x, ... with
 //   warp PP_EW      TMA producer: A/B K-chunks of all its tiles through a ring of `stages`
 //                   stages, running ahead of the MMAs across tile boundaries;
@@ -507,6 +507,22 @@ template <int MODE>
 __host__ __device__ constexpr int pp_na() {
   return (MODE == EPI_HEAD || MODE == EPI_SILU_RES || MODE == EPI_RES_DS) ? 3 : 4;
 }
+// Row epilogue (ROW; see row_chunk): one row per lane, straight from tensor memory, for STORE,
+// DSILU, SILU_RES and HEAD with bf16 output; the others transpose through a shared tile.  Modes
+// with an input tile, and the one that also stores the pre-activations:
+template <int MODE>
+__host__ __device__ constexpr bool row_in() { return MODE != EPI_STORE; }
+template <int MODE>
+__host__ __device__ constexpr bool row_pre() { return MODE == EPI_SILU_RES; }
+// Shared bytes of one epilogue warp: transposing tile and input tile, or, for the row epilogue,
+// two 32 x 32 bf16 tiles that hold the input and then the output of a chunk, and two for the
+// pre-activations.  (A third input tile cost the residual update a ring stage: 224 against
+// 204 us at 600,000 rows.)
+constexpr int kRowTile = 32 * 32 * 2;
+template <int MODE, bool ROW>
+__host__ __device__ constexpr int pp_warp_bytes() {
+  return ROW ? (row_pre<MODE>() ? 4 : 2) * kRowTile : 32 * 32 * 4 + aux_tile_bytes<MODE>();
+}
 template <int MODE>
 __host__ __device__ constexpr int pp_threads() {
   return 32 * (4 * pp_na<MODE>() + 2);
@@ -516,12 +532,98 @@ __host__ __device__ inline size_t pp_ring_bytes(int stages, int nbw) {
   return (size_t)stages * (TM * TK * 2 + (size_t)nbw * TK * 2);
 }
 
+__device__ __forceinline__ void tma_store_2d(const CUtensorMap* map, uint32_t src, int x, int y) {
+  asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.tile.bulk_group [%0, {%1, %2}], [%3];"
+               ::"l"((unsigned long long)map), "r"(x), "r"(y), "r"(src)
+               : "memory");
+}
+
+// sigm_fast on the flush-to-zero units: the same bits for every input (the argument of the
+// reciprocal is at least 1, and an exponential below the normal range adds nothing to 1), in
+// two thirds of the instructions
+__device__ __forceinline__ float sigm_ftz(float z) {
+  float e, r;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"(z * -1.4426950408889634f));
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(1.f + e));
+  return r;
+}
+__device__ __forceinline__ uint32_t pack_b16(float lo, float hi) {
+  const __nv_bfloat162 p = __floats2bfloat162_rn(lo, hi);
+  return *reinterpret_cast<const uint32_t*>(&p);
+}
+
+// Row epilogue of 32 columns: lane l has row l of the warp's 32 rows.  t: this lane's row of the
+// chunk's tile (64-byte swizzle: 16-byte group q of row l sits at q ^ (l >> 1 & 3)), on entry
+// the residual stream (SILU_RES, HEAD) or the pre-activations (DSILU), the output on return;
+// zt: its row of the pre-activation tile; out32: its row of an FP32 copy of x' (SILU_RES) or
+// null.  w: readout vector of the chunk; nc: columns inside the matrix.  HEAD: s0[k], s1[k] sum
+// w a and w silu(v) over the columns 4k..4k+3, in column order (what the lane that owned them
+// summed when eight lanes shared a row).
+// Against the transposing epilogue: half the instructions (no shared-memory transpose, no
+// address and predicate per row segment).  At 600,000 rows, us: readout 250 -> 183, residual
+// update 236 -> 204.
 template <int MODE>
+__device__ __forceinline__ void row_chunk(const EpiParams& ep, const float (&acc)[32], uint8_t* t,
+                                          uint8_t* zt, float f, const float* w, float* out32,
+                                          int nc, float (&s0)[8], float (&s1)[8]) {
+  const int sw = (threadIdx.x >> 1) & 3;
+  const float bf = __fmul_rn(ep.beta, f);
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    uint4* p = reinterpret_cast<uint4*>(t + ((q ^ sw) << 4));
+    uint4 a = make_uint4(0u, 0u, 0u, 0u);
+    if (row_in<MODE>()) a = *p;
+    const uint32_t ai[4] = {a.x, a.y, a.z, a.w};
+    uint32_t o[4], z[4];
+    float wq[8];
+    if (MODE == EPI_HEAD) {
+#pragma unroll
+      for (int j = 0; j < 8; ++j) wq[j] = 8 * q + j < nc ? w[8 * q + j] : 0.f;
+    }
+#pragma unroll
+    for (int h = 0; h < 4; ++h) {
+      float v[2], r[2];
+#pragma unroll
+      for (int j = 0; j < 2; ++j) {
+        const int c = 8 * q + 2 * h + j;
+        const float x = __uint_as_float(j ? ai[h] & 0xffff0000u : ai[h] << 16);
+        v[j] = __fmul_rn(ep.alpha, acc[c]);
+        if (MODE == EPI_STORE) {
+          r[j] = v[j];
+          continue;
+        }
+        const float sg = sigm_ftz(MODE == EPI_DSILU ? x : v[j]);
+        if (MODE == EPI_DSILU) {
+          r[j] = __fmul_rn(v[j], __fmul_rn(sg, __fmaf_rn(x, __fsub_rn(1.f, sg), 1.f)));
+          continue;
+        }
+        const float sv = __fmul_rn(v[j], sg);
+        if (MODE == EPI_SILU_RES) r[j] = __fmul_rn(ep.beta, __fmaf_rn(f, sv, x));
+        else {
+          if (c < nc) {
+            s0[c / 4] = __fmaf_rn(wq[2 * h + j], x, s0[c / 4]);
+            s1[c / 4] = __fmaf_rn(wq[2 * h + j], sv, s1[c / 4]);
+          }
+          r[j] = __fmul_rn(__fmul_rn(bf, wq[2 * h + j]), __fmaf_rn(sv, __fsub_rn(1.f, sg), sg));
+        }
+      }
+      o[h] = pack_b16(r[0], r[1]);
+      if (MODE == EPI_SILU_RES && out32 && 8 * q < nc)
+        *reinterpret_cast<float2*>(out32 + 8 * q + 2 * h) = make_float2(r[0], r[1]);
+      if (row_pre<MODE>()) z[h] = pack_b16(v[0], v[1]);
+    }
+    *p = make_uint4(o[0], o[1], o[2], o[3]);
+    if (row_pre<MODE>())
+      *reinterpret_cast<uint4*>(zt + ((q ^ sw) << 4)) = make_uint4(z[0], z[1], z[2], z[3]);
+  }
+}
+
+template <int MODE, bool ROW>
 __global__ void __launch_bounds__(pp_threads<MODE>(), 1)
 k_gemm_pp(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmA2,
           const __grid_constant__ CUtensorMap tmB, const __grid_constant__ CUtensorMap tmX,
-          const __grid_constant__ CUtensorMap tmX2, int M, int N, int K, int k1c, int nslices,
-          int nbw, int stages, int aux_tma, EpiParams ep, int* __restrict__ err) {
+          const __grid_constant__ CUtensorMap tmX2, const __grid_constant__ CUtensorMap tmO,
+          int M, int N, int K, int k1c, int nslices, int nbw, int stages, int aux_tma, EpiParams ep, int* __restrict__ err) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   constexpr int PP_NA = pp_na<MODE>();
@@ -533,13 +635,15 @@ k_gemm_pp(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUten
   const size_t ring = pp_ring_bytes(stages, nbw);
   float* tiles = reinterpret_cast<float*>(smem + ring);                  // PP_EW x 4 KB
   uint8_t* auxbuf = smem + ring + (size_t)PP_EW * 32 * 32 * 4;           // PP_EW x AUXB
-  uint64_t* bars = (uint64_t*)(auxbuf + (size_t)PP_EW * AUXB);
+  uint64_t* bars = (uint64_t*)(smem + ring + (size_t)PP_EW * pp_warp_bytes<MODE, ROW>());
   uint64_t* full = bars;
   uint64_t* empty = bars + stages;
   uint64_t* accf = bars + 2 * stages;     // PP_NA: accumulator complete
   uint64_t* acce = accf + PP_NA;          // PP_NA: accumulator drained (4 arrivals)
-  uint64_t* auxf = acce + PP_NA;          // PP_EW: epilogue input tile landed
-  uint64_t* fin = auxf + PP_EW;           // the MMA issuer's last commit
+  // epilogue input tile landed (row epilogue: two tiles a warp)
+  constexpr int NAUXB = PP_EW * (ROW ? 2 : 1);
+  uint64_t* auxf = acce + PP_NA;
+  uint64_t* fin = auxf + NAUXB;           // the MMA issuer's last commit
   uint32_t* tslot = (uint32_t*)(fin + 1);
   __shared__ int s_fail;
   __shared__ volatile int s_abort;
@@ -559,7 +663,7 @@ k_gemm_pp(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUten
       mbar_init(smem_u32(&accf[a]), 1);
       mbar_init(smem_u32(&acce[a]), 4);
     }
-    for (int w = 0; w < PP_EW; ++w) mbar_init(smem_u32(&auxf[w]), 1);
+    for (int w = 0; w < NAUXB; ++w) mbar_init(smem_u32(&auxf[w]), 1);
     mbar_init(smem_u32(fin), 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -578,14 +682,15 @@ k_gemm_pp(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUten
   if (warp == PP_EW) {
     // ---- TMA producer
     if (lane == 0) {
-      long q = 0;   // K-chunks issued so far (ring position)
+      // ring position (stage, parity of its use), kept by increments: dividing a 64-bit count by
+      // the runtime stage number took longer than a chunk's MMAs, here and in the MMA issuer
+      int st = 0;
+      uint32_t par = 1, used = 0;   // (parity 1: the first use of a stage finds it empty)
       bool good = true;
       for (int t = blockIdx.x; t < ntiles && good; t += gridDim.x) {
         const int m0 = (t / nslices) * TM, n0 = (t % nslices) * nbw;
-        for (int kc = 0; kc < nk; ++kc, ++q) {
-          const int st = (int)(q % stages);
-          if (q >= stages &&
-              !mbar_wait_ab(smem_u32(&empty[st]), (uint32_t)(((q / stages) - 1) & 1), &s_abort)) {
+        for (int kc = 0; kc < nk; ++kc) {
+          if (!mbar_wait_ab(smem_u32(&empty[st]), par, &s_abort)) {
             good = false;
             break;
           }
@@ -594,35 +699,43 @@ k_gemm_pp(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUten
           if (kc < k1c) tma_load_2d(smem_u32(sa), &tmA, kc * TK, m0, smem_u32(&full[st]));
           else tma_load_2d(smem_u32(sa), &tmA2, (kc - k1c) * TK, m0, smem_u32(&full[st]));
           tma_load_2d(smem_u32(sa + a_bytes), &tmB, kc * TK, n0, smem_u32(&full[st]));
+          if (used < (uint32_t)stages) ++used;
+          if (++st == stages) {
+            st = 0;
+            par ^= 1;
+          }
         }
       }
       if (!good) {
         s_fail = 1;
         s_abort = 1;
       }
-      // the loads issued last land before the CTA may exit
-      for (long p = q - 1; p >= 0 && p >= q - stages; --p)
-        mbar_wait(smem_u32(&full[p % stages]), (uint32_t)((p / stages) & 1));
+      // the last load of every stage lands before the CTA may exit
+      for (; used > 0; --used) {
+        if (st == 0) {
+          st = stages;
+          par ^= 1;
+        }
+        --st;
+        mbar_wait(smem_u32(&full[st]), par ^ 1);
+      }
     }
   } else if (warp == PP_EW + 1) {
     // ---- MMA issuer
     if (lane == 0) {
       const uint32_t idesc = instr_desc(TM, nbw);
-      long q = 0;
+      int st = 0, a = 0, j = 0;         // ring stage, accumulator, tiles so far
+      uint32_t par = 0, apar = 1;       // parities of their use
       bool good = true;
-      int j = 0;
       for (int t = blockIdx.x; t < ntiles && good; t += gridDim.x, ++j) {
-        const int a = j % PP_NA;
-        if (j >= PP_NA &&
-            !mbar_wait_ab(smem_u32(&acce[a]), (uint32_t)(((j / PP_NA) - 1) & 1), &s_abort)) {
+        if (!mbar_wait_ab(smem_u32(&acce[a]), apar, &s_abort)) {
           good = false;
           break;
         }
         fence_after();
         const uint32_t dacc = tbase + (uint32_t)(a * 128);
-        for (int kc = 0; kc < nk; ++kc, ++q) {
-          const int st = (int)(q % stages);
-          if (!mbar_wait_ab(smem_u32(&full[st]), (uint32_t)((q / stages) & 1), &s_abort)) {
+        for (int kc = 0; kc < nk; ++kc) {
+          if (!mbar_wait_ab(smem_u32(&full[st]), par, &s_abort)) {
             good = false;
             break;
           }
@@ -635,10 +748,18 @@ k_gemm_pp(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUten
             mma_bf16(dacc, da + (uint64_t)(kk * 2), db + (uint64_t)(kk * 2), idesc,
                      (kc > 0 || kk > 0) ? 1u : 0u);
           mma_commit(smem_u32(&empty[st]));
+          if (++st == stages) {
+            st = 0;
+            par ^= 1;
+          }
         }
         // (test hook: the accumulator of this CTA's first tile is never signalled, so its
         // epilogue group's bounded wait runs out and every role leaves through the abort path)
         if (good && !(ep.test_stall && j == 0)) mma_commit(smem_u32(&accf[a]));
+        if (++a == PP_NA) {
+          a = 0;
+          apar ^= 1;
+        }
       }
       if (!good) {
         s_fail = 1;
@@ -647,6 +768,100 @@ k_gemm_pp(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUten
       // every MMA issued above has completed before the tensor memory is released
       mma_commit(smem_u32(fin));
       mbar_wait(smem_u32(fin), 0);
+    }
+  } else if constexpr (ROW) {
+    // ---- row epilogue, group g = warp / 4, lane quadrant warp & 3.  A chunk's tile is filled
+    // by TMA a chunk ahead (over tile boundaries), turned into its output in place and written
+    // back by TMA, which clips rows and columns outside the matrix.
+    const int g = warp >> 2, quad = warp & 3;
+    uint8_t* mine = smem + ring + (size_t)warp * pp_warp_bytes<MODE, ROW>();
+    const int nchunks = (nbw + 31) / 32;
+    int ft = blockIdx.x + g * gridDim.x, fc = 0;   // next chunk to fetch (lane 0)
+    uint32_t fn = 0;
+    auto fetch = [&]() {
+      if (ft < ntiles) {
+        const uint32_t b = smem_u32(&auxf[warp * 2 + (fn & 1)]);
+        mbar_expect_tx(b, kRowTile);
+        tma_load_2d(smem_u32(mine + (fn & 1) * kRowTile), &tmX, (ft % nslices) * nbw + 32 * fc,
+                    (ft / nslices) * TM + quad * 32, b);
+        ++fn;
+        if (++fc == nchunks) {
+          fc = 0;
+          ft += PP_NA * gridDim.x;
+        }
+      }
+    };
+    if (row_in<MODE>() && lane == 0) fetch();
+    uint32_t n = 0;   // chunks done
+    bool good = true;
+    int j = g;
+    for (int t = blockIdx.x + g * gridDim.x; t < ntiles && good; t += PP_NA * gridDim.x,
+             j += PP_NA) {
+      const int y = (t / nslices) * TM + quad * 32, n0 = (t % nslices) * nbw;
+      const int row = y + lane;
+      const float f = (MODE == EPI_SILU_RES || MODE == EPI_HEAD) && row < M
+                          ? ep.f[(size_t)row * ep.ldf]
+                          : 0.f;
+      good = __all_sync(
+          0xffffffffu, mbar_wait_ab(smem_u32(&accf[g]), (uint32_t)((j / PP_NA) & 1), &s_abort,
+                                    ep.test_stall ? kTestWaitLimit : kWaitLimit));
+      if (!good) break;
+      fence_after();
+      float s0[8], s1[8];
+#pragma unroll
+      for (int k = 0; k < 8; ++k) s0[k] = s1[k] = 0.f;
+      for (int ci = 0; ci < nchunks; ++ci, ++n) {
+        float acc[32];
+        tmem_ld32(tbase + ((uint32_t)(quad * 32) << 16) + (uint32_t)(g * 128 + 32 * ci), acc);
+        if (row_in<MODE>()) {
+          good = __all_sync(0xffffffffu, mbar_wait_ab(smem_u32(&auxf[warp * 2 + (n & 1)]),
+                                                      (n >> 1) & 1, &s_abort));
+          if (!good) break;
+        }
+        uint8_t* tile = mine + (n & 1) * kRowTile;
+        uint8_t* zt = mine + (2 + (n & 1)) * kRowTile;   // (pre-activations)
+        const int x = n0 + 32 * ci;
+        row_chunk<MODE>(ep, acc, tile + lane * 64, zt + lane * 64, f, ep.wv + x,
+                        MODE == EPI_SILU_RES && ep.out && row < M
+                            ? ep.out + (size_t)row * ep.ldo + x : nullptr,
+                        N - x, s0, s1);
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        __syncwarp();
+        if (lane == 0) {
+          if (x < N) {
+            tma_store_2d(&tmO, smem_u32(tile), x, y);
+            if (row_pre<MODE>()) tma_store_2d(&tmX2, smem_u32(zt), x, y);
+          }
+          asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+          // the stores of the chunk before have read their tiles: the next chunk goes there
+          asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
+          if (row_in<MODE>()) fetch();
+        }
+        __syncwarp();
+      }
+      if (MODE == EPI_HEAD && good && row < M) {
+        // the row's sums over this slice, added pairwise as before, into the slice's own slot
+        const float a_ = ((s0[0] + s0[1]) + (s0[2] + s0[3])) + ((s0[4] + s0[5]) + (s0[6] + s0[7]));
+        const float g_ = ((s1[0] + s1[1]) + (s1[2] + s1[3])) + ((s1[4] + s1[5]) + (s1[6] + s1[7]));
+        const size_t at = (size_t)(t % nslices) * ep.gfp_ld + row;
+        ep.eout[at] = __fmul_rn(ep.beta, __fmaf_rn(f, g_, a_));
+        ep.gfp[at] = __fmul_rn(ep.beta, g_);
+      }
+      // the accumulator buffer is free again
+      fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(smem_u32(&acce[g]));
+    }
+    if (lane == 0) {
+      // every load issued has landed and every store has been done before the CTA may exit
+      // (after an abort, loads that no chunk waited for)
+      for (uint32_t k = n; k < fn; ++k)
+        mbar_wait(smem_u32(&auxf[warp * 2 + (k & 1)]), (k >> 1) & 1);
+      asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
+      if (!good) {
+        s_fail = 1;
+        s_abort = 1;
+      }
     }
   } else {
     // ---- epilogue group g = warp / 4, lane quadrant warp & 3
@@ -721,31 +936,6 @@ k_gemm_pp(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUten
           for (int i = 0; i < 8; ++i) {
             const int row = m0 + quad * 32 + 4 * i + (lane >> 3);
             if (row < M) dst[row] = ep.alpha2 * racc[i][0];
-          }
-        }
-      }
-      if (MODE == EPI_HEAD && good) {
-        // readout of this 128-column slice: the 8 lanes sharing a row sum their columns,
-        // then one lane adds the row's partial energy and envelope-gradient sums into the
-        // zeroed outputs (two slices per 256-wide row: 0 + a + b is the same in any order)
-#pragma unroll
-        for (int i = 0; i < 8; ++i)
-#pragma unroll
-          for (int q = 0; q < 2; ++q) {
-            float t = racc[i][q];
-            t += __shfl_xor_sync(0xffffffffu, t, 1);
-            t += __shfl_xor_sync(0xffffffffu, t, 2);
-            t += __shfl_xor_sync(0xffffffffu, t, 4);
-            racc[i][q] = t;
-          }
-        if ((lane & 7) == 0) {
-#pragma unroll
-          for (int i = 0; i < 8; ++i) {
-            const int row = m0 + quad * 32 + 4 * i + (lane >> 3);
-            if (row < M) {
-              atomicAdd(&ep.eout[row], ep.beta * (racc[i][0] + fr[i] * racc[i][1]));
-              atomicAdd(&ep.gfo[row], ep.beta * racc[i][1]);
-            }
           }
         }
       }
@@ -830,7 +1020,7 @@ bool launch_nw(const CUtensorMap& ta, const CUtensorMap& ta2, const CUtensorMap&
 }
 
 // Persistent launch: one CTA per SM (at most one per tile), the deepest ring that fits.
-template <int MODE>
+template <int MODE, bool ROW>
 bool launch_pp(const CUtensorMap& ta, const CUtensorMap& ta2, const CUtensorMap& tb, int M,
                int N, int K, int k1c, int nslices, int nbw, const EpiParams& ep, int* err,
                cudaStream_t s) {
@@ -843,33 +1033,43 @@ bool launch_pp(const CUtensorMap& ta, const CUtensorMap& ta2, const CUtensorMap&
         cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) !=
             cudaSuccess ||
-        cudaFuncGetAttributes(&fa, k_gemm_pp<MODE>) != cudaSuccess) {
+        cudaFuncGetAttributes(&fa, k_gemm_pp<MODE, ROW>) != cudaSuccess) {
       cudaGetLastError();
       return false;
     }
     const size_t lim = (size_t)optin - fa.sharedSizeBytes;
-    if (cudaFuncSetAttribute(k_gemm_pp<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    if (cudaFuncSetAttribute(k_gemm_pp<MODE, ROW>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)lim) != cudaSuccess) {
       cudaGetLastError();
       return false;
     }
     kMaxSmem = lim;
   }
-  CUtensorMap tx = ta, tx2 = ta;
-  int aux_tma = aux_map<MODE>(&tx, ep, M, N);
+  CUtensorMap tx = ta, tx2 = ta, to = ta;
+  int aux_tma = 0;
+  if constexpr (ROW) {
+    // input in, output and pre-activations out: 32 x 32 boxes, 64-byte swizzle
+    if (!make_map(&to, ep.outb, M, N, ep.ldob, 32, 32)) return false;
+    if (row_in<MODE>() && !make_map(&tx, MODE == EPI_DSILU ? ep.zb : ep.resb, M, N,
+                                    MODE == EPI_DSILU ? ep.ldz : ep.ldr, 32, 32))
+      return false;
+    if (row_pre<MODE>() && !make_map(&tx2, ep.preb, M, N, ep.ldp, 32, 32)) return false;
+  } else {
+    aux_tma = aux_map<MODE>(&tx, ep, M, N);
+  }
   if constexpr (MODE == EPI_RES_DS) {
     if (ep.ldzs <= 0 || !make_aux_map(&tx2, ep.zs, M, N, (size_t)ep.ldzs * 2, 2)) return false;
   }
   constexpr int PP_EW = 4 * pp_na<MODE>();
-  const size_t fixed = (size_t)PP_EW * 32 * 32 * 4 + (size_t)PP_EW * aux_tile_bytes<MODE>() +
-                       1024 + 512;   // epilogue tiles, input tiles, alignment, barriers
+  const size_t fixed = (size_t)PP_EW * pp_warp_bytes<MODE, ROW>() + 1024 + 512;   // epilogue warps,
+                                                                             // alignment, barriers
   int stages = 4;
   while (stages > 1 && pp_ring_bytes(stages, nbw) + fixed > kMaxSmem) --stages;
   if (pp_ring_bytes(stages, nbw) + fixed > kMaxSmem) return false;
   const int ntiles = ff_cdiv(M, TM) * nslices;
   const int grid = ntiles < n_sm ? ntiles : n_sm;
-  k_gemm_pp<MODE><<<grid, pp_threads<MODE>(), pp_ring_bytes(stages, nbw) + fixed, s>>>(
-      ta, ta2, tb, tx, tx2, M, N, K, k1c, nslices, nbw, stages, aux_tma, ep, err);
+  k_gemm_pp<MODE, ROW><<<grid, pp_threads<MODE>(), pp_ring_bytes(stages, nbw) + fixed, s>>>(
+      ta, ta2, tb, tx, tx2, to, M, N, K, k1c, nslices, nbw, stages, aux_tma, ep, err);
   return true;
 }
 
@@ -877,8 +1077,19 @@ template <int MODE>
 bool launch_mode(const CUtensorMap& ta, const CUtensorMap& ta2, const CUtensorMap& tb, int M,
                  int N, int K, int k1c, int nslices, int nbw, int stages, const EpiParams& ep,
                  int* err, cudaStream_t s) {
-  if (nbw <= 128 && stages == 0)
-    return launch_pp<MODE>(ta, ta2, tb, M, N, K, k1c, nslices, nbw, ep, err, s);
+  if (nbw <= 128 && stages == 0) {
+    // the row epilogue where it is the faster one (at 600,000 rows, us, transposing and row:
+    // readout 250 and 188, residual update 236 and 205, DSILU to bf16 100 and 97, STORE to bf16
+    // 79 and 77, but SILU 64 and 71, SILU_F 126 and 136: with no input to read, their two output
+    // streams by TMA cost more than they save); an FP32 output always transposes
+    if constexpr (MODE == EPI_RES || MODE == EPI_RES_DS || MODE == EPI_SILU || MODE == EPI_SILU_F)
+      return launch_pp<MODE, false>(ta, ta2, tb, M, N, K, k1c, nslices, nbw, ep, err, s);
+    else if constexpr (MODE == EPI_STORE || MODE == EPI_DSILU)   // bf16 or FP32 output
+      return ep.out ? launch_pp<MODE, false>(ta, ta2, tb, M, N, K, k1c, nslices, nbw, ep, err, s)
+                    : launch_pp<MODE, true>(ta, ta2, tb, M, N, K, k1c, nslices, nbw, ep, err, s);
+    else
+      return launch_pp<MODE, true>(ta, ta2, tb, M, N, K, k1c, nslices, nbw, ep, err, s);
+  }
   if constexpr (MODE == EPI_RES_DS) {
     return false;   // the fused SiLU adjoint exists only in the persistent kernel
   } else {
@@ -920,8 +1131,8 @@ bool launch_gemm_bf16(int mode, int M, int N, int K, const __nv_bfloat16* A, int
   if (slice != 128 && slice != 256) slice = 256;
   if (mode == EPI_HEAD) {
     if (N > 256) return false;
-    // the persistent kernel adds the row sums of 128-column slices into zeroed outputs;
-    // the one-tile kernel needs whole rows in one CTA
+    // the persistent kernel writes the row sums of each 128-column slice (eout and gfp, slices
+    // gfp_ld apart); the one-tile kernel needs whole rows in one CTA (eout and gfo)
     if (!(slice == 128 && stages_req == 0)) slice = 256;
   }
   // all column slices in one launch; a partial last slice reads zero-filled B rows and
@@ -942,10 +1153,6 @@ bool launch_gemm_bf16(int mode, int M, int N, int K, const __nv_bfloat16* A, int
   // deepest ring that fits), 256-column slices two stages (<= 96 KB: two CTAs per SM); the
   // autotuner may ask for the non-persistent kernel with 1..4 stages
   const int stages = (stages_req >= 1 && stages_req <= 4) ? stages_req : (nbw > 128 ? 2 : 0);
-  if (mode == EPI_HEAD && nbw <= 128 && stages == 0 &&
-      (cudaMemsetAsync(ep.eout, 0, (size_t)M * sizeof(float), s) != cudaSuccess ||
-       cudaMemsetAsync(ep.gfo, 0, (size_t)M * sizeof(float), s) != cudaSuccess))
-    return false;
   if (!kLaunch[mode](ta, ta2, tb, M, N, Ktot, k1c, nslices, nbw, stages, ep, err, s))
     return false;
   ff_count_launch(1);

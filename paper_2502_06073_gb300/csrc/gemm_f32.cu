@@ -103,7 +103,8 @@ __device__ __forceinline__ void fs_cp16(uint32_t dst, const float* src) {
 // -80 is 2e-35).
 __device__ __forceinline__ float sigm_nr(float z) {
   const float d = 1.f + expf(fminf(-z, 80.f));
-  const float r = __fdividef(1.f, d);
+  float r;   // d in [1, 6e34]: no denormals either side
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(d));
   return fmaf(r, fmaf(-d, r, 1.f), r);
 }
 __device__ __forceinline__ float silu_nr(float z) { return z * sigm_nr(z); }
@@ -161,16 +162,20 @@ __device__ __forceinline__ void ld8(const float* p, float (&v)[8]) {
                : "l"(p));
 }
 
-// Weights Wt [N][K] FP32 (K % 16 == 0) -> three slices [3][N][K] bf16; one warp per row and
-// chunk.  Run once per weight matrix, at creation.
-__global__ void k_split_weights(const float* __restrict__ Wt, int N, int K,
+// Weights B^T = [W1 | 0 | scale W2], W1 [N][K1] and W2 [N][K2] FP32 (K2 = 0: W1 alone), the
+// first part padded to a multiple of a chunk where there is a second -> three slices
+// [3][N][ktot] bf16; one warp per row and chunk.  Run once per weight matrix, at creation.
+__global__ void k_split_weights(const float* __restrict__ W1, const float* __restrict__ W2, int N,
+                                int K1, int K2, int k1p, double scale,
                                 __nv_bfloat16* __restrict__ out) {
-  const int nk = (K + FS_TK - 1) / FS_TK;
+  const int K = k1p + K2, nk = (K + FS_TK - 1) / FS_TK;
   const long long t = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   if (t >= (long long)N * nk) return;
   const int n = (int)(t / nk), k = (int)(t % nk) * FS_TK + (threadIdx.x & 31);
   const size_t i = (size_t)n * K + k, sl = (size_t)N * K;
-  const float w = k < K ? Wt[i] : 0.f;
+  float w = 0.f;
+  if (k < K1) w = W1[(size_t)n * K1 + k];
+  else if (k >= k1p && k < K) w = (float)(scale * (double)W2[(size_t)n * K2 + (k - k1p)]);
   float m = fabsf(w), c1, c2, a1, a2, a3;
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
@@ -250,7 +255,10 @@ k_gemm_fs(const __grid_constant__ CUtensorMap tmB, const float* __restrict__ A, 
 
   if (warp >= FS_EW && warp < FS_EW + FS_CW) {
     // ---- splitting group g: chunks q = g mod 2 of this CTA's (tile, K-chunk) sequence; two
-    // of them are in flight in registers
+    // of them are in flight in registers.  (A group's wait for a stage tells one phase from the
+    // next only because its chunk before, q - 2, has seen chunk q - 2 - S done, which is no
+    // earlier than the stage's phase before last: S >= 2.)
+    static_assert(S >= 2, "a stage per splitting group");
     const int g = (warp - FS_EW) >> 2, w = warp & 3;
     const int j = lane & 3, rsub = lane >> 2;
     float v[2][4][8];
@@ -300,15 +308,21 @@ k_gemm_fs(const __grid_constant__ CUtensorMap tmB, const float* __restrict__ A, 
         m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 2));
         float c1, c2;
         split_consts(m, c1, c2);
+        const float2 k1 = make_float2(c1, c1), n1 = make_float2(-c1, -c1);
+        const float2 k2 = make_float2(c2, c2), n2 = make_float2(-c2, -c2);
+        const float2 m1 = make_float2(-1.f, -1.f);
         uint32_t p1[4], p2[4], p3[4];
 #pragma unroll
         for (int x = 0; x < 4; ++x) {
-          float a1, a2, a3, b1, b2, b3;
-          split3(d[i][2 * x], c1, c2, a1, a2, a3);
-          split3(d[i][2 * x + 1], c1, c2, b1, b2, b3);
-          p1[x] = pack2(a1, b1);
-          p2[x] = pack2(a2, b2);
-          p3[x] = pack2(a3, b3);
+          // split3 of two elements in packed instructions
+          const float2 a = make_float2(d[i][2 * x], d[i][2 * x + 1]);
+          const float2 s1 = __fadd2_rn(__fadd2_rn(a, k1), n1);
+          const float2 r = __ffma2_rn(s1, m1, a);
+          const float2 s2 = __fadd2_rn(__fadd2_rn(r, k2), n2);
+          const float2 s3 = __ffma2_rn(s2, m1, r);
+          p1[x] = pack2(s1.x, s1.y);
+          p2[x] = pack2(s2.x, s2.y);
+          p3[x] = pack2(s3.x, s3.y);
         }
         const int r = w * 32 + 8 * i + rsub;
         uint8_t* dst = sa + r * 64 + ((j ^ ((r >> 1) & 3)) << 4);
@@ -630,9 +644,15 @@ const FsFn kFs[] = {launch_fs<EPI_STORE>,    launch_fs<EPI_SILU>,  launch_fs<EPI
 
 }  // namespace
 
-void launch_split_weights(const float* Wt, int N, int K, __nv_bfloat16* out, cudaStream_t s) {
-  const long long n = (long long)N * ((K + FS_TK - 1) / FS_TK);
-  k_split_weights<<<ff_cdiv(n, 8), 256, 0, s>>>(Wt, N, K, out);
+int split_ld(int K1, int K2) {
+  return K2 > 0 ? (K1 + FS_TK - 1) / FS_TK * FS_TK + K2 : K1;
+}
+
+void launch_split_weights(const float* W1, int N, int K1, const float* W2, int K2, double scale,
+                          __nv_bfloat16* out, cudaStream_t s) {
+  const int ld = split_ld(K1, K2);
+  const long long n = (long long)N * ((ld + FS_TK - 1) / FS_TK);
+  k_split_weights<<<ff_cdiv(n, 8), 256, 0, s>>>(W1, W2, N, K1, K2, ld - K2, scale, out);
   ff_count_launch(1);
 }
 
@@ -644,7 +664,7 @@ bool launch_gemm_f32(int mode, int M, int N, int K, const float* A, int lda,
   if (mode < EPI_STORE || mode > EPI_RES_DS || !kFs[mode]) return false;
   if (N % 16 != 0 || K % 16 != 0 || lda % 8 != 0 || ((uintptr_t)A & 31)) return false;
   if (A2 && (K2 <= 0 || K2 % 16 != 0 || lda2 % 8 != 0 || ((uintptr_t)A2 & 31))) return false;
-  const int ktot = A2 ? (K + FS_TK - 1) / FS_TK * FS_TK + K2 : K;
+  const int ktot = split_ld(K, A2 ? K2 : 0);
   if (ldb < ktot || ldb % 8 != 0) return false;
   const int nslices = (N + 127) / 128;
   const int nbw = nslices == 1 ? N : 128;
