@@ -15,6 +15,9 @@
 //   ran on the tensor cores: read as bf16, widened to FP32 for every product);
 //   V [E][dim][C];  G [atoms][9][C];
 //   the scalars go to X[e][D + q*C + c].
+// (A header: the forward and adjoint kernels are instantiated in two translation units.)
+#pragma once
+
 #include <type_traits>
 
 #include "ff_internal.cuh"
@@ -196,7 +199,8 @@ __device__ __forceinline__ int rs_index(int lane) {
 template <int LMAX, int INK, int OUTK>
 using TPK = TP<LMAX, INK == 3 ? 0 : INK, OUTK>;
 
-template <int LMAX, int INK, int OUTK, int CT, bool BWD, bool WB>
+// SMALL: the variant for systems of few atoms (see use_small), one block per (atom, group).
+template <int LMAX, int INK, int OUTK, int CT, bool BWD, bool WB, bool SMALL>
 struct EdgeRec {
   using K = TPK<LMAX, INK, OUTK>;
   static constexpr bool LAST = OUTK == 2;
@@ -208,10 +212,12 @@ struct EdgeRec {
   static constexpr int OFF_GVO = OFF_GS + (BWD ? K::NS * CT : 0);
   static constexpr int SST = OFF_GVO + ((BWD && !LAST) ? K::DOUT * CT : 0);
   // ring depth: up to 4 records within ~40 KB (adjoint) or ~24 KB (forward, which keeps
-  // more blocks resident) of shared memory per block, at least double buffering
-  static constexpr int BUDGET = (BWD ? 40 : 24) * 1024;
+  // more blocks resident) of shared memory per block, at least double buffering; SMALL: as
+  // deep as the static shared memory allows, up to 8
+  static constexpr int BUDGET = SMALL ? 46 * 1024 : (BWD ? 40 : 24) * 1024;
+  static constexpr int MAXSTG = SMALL ? 8 : 4;
   static constexpr int NSTG_FIT = BUDGET / (TEAMS * SST * 4);
-  static constexpr int NSTG = NSTG_FIT < 2 ? 2 : (NSTG_FIT > 4 ? 4 : NSTG_FIT);
+  static constexpr int NSTG = NSTG_FIT < 2 ? 2 : (NSTG_FIT > MAXSTG ? MAXSTG : NSTG_FIT);
   // the passes that read only the edge-feature row and the env weights use the same
   // buffer as a deeper ring of smaller records (2 to 8 of them); in the adjoint of the
   // first layer these also carry the FP32 weight gradients of its first pass
@@ -233,18 +239,18 @@ __device__ __forceinline__ void stage_ef_w(float* rec, int e, int lane, int C, i
   stage_w<CT, LMAX + 1>(rec + FF_EF_STRIDE, W + (size_t)e * ldw + grp * CT, C, lane);
 }
 
-template <int LMAX, int INK, int OUTK, int CT, bool BWD, bool WB, typename TW>
+template <int LMAX, int INK, int OUTK, int CT, bool BWD, bool WB, bool SMALL, typename TW>
 __device__ __forceinline__ void stage_edge(float* rec, int e, int lane, int C, int grp,
                                            const float* ef, const TW* W, int ldw,
                                            const float* vin, const float* GX, int ldx, int D,
-                                           const float* gvout) {
-  using R = EdgeRec<LMAX, INK, OUTK, CT, BWD, WB>;
+                                           const float* gvout, bool need_v = true) {
+  using R = EdgeRec<LMAX, INK, OUTK, CT, BWD, WB, SMALL>;
   using K = TPK<LMAX, INK, OUTK>;
   if (INK == 0) {
     if (lane < FF_EF_STRIDE / 4)
       cp_async16(rec + 4 * lane, ef + (size_t)e * FF_EF_STRIDE + 4 * lane);
     stage_w<CT, LMAX + 1>(rec + R::OFF_W, W + (size_t)e * ldw + grp * CT, C, lane);
-  } else {
+  } else if (need_v) {
     stage<CT, K::DIN>(rec + R::OFF_V, vin + (size_t)e * K::DIN * C, C, lane);
   }
   if (BWD) {
@@ -254,8 +260,8 @@ __device__ __forceinline__ void stage_edge(float* rec, int e, int lane, int C, i
   }
 }
 
-template <int LMAX, int INK, int OUTK, int CT, bool WB>
-__global__ void __launch_bounds__(128, 8)
+template <int LMAX, int INK, int OUTK, int CT, bool WB, bool SMALL>
+__global__ void __launch_bounds__(128, SMALL ? 4 : 8)
 k_env_tp_fwd(int n_atoms, int C, const int* __restrict__ row_ptr, int e0,
              const float* __restrict__ ef,
              const typename std::conditional<WB, __nv_bfloat16, float>::type* __restrict__ W,
@@ -264,22 +270,26 @@ k_env_tp_fwd(int n_atoms, int C, const int* __restrict__ row_ptr, int e0,
              float* __restrict__ X, __nv_bfloat16* __restrict__ Xb, int ldx, int D,
              float* __restrict__ Vout, float* __restrict__ Gam, float inv_sqrt_nu) {
   using K = TPK<LMAX, INK, OUTK>;
-  using R = EdgeRec<LMAX, INK, OUTK, CT, false, WB>;
+  using R = EdgeRec<LMAX, INK, OUTK, CT, false, WB, SMALL>;
   constexpr bool LAST = R::LAST;
   constexpr int NY = (LMAX + 1) * (LMAX + 1);
   constexpr int NSTG = R::NSTG, SST = R::SST;
   __shared__ __align__(16) float s_rec[R::TEAMS * R::BUF];
   const int G = C / CT;
   const int team = threadIdx.x / CT, lane = threadIdx.x % CT;
-  const long long tg = (long long)blockIdx.x * R::TEAMS + team;
+  // SMALL: the block's teams share an atom; each sums the environment itself (the same sum)
+  // and takes its part of the edges in the tensor products
+  const long long tg = SMALL ? blockIdx.x : (long long)blockIdx.x * R::TEAMS + team;
   const int a = (int)(tg / G), grp = (int)(tg - (long long)a * G);
   if (a >= n_atoms) return;
   const int c = grp * CT + lane;
   const int eb = row_ptr[a] - e0, ee = row_ptr[a + 1] - e0;
+  const int tb = SMALL ? eb + (ee - eb) * team / R::TEAMS : eb;
+  const int te = SMALL ? eb + (ee - eb) * (team + 1) / R::TEAMS : ee;
   float* buf = s_rec + team * R::BUF;
   const float* vin = Vin + grp * CT;
   auto fetch = [&](int e, int slot) {
-    stage_edge<LMAX, INK, OUTK, CT, false, WB>(buf + slot * SST, e, lane, C, grp, ef, W, ldw,
+    stage_edge<LMAX, INK, OUTK, CT, false, WB, SMALL>(buf + slot * SST, e, lane, C, grp, ef, W, ldw,
                                                vin, nullptr, 0, 0, nullptr);
   };
   // environment sum over a ring of (edge-feature row, env-weight slice) records
@@ -315,18 +325,18 @@ k_env_tp_fwd(int n_atoms, int C, const int* __restrict__ row_ptr, int e0,
 #pragma unroll
   for (int k = 0; k < NY; ++k) {
     G_[k] *= inv_sqrt_nu;
-    Gam[((size_t)a * NY + k) * C + c] = G_[k];
+    if (!SMALL || team == 0) Gam[((size_t)a * NY + k) * C + c] = G_[k];
   }
   // tensor products over the ring of full records
 #pragma unroll
   for (int p = 0; p < NSTG - 1; ++p) {
-    if (eb + p < ee) fetch(eb + p, p);
+    if (tb + p < te) fetch(tb + p, p);
     cp_commit();
   }
   const float* th = thetaT + (size_t)c * K::NP;
-  for (int e = eb; e < ee; ++e) {
-    const int i = e - eb;
-    if (e + NSTG - 1 < ee) fetch(e + NSTG - 1, (i + NSTG - 1) % NSTG);
+  for (int e = tb; e < te; ++e) {
+    const int i = e - tb;
+    if (e + NSTG - 1 < te) fetch(e + NSTG - 1, (i + NSTG - 1) % NSTG);
     cp_commit();
     cp_wait<NSTG - 1>();
     __syncwarp(team_mask<CT>());
@@ -370,8 +380,13 @@ k_env_tp_fwd(int n_atoms, int C, const int* __restrict__ row_ptr, int e0,
 // (Resident blocks of 4 warps per SM: eight for the last layer, whose adjoint has no
 // feature gradients to keep, five for the others, the count the first layer's shared
 // memory allows; the register budget follows, at most 64 and 96 a thread.)
-template <int LMAX, int INK, int OUTK, int CT, bool WB>
-__global__ void __launch_bounds__(128, OUTK == 2 ? 8 : 5)
+//
+// SMALL: the block's teams share an atom.  The environment gradient is a sum over the edges in
+// order, so one team forms it for all of them and nothing else, while the others form the
+// feature gradients of their parts of the edges; the second pass is split among all.  The two
+// halves of the tensor-product adjoint share only the gradients of the products.
+template <int LMAX, int INK, int OUTK, int CT, bool WB, bool SMALL>
+__global__ void __launch_bounds__(128, SMALL ? 4 : (OUTK == 2 ? 8 : 5))
 k_env_tp_bwd(int n_atoms, int C, const int* __restrict__ row_ptr, int e0,
              const float* __restrict__ ef,
              const typename std::conditional<WB, __nv_bfloat16, float>::type* __restrict__ W,
@@ -382,28 +397,36 @@ k_env_tp_bwd(int n_atoms, int C, const int* __restrict__ row_ptr, int e0,
              float* __restrict__ gY_v0, float* __restrict__ gY_env, int gy_stride,
              const float* __restrict__ Gam, float inv_sqrt_nu) {
   using K = TPK<LMAX, INK, OUTK>;
-  using R = EdgeRec<LMAX, INK, OUTK, CT, true, WB>;
+  using R = EdgeRec<LMAX, INK, OUTK, CT, true, WB, SMALL>;
   constexpr bool LAST = R::LAST;
   constexpr int NY = (LMAX + 1) * (LMAX + 1);
   constexpr int NSTG = R::NSTG, SST = R::SST;
   __shared__ __align__(16) float s_rec[R::TEAMS * R::BUF];
   const int G = C / CT;
   const int team = threadIdx.x / CT, lane = threadIdx.x % CT;
-  const long long tg = (long long)blockIdx.x * R::TEAMS + team;
+  const long long tg = SMALL ? blockIdx.x : (long long)blockIdx.x * R::TEAMS + team;
   const int a = (int)(tg / G), grp = (int)(tg - (long long)a * G);
   if (a >= n_atoms) return;
   const int c = grp * CT + lane;
   const int eb = row_ptr[a] - e0, ee = row_ptr[a + 1] - e0;
+  // roles and edge ranges of the passes: with teams of half a warp, the other half of the
+  // environment team's warp idles in the first pass
+  constexpr int VT0 = 32 / CT;                  // first team of the feature gradients
+  constexpr int NVT = R::TEAMS - VT0;
+  const bool do_g = !SMALL || team == 0, do_v = !SMALL || team >= VT0;
+  const int len = ee - eb;
+  const int tb = SMALL ? (do_g ? eb : do_v ? eb + len * (team - VT0) / NVT : ee) : eb;
+  const int te = SMALL && !do_g && do_v ? eb + len * (team - VT0 + 1) / NVT : ee;
   float* buf = s_rec + team * R::BUF;
   const float* vin = Vin + grp * CT;
   const float* gvout = gVout + grp * CT;
   auto fetch = [&](int e, int slot) {
-    stage_edge<LMAX, INK, OUTK, CT, true, WB>(buf + slot * SST, e, lane, C, grp, ef, W, ldw,
-                                              vin, GX, ldx, D, gvout);
+    stage_edge<LMAX, INK, OUTK, CT, true, WB, SMALL>(buf + slot * SST, e, lane, C, grp, ef, W,
+                                                     ldw, vin, GX, ldx, D, gvout, do_g);
   };
 #pragma unroll
   for (int p = 0; p < NSTG - 1; ++p) {
-    if (eb + p < ee) fetch(eb + p, p);
+    if (tb + p < te) fetch(tb + p, p);
     cp_commit();
   }
   float G_[NY], gG[NY];
@@ -414,9 +437,9 @@ k_env_tp_bwd(int n_atoms, int C, const int* __restrict__ row_ptr, int e0,
   }
   const float* th = thetaT + (size_t)c * K::NP;
   const int ridx = rs_index<CT, NY>(lane);
-  for (int e = eb; e < ee; ++e) {
-    const int i = e - eb;
-    if (e + NSTG - 1 < ee) fetch(e + NSTG - 1, (i + NSTG - 1) % NSTG);
+  for (int e = tb; e < te; ++e) {
+    const int i = e - tb;
+    if (e + NSTG - 1 < te) fetch(e + NSTG - 1, (i + NSTG - 1) % NSTG);
     cp_commit();
     cp_wait<NSTG - 1>();
     __syncwarp(team_mask<CT>());
@@ -434,7 +457,7 @@ k_env_tp_bwd(int n_atoms, int C, const int* __restrict__ row_ptr, int e0,
         for (int m = 0; m < 2 * l + 1; ++m) v[l * l + m] = wl[l] * y[l * l + m];
     } else {
 #pragma unroll
-      for (int k = 0; k < K::DIN; ++k) v[k] = rec[R::OFF_V + k * CT + lane];
+      for (int k = 0; k < K::DIN; ++k) v[k] = do_g ? rec[R::OFF_V + k * CT + lane] : 0.f;
     }
 #pragma unroll
     for (int k = 0; k < K::DIN; ++k) gv[k] = 0.f;
@@ -443,7 +466,22 @@ k_env_tp_bwd(int n_atoms, int C, const int* __restrict__ row_ptr, int e0,
     for (int q = 0; q < K::NS; ++q) gs[q] = rec[R::OFF_GS + q * CT + lane];
 #pragma unroll
     for (int k = 0; k < K::DOUT; ++k) gvo[k] = LAST ? 0.f : rec[R::OFF_GVO + k * CT + lane];
-    K::template bwd<1>(v, G_, th, gs, gvo, gv, gG);
+    if (SMALL && do_g) {
+      float unused[K::DIN];
+#pragma unroll
+      for (int k = 0; k < K::DIN; ++k) unused[k] = 0.f;
+      K::template bwd<1>(v, G_, th, gs, gvo, unused, gG);   // its gG half
+      __syncwarp(team_mask<CT>());
+      continue;
+    }
+    if (SMALL) {
+      float unused[NY];
+#pragma unroll
+      for (int k = 0; k < NY; ++k) unused[k] = 0.f;
+      K::template bwd<1>(v, G_, th, gs, gvo, gv, unused);   // its gv half
+    } else {
+      K::template bwd<1>(v, G_, th, gs, gvo, gv, gG);
+    }
     if (INK == 0) {
       // V^0 = w (x) Y: gradient to the env weights and to the harmonics
       float p[NY];
@@ -472,6 +510,18 @@ k_env_tp_bwd(int n_atoms, int C, const int* __restrict__ row_ptr, int e0,
   // are fetched as far ahead as the rest of the record
 #pragma unroll
   for (int k = 0; k < NY; ++k) gG[k] *= inv_sqrt_nu;
+  if (SMALL) {   // (the barrier also orders the first pass's weight gradients before their reads)
+    __shared__ float s_gG[NY][CT];
+    if (do_g) {
+#pragma unroll
+      for (int k = 0; k < NY; ++k) s_gG[k][lane] = gG[k];
+    }
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < NY; ++k) gG[k] = s_gG[k][lane];
+  }
+  const int pb = SMALL ? eb + len * team / R::TEAMS : eb;
+  const int pe = SMALL ? eb + len * (team + 1) / R::TEAMS : ee;
   constexpr int SR = R::SR, NSR = R::NSR;
   auto fetch1 = [&](int e, int slot) {
     stage_ef_w<LMAX, CT>(buf + slot * SR, e, lane, C, grp, ef, W, ldw);
@@ -482,12 +532,12 @@ k_env_tp_bwd(int n_atoms, int C, const int* __restrict__ row_ptr, int e0,
   __syncwarp(team_mask<CT>());
 #pragma unroll
   for (int p = 0; p < NSR - 1; ++p) {
-    if (eb + p < ee) fetch1(eb + p, p);
+    if (pb + p < pe) fetch1(pb + p, p);
     cp_commit();
   }
-  for (int e = eb; e < ee; ++e) {
-    const int i = e - eb;
-    if (e + NSR - 1 < ee) fetch1(e + NSR - 1, (i + NSR - 1) % NSR);
+  for (int e = pb; e < pe; ++e) {
+    const int i = e - pb;
+    if (e + NSR - 1 < pe) fetch1(e + NSR - 1, (i + NSR - 1) % NSR);
     cp_commit();
     cp_wait<NSR - 1>();
     __syncwarp(team_mask<CT>());
@@ -515,37 +565,21 @@ k_env_tp_bwd(int n_atoms, int C, const int* __restrict__ row_ptr, int e0,
   }
 }
 
-template <int LMAX, int INK, int OUTK, int CT>
-void fwd_one(int n_atoms, int C, const int* row_ptr, int e0, const float* ef, const void* W,
-             int wb, int ldw, const float* Vin, const float* thetaT, float* X,
-             __nv_bfloat16* Xb, int ldx, int D, float* Vout, float* Gam, float inv_sqrt_nu,
-             cudaStream_t s) {
-  const long long teams = (long long)n_atoms * (C / CT);
-  if (wb)
-    k_env_tp_fwd<LMAX, INK, OUTK, CT, true><<<ff_cdiv(teams * CT, 128), 128, 0, s>>>(
-        n_atoms, C, row_ptr, e0, ef, (const __nv_bfloat16*)W, ldw, Vin, thetaT, X, Xb, ldx, D,
-        Vout, Gam, inv_sqrt_nu);
-  else
-    k_env_tp_fwd<LMAX, INK, OUTK, CT, false><<<ff_cdiv(teams * CT, 128), 128, 0, s>>>(
-        n_atoms, C, row_ptr, e0, ef, (const float*)W, ldw, Vin, thetaT, X, Xb, ldx, D, Vout,
-        Gam, inv_sqrt_nu);
-}
-
-template <int LMAX, int INK, int OUTK, int CT>
-void bwd_one(int n_atoms, int C, const int* row_ptr, int e0, const float* ef, const void* W,
-             int wb, int ldw, const float* Vin, const float* thetaT, const float* GX, int ldx,
-             int D, const float* gVout, float* gVin, float* GW, __nv_bfloat16* GWb,
-             float* gY_v0, float* gY_env, int gy_stride, const float* Gam, float inv_sqrt_nu,
-             cudaStream_t s) {
-  const long long teams = (long long)n_atoms * (C / CT);
-  if (wb)
-    k_env_tp_bwd<LMAX, INK, OUTK, CT, true><<<ff_cdiv(teams * CT, 128), 128, 0, s>>>(
-        n_atoms, C, row_ptr, e0, ef, (const __nv_bfloat16*)W, ldw, Vin, thetaT, GX, ldx, D,
-        gVout, gVin, GW, GWb, gY_v0, gY_env, gy_stride, Gam, inv_sqrt_nu);
-  else
-    k_env_tp_bwd<LMAX, INK, OUTK, CT, false><<<ff_cdiv(teams * CT, 128), 128, 0, s>>>(
-        n_atoms, C, row_ptr, e0, ef, (const float*)W, ldw, Vin, thetaT, GX, ldx, D, gVout,
-        gVin, GW, GWb, gY_v0, gY_env, gy_stride, Gam, inv_sqrt_nu);
+// Whether a launch over `teams` (atom, channel group) pairs uses the SMALL variant: a block per
+// pair fills the SMs' issue slots that a warp per pair leaves idle, but computes the products'
+// gradients twice.  Per evaluation, forward + adjoint, us, without and with it: 96 atoms (l <= 1)
+// 130 and 79, 512 teams 420 and 335, but 2,048 teams 451 and 492 (C = 32), 308 and 392 (C = 128),
+// 4,095 teams 1,738 and 2,129.
+inline bool use_small(long long teams) {
+  static int n_sm = 0;
+  if (!n_sm) {
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+      cudaGetLastError();
+    n_sm = sms > 0 ? sms : 1;
+  }
+  return teams <= 4LL * n_sm;
 }
 
 // (input kind, output kind) of every layer of a 1- to 4-layer model; see TPK above.
@@ -586,30 +620,3 @@ void bwd_one(int n_atoms, int C, const int* row_ptr, int e0, const float* ef, co
   } while (0)
 
 }  // namespace
-
-
-void launch_env_tp_fwd(int lmax, int in_kind, int out_kind, int C, int n_atoms,
-                       const int* row_ptr, int e0, const float* ef, const void* W, int w_bf16,
-                       int ldw,
-                       const float* Vin, const float* theta, float* X, __nv_bfloat16* Xb,
-                       int ldx, int D, float* Vout, float* Gam, float inv_sqrt_nu,
-                       cudaStream_t s) {
-  ProfScope ps_(PC_TP_FWD, s);
-  if (n_atoms <= 0) return;
-  FF_TP_DISPATCH(fwd_one, n_atoms, C, row_ptr, e0, ef, W, w_bf16, ldw, Vin, theta, X, Xb, ldx,
-                 D, Vout, Gam, inv_sqrt_nu, s);
-  ff_count_launch(1);
-}
-
-void launch_env_tp_bwd(int lmax, int in_kind, int out_kind, int C, int n_atoms,
-                       const int* row_ptr, int e0, const float* ef, const void* W, int w_bf16,
-                       int ldw,
-                       const float* Vin, const float* theta, const float* GX, int ldx, int D,
-                       const float* gVout, float* gVin, float* GW, __nv_bfloat16* GWb, float* gY_v0, float* gY_env,
-                       int gy_stride, const float* Gam, float inv_sqrt_nu, cudaStream_t s) {
-  ProfScope ps_(PC_TP_BWD, s);
-  if (n_atoms <= 0) return;
-  FF_TP_DISPATCH(bwd_one, n_atoms, C, row_ptr, e0, ef, W, w_bf16, ldw, Vin, theta, GX, ldx, D,
-                 gVout, gVin, GW, GWb, gY_v0, gY_env, gy_stride, Gam, inv_sqrt_nu, s);
-  ff_count_launch(1);
-}
