@@ -171,10 +171,11 @@ __global__ void k_cell_scatter(const int* __restrict__ cell_of, int n,
   cell_atoms[cell_start[c] + slot] = i;
 }
 
-// Rank sort of one warp's candidate keys (distinct) into the atom's Verlet row.
-__device__ void warp_rank_store(const unsigned long long* keys, int cnt, int lane,
-                                int* __restrict__ vj, int* __restrict__ vs) {
-  for (int a = lane; a < cnt; a += 32) {
+// Rank sort of an atom's candidate keys (distinct, in any order) into its Verlet row by
+// `nthr` threads.
+__device__ void rank_store(const unsigned long long* keys, int cnt, int thr, int nthr,
+                           int* __restrict__ vj, int* __restrict__ vs) {
+  for (int a = thr; a < cnt; a += nthr) {
     const unsigned long long k = keys[a];
     int rank = 0;
     for (int b = 0; b < cnt; ++b) rank += keys[b] < k;
@@ -187,6 +188,58 @@ __device__ void warp_rank_store(const unsigned long long* keys, int cnt, int lan
 
 constexpr int kWarpsPerBlockNbr = 4;
 
+// Candidates of atom i from stencil cells sub, sub + nsub, ... (one warp); store(ok, key) takes
+// a key from every lane that has one.
+template <typename S>
+__device__ __forceinline__ bool scan_stencil(int i, int sub, int nsub, const NbrGrid& g,
+                                             const int* cell_of, const int4* img,
+                                             const float4* xf, const int* cell_start,
+                                             const int* cell_atoms, float rl2, S store) {
+  const int lane = threadIdx.x & 31;
+  const int cell = cell_of[i];
+  const int c2 = cell % g.ncell[2], c1 = (cell / g.ncell[2]) % g.ncell[1],
+            c0 = cell / (g.ncell[2] * g.ncell[1]);
+  const float4 xi = xf[i];
+  const int4 imi = img[i];
+  const int n1 = 2 * g.reach[1] + 1, n2 = 2 * g.reach[2] + 1;
+  const int ncells = (2 * g.reach[0] + 1) * n1 * n2;
+  bool bad_shift = false;
+  for (int k = sub; k < ncells; k += nsub) {
+    const int k01 = k / n2;
+    int t0 = c0 + k01 / n1 - g.reach[0], q0 = 0;
+    if (g.pbc[0]) { q0 = floordiv(t0, g.ncell[0]); t0 -= q0 * g.ncell[0]; }
+    else if (t0 < 0 || t0 >= g.ncell[0]) continue;
+    int t1 = c1 + k01 % n1 - g.reach[1], q1 = 0;
+    if (g.pbc[1]) { q1 = floordiv(t1, g.ncell[1]); t1 -= q1 * g.ncell[1]; }
+    else if (t1 < 0 || t1 >= g.ncell[1]) continue;
+    int t2 = c2 + k % n2 - g.reach[2], q2 = 0;
+    if (g.pbc[2]) { q2 = floordiv(t2, g.ncell[2]); t2 -= q2 * g.ncell[2]; }
+    else if (t2 < 0 || t2 >= g.ncell[2]) continue;
+    const int cc = (t0 * g.ncell[1] + t1) * g.ncell[2] + t2;
+    const int beg = cell_start[cc], end = cell_start[cc + 1];
+    for (int base = beg; base < end; base += 32) {
+      const int idx = base + lane;
+      bool ok = false;
+      int j = 0, s0 = 0, s1 = 0, s2 = 0;
+      if (idx < end) {
+        j = cell_atoms[idx];
+        const int4 imj = img[j];
+        s0 = g.pbc[0] ? q0 + imi.x - imj.x : 0;
+        s1 = g.pbc[1] ? q1 + imi.y - imj.y : 0;
+        s2 = g.pbc[2] ? q2 + imi.z - imj.z : 0;
+        const float r2 = d2_f32(xi, xf[j], s0, s1, s2, g.Lf[0], g.Lf[1], g.Lf[2]);
+        ok = (r2 < rl2) && !(j == i && s0 == 0 && s1 == 0 && s2 == 0);
+        if (ok && (abs(s0) > 100 || abs(s1) > 100 || abs(s2) > 100)) {
+          bad_shift = true;
+          ok = false;
+        }
+      }
+      store(ok, nbr_key(j, s0, s1, s2));
+    }
+  }
+  return __any_sync(kFull, bad_shift);
+}
+
 __global__ void __launch_bounds__(32 * kWarpsPerBlockNbr)
 k_verlet_cells(int n, NbrGrid g, const int* __restrict__ cell_of, const int4* __restrict__ img,
                const float4* __restrict__ xf, const int* __restrict__ cell_start,
@@ -197,58 +250,55 @@ k_verlet_cells(int n, NbrGrid g, const int* __restrict__ cell_of, const int4* __
   const int i = blockIdx.x * kWarpsPerBlockNbr + wib;
   if (i >= n) return;
   unsigned long long* keys = sh_keys + (size_t)wib * vmax;
-  const int cell = cell_of[i];
-  const int c2 = cell % g.ncell[2], c1 = (cell / g.ncell[2]) % g.ncell[1],
-            c0 = cell / (g.ncell[2] * g.ncell[1]);
-  const float4 xi = xf[i];
-  const int4 imi = img[i];
   int cnt = 0;
-  bool bad_shift = false;
-  for (int d0 = -g.reach[0]; d0 <= g.reach[0]; ++d0) {
-    int t0 = c0 + d0, q0 = 0;
-    if (g.pbc[0]) { q0 = floordiv(t0, g.ncell[0]); t0 -= q0 * g.ncell[0]; }
-    else if (t0 < 0 || t0 >= g.ncell[0]) continue;
-    for (int d1 = -g.reach[1]; d1 <= g.reach[1]; ++d1) {
-      int t1 = c1 + d1, q1 = 0;
-      if (g.pbc[1]) { q1 = floordiv(t1, g.ncell[1]); t1 -= q1 * g.ncell[1]; }
-      else if (t1 < 0 || t1 >= g.ncell[1]) continue;
-      for (int d2 = -g.reach[2]; d2 <= g.reach[2]; ++d2) {
-        int t2 = c2 + d2, q2 = 0;
-        if (g.pbc[2]) { q2 = floordiv(t2, g.ncell[2]); t2 -= q2 * g.ncell[2]; }
-        else if (t2 < 0 || t2 >= g.ncell[2]) continue;
-        const int cc = (t0 * g.ncell[1] + t1) * g.ncell[2] + t2;
-        const int beg = cell_start[cc], end = cell_start[cc + 1];
-        for (int base = beg; base < end; base += 32) {
-          const int idx = base + lane;
-          bool ok = false;
-          int j = 0, s0 = 0, s1 = 0, s2 = 0;
-          if (idx < end) {
-            j = cell_atoms[idx];
-            const int4 imj = img[j];
-            s0 = g.pbc[0] ? q0 + imi.x - imj.x : 0;
-            s1 = g.pbc[1] ? q1 + imi.y - imj.y : 0;
-            s2 = g.pbc[2] ? q2 + imi.z - imj.z : 0;
-            const float r2 = d2_f32(xi, xf[j], s0, s1, s2, g.Lf[0], g.Lf[1], g.Lf[2]);
-            ok = (r2 < rl2) && !(j == i && s0 == 0 && s1 == 0 && s2 == 0);
-            if (ok && (abs(s0) > 100 || abs(s1) > 100 || abs(s2) > 100)) {
-              bad_shift = true;
-              ok = false;
-            }
-          }
-          const unsigned b = __ballot_sync(kFull, ok);
-          const int p = cnt + __popc(b & ((1u << lane) - 1u));
-          if (ok && p < vmax) keys[p] = nbr_key(j, s0, s1, s2);
-          cnt += __popc(b);
-        }
-      }
-    }
-  }
-  if (__any_sync(kFull, bad_shift) && lane == 0) atomicOr(err, FF_FLAG_BOX);
+  const bool bad = scan_stencil(i, 0, 1, g, cell_of, img, xf, cell_start, cell_atoms, rl2,
+                                [&](bool ok, unsigned long long key) {
+                                  const unsigned b = __ballot_sync(kFull, ok);
+                                  const int p = cnt + __popc(b & ((1u << lane) - 1u));
+                                  if (ok && p < vmax) keys[p] = key;
+                                  cnt += __popc(b);
+                                });
+  if (bad && lane == 0) atomicOr(err, FF_FLAG_BOX);
   if (cnt > vmax && lane == 0) atomicOr(err, FF_FLAG_CAPACITY);
   __syncwarp();
   const int cw = cnt < vmax ? cnt : vmax;
-  warp_rank_store(keys, cw, lane, vl_j + (size_t)i * vmax, vl_s + (size_t)i * vmax);
+  rank_store(keys, cw, lane, 32, vl_j + (size_t)i * vmax, vl_s + (size_t)i * vmax);
   if (lane == 0) vl_cnt[i] = cnt;
+}
+
+// The same list with a block of kNbrSplit warps per atom, the stencil cells dealt out among
+// them: for few atoms, where a warp walking 27 cells one after the other (a chain of three
+// dependent loads each) is all there is on an SM.  96 atoms: 25 -> 9 us.  The keys land in any
+// order; their ranks do not depend on it.
+constexpr int kNbrSplit = 8;
+__global__ void __launch_bounds__(32 * kNbrSplit)
+k_verlet_cells_split(int n, NbrGrid g, const int* __restrict__ cell_of,
+                     const int4* __restrict__ img, const float4* __restrict__ xf,
+                     const int* __restrict__ cell_start, const int* __restrict__ cell_atoms,
+                     float rl2, int vmax, int* __restrict__ vl_j, int* __restrict__ vl_s,
+                     int* __restrict__ vl_cnt, int* __restrict__ err) {
+  extern __shared__ unsigned long long sh_keys[];
+  __shared__ int s_cnt;
+  const int lane = threadIdx.x & 31, i = blockIdx.x;
+  if (threadIdx.x == 0) s_cnt = 0;
+  __syncthreads();
+  const bool bad = scan_stencil(i, threadIdx.x >> 5, kNbrSplit, g, cell_of, img, xf, cell_start,
+                                cell_atoms, rl2, [&](bool ok, unsigned long long key) {
+                                  const unsigned b = __ballot_sync(kFull, ok);
+                                  if (b == 0) return;
+                                  int base = 0;
+                                  if (lane == 0) base = atomicAdd(&s_cnt, __popc(b));
+                                  base = __shfl_sync(kFull, base, 0);
+                                  const int p = base + __popc(b & ((1u << lane) - 1u));
+                                  if (ok && p < vmax) sh_keys[p] = key;
+                                });
+  if (bad && lane == 0) atomicOr(err, FF_FLAG_BOX);
+  __syncthreads();
+  const int cnt = s_cnt;
+  if (cnt > vmax && threadIdx.x == 0) atomicOr(err, FF_FLAG_CAPACITY);
+  rank_store(sh_keys, cnt < vmax ? cnt : vmax, threadIdx.x, 32 * kNbrSplit,
+             vl_j + (size_t)i * vmax, vl_s + (size_t)i * vmax);
+  if (threadIdx.x == 0) vl_cnt[i] = cnt;
 }
 
 __global__ void k_verlet_allpairs(int n, const int* __restrict__ sys_of,
@@ -419,7 +469,14 @@ void launch_verlet_cells(int n, NbrGrid g, const int* cell_of, const int4* img, 
                          int* vl_j, int* vl_s, int* vl_cnt, int* err, cudaStream_t s) {
   ProfScope ps_(PC_NEIGHBOR, s);
   if (n <= 0) return;
-  const size_t smem = (size_t)kWarpsPerBlockNbr * vmax * sizeof(unsigned long long);
+  const size_t key_bytes = (size_t)vmax * sizeof(unsigned long long);
+  if (n <= 1024) {   // up to some seven blocks per SM
+    k_verlet_cells_split<<<n, 32 * kNbrSplit, key_bytes, s>>>(
+        n, g, cell_of, img, xf, cell_start, cell_atoms, rl2, vmax, vl_j, vl_s, vl_cnt, err);
+    ff_count_launch(1);
+    return;
+  }
+  const size_t smem = kWarpsPerBlockNbr * key_bytes;
   k_verlet_cells<<<ff_cdiv(n, kWarpsPerBlockNbr), 32 * kWarpsPerBlockNbr, smem, s>>>(
       n, g, cell_of, img, xf, cell_start, cell_atoms, rl2, vmax, vl_j, vl_s, vl_cnt, err);
   ff_count_launch(1);
