@@ -348,6 +348,7 @@ k_gemm_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUten
   __syncthreads();
   fence_after();
   const uint32_t tbase = *tslot;
+  ff_pdl();   // (the set-up above ran while the kernel ahead finished)
   const int nk = (K + TK - 1) / TK;
   const int quad = warp & 3, half = warp >> 2;
   const int nchunks = (nbw + 31) / 32;
@@ -678,6 +679,7 @@ k_gemm_pp(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUten
   __syncthreads();
   fence_after();
   const uint32_t tbase = *tslot;
+  ff_pdl();   // (the set-up above ran while the kernel ahead finished)
 
   if (warp == PP_EW) {
     // ---- TMA producer
@@ -1014,8 +1016,8 @@ bool launch_nw(const CUtensorMap& ta, const CUtensorMap& ta2, const CUtensorMap&
   if (bytes > 200 * 1024) return false;
   // one CTA per (row tile, column slice), the slices of a row tile adjacent so the second
   // reads the A tile from L2
-  k_gemm_tc<MODE, NW><<<ff_cdiv(M, TM) * nslices, 32 * NW, bytes, s>>>(
-      ta, ta2, tb, tx, M, N, K, k1c, nslices, nbw, stages, aux_tma, ep, err);
+  ff_launch(k_gemm_tc<MODE, NW>, ff_cdiv(M, TM) * nslices, 32 * NW, bytes, s, ta, ta2, tb, tx, M,
+            N, K, k1c, nslices, nbw, stages, aux_tma, ep, err);
   return true;
 }
 
@@ -1068,8 +1070,9 @@ bool launch_pp(const CUtensorMap& ta, const CUtensorMap& ta2, const CUtensorMap&
   if (pp_ring_bytes(stages, nbw) + fixed > kMaxSmem) return false;
   const int ntiles = ff_cdiv(M, TM) * nslices;
   const int grid = ntiles < n_sm ? ntiles : n_sm;
-  k_gemm_pp<MODE, ROW><<<grid, pp_threads<MODE>(), pp_ring_bytes(stages, nbw) + fixed, s>>>(
-      ta, ta2, tb, tx, tx2, to, M, N, K, k1c, nslices, nbw, stages, aux_tma, ep, err);
+  ff_launch_work(ntiles, k_gemm_pp<MODE, ROW>, grid, pp_threads<MODE>(),
+                 pp_ring_bytes(stages, nbw) + fixed, s, ta, ta2, tb, tx, tx2, to, M, N, K, k1c,
+                 nslices, nbw, stages, aux_tma, ep, err);
   return true;
 }
 

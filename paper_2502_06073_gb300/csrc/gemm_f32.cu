@@ -168,6 +168,7 @@ __device__ __forceinline__ void ld8(const float* p, float (&v)[8]) {
 __global__ void k_split_weights(const float* __restrict__ W1, const float* __restrict__ W2, int N,
                                 int K1, int K2, int k1p, double scale,
                                 __nv_bfloat16* __restrict__ out) {
+  ff_pdl();
   const int K = k1p + K2, nk = (K + FS_TK - 1) / FS_TK;
   const long long t = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   if (t >= (long long)N * nk) return;
@@ -252,6 +253,7 @@ k_gemm_fs(const __grid_constant__ CUtensorMap tmB, const float* __restrict__ A, 
   __syncthreads();
   fence_after();
   const uint32_t tbase = *tslot;
+  ff_pdl();   // (the set-up above ran while the kernel ahead finished)
 
   if (warp >= FS_EW && warp < FS_EW + FS_CW) {
     // ---- splitting group g: chunks q = g mod 2 of this CTA's (tile, K-chunk) sequence; two
@@ -630,8 +632,8 @@ bool launch_fs(const CUtensorMap& tb, const float* A, int lda, const float* A2, 
                        FS_EW * 32 * 16 * 4 + FS_EW * fs_auxn<MODE>() * fs_naux<MODE>() * 2048 +
                        1024 + 256;
   const int ntiles = ff_cdiv(M, TM) * nslices;
-  k_gemm_fs<MODE><<<ntiles < n_sm ? ntiles : n_sm, FS_THREADS, bytes, s>>>(
-      tb, A, lda, A2, lda2, M, N, K1, K2, nslices, nbw, ep, err);
+  ff_launch_work(ntiles, k_gemm_fs<MODE>, ntiles < n_sm ? ntiles : n_sm, FS_THREADS, bytes, s, tb,
+                 A, lda, A2, lda2, M, N, K1, K2, nslices, nbw, ep, err);
   return true;
 }
 
@@ -652,7 +654,7 @@ void launch_split_weights(const float* W1, int N, int K1, const float* W2, int K
                           __nv_bfloat16* out, cudaStream_t s) {
   const int ld = split_ld(K1, K2);
   const long long n = (long long)N * ((ld + FS_TK - 1) / FS_TK);
-  k_split_weights<<<ff_cdiv(n, 8), 256, 0, s>>>(W1, W2, N, K1, K2, ld - K2, scale, out);
+  ff_launch(k_split_weights, ff_cdiv(n, 8), 256, 0, s, W1, W2, N, K1, K2, ld - K2, scale, out);
   ff_count_launch(1);
 }
 

@@ -47,6 +47,7 @@ __global__ void k_edge_features(long long E, const int* __restrict__ src,
                                 const int* __restrict__ Z, float rc, int n_basis, int p,
                                 int lmax, float* __restrict__ ef, int* __restrict__ zz,
                                 float* __restrict__ fenv) {
+  ff_pdl();
   const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= E) return;
   const int i = src[e], j = col[e];
@@ -114,6 +115,7 @@ __global__ void k_twobody_in(long long E, int width, int n_basis, const float* _
                              __nv_bfloat16* __restrict__ preb, float* __restrict__ out,
                              int ldo, __nv_bfloat16* __restrict__ outb, int ldob,
                              int final_layer) {
+  ff_pdl();
   const int tpe = width >> 2;                 // threads per edge
   const int epb = blockDim.x / tpe;
   const int slot = threadIdx.x / tpe, o = 4 * (threadIdx.x - slot * tpe);
@@ -178,6 +180,7 @@ constexpr int kEnergyCols = 16, kEnergyRows = 4;
 __global__ void k_energy(int n_atoms, const int* __restrict__ row_ptr, int e0,
                          const float* __restrict__ X, int ldx, int D,
                          const float* __restrict__ w_eff, float* __restrict__ E_atom) {
+  ff_pdl();
   const int a = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (a >= n_atoms) return;
@@ -211,6 +214,7 @@ __global__ void k_energy(int n_atoms, const int* __restrict__ row_ptr, int e0,
 __global__ void k_energy_sum(int n_atoms, const int* __restrict__ row_ptr, int e0,
                              const float* __restrict__ E_edge, int nsl, long long ld,
                              float* __restrict__ E_atom) {
+  ff_pdl();
   const int a = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (a >= n_atoms) return;
@@ -235,6 +239,7 @@ __global__ void k_rowred_bwd(long long E, int N, const float* __restrict__ gx, i
                              const __nv_bfloat16* __restrict__ zb, int ldz,
                              const float* __restrict__ ef, float alpha, float* __restrict__ gz,
                              int ldgz, __nv_bfloat16* __restrict__ gzb, float* __restrict__ gf) {
+  ff_pdl();
   const long long eb = ((long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * EPW;
   const int lane = threadIdx.x & 31;
   if (eb >= E) return;
@@ -297,8 +302,8 @@ template <int NGL, int EPW>
 void rowred_one(long long E, int N, const float* gx, int ldgx, const __nv_bfloat16* zb, int ldz,
                 const float* ef, float alpha, float* gz, int ldgz, __nv_bfloat16* gzb, float* gf,
                 cudaStream_t s) {
-  k_rowred_bwd<NGL, EPW><<<ff_cdiv(E, 8 * EPW), 256, 0, s>>>(E, N, gx, ldgx, zb, ldz, ef, alpha,
-                                                             gz, ldgz, gzb, gf);
+  ff_launch(k_rowred_bwd<NGL, EPW>, ff_cdiv(E, 8 * EPW), 256, 0, s, E, N, gx, ldgx, zb, ldz, ef,
+            alpha, gz, ldgz, gzb, gf);
 }
 
 // dE/dr_e from the radial-basis gradient (via the first two-body layer), the envelope
@@ -315,6 +320,7 @@ __global__ void k_edge_grad(long long E, int w0, int n_basis, float rc, int p, i
                             int gy_groups, const int* __restrict__ src,
                             const int* __restrict__ sys_of, const double* __restrict__ seed,
                             float4* __restrict__ g) {
+  ff_pdl();
   extern __shared__ float s_wb[];
   for (int i = threadIdx.x; i < n_basis * w0; i += blockDim.x) s_wb[i] = WB[i];
   __syncthreads();
@@ -392,6 +398,7 @@ __global__ void k_edge_grad(long long E, int w0, int n_basis, float rc, int p, i
 // F_m = sum_{e in seg(m)} (g_e - g_rev(e)); one warp per atom, fixed order.
 __global__ void k_force_gather(int n, const int* __restrict__ row_ptr, const int* __restrict__ rev,
                                const float4* __restrict__ g, float* __restrict__ F) {
+  ff_pdl();
   const int m = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (m >= n) return;
@@ -435,6 +442,7 @@ __global__ void k_virial_part(const int* __restrict__ sys_ptr, const int* __rest
                               const int* __restrict__ shift, const double* __restrict__ pos,
                               const double* __restrict__ L, const float4* __restrict__ g,
                               double* __restrict__ part) {
+  ff_pdl();
   __shared__ double sh[32];
   const int k = blockIdx.y, b = blockIdx.x;
   const long long e0 = row_ptr[sys_ptr[k]], e1 = row_ptr[sys_ptr[k + 1]];
@@ -466,6 +474,7 @@ __global__ void k_virial_part(const int* __restrict__ sys_ptr, const int* __rest
 }
 
 __global__ void k_virial_final(const double* __restrict__ part, int n_sys, double* __restrict__ W) {
+  ff_pdl();
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= n_sys * 9) return;
   const int k = t / 9, q = t % 9;
@@ -476,6 +485,7 @@ __global__ void k_virial_final(const double* __restrict__ part, int n_sys, doubl
 
 __global__ void k_esys(const float* __restrict__ E_atom, const int* __restrict__ sys_ptr,
                        double* __restrict__ E_sys) {
+  ff_pdl();
   __shared__ double sh[32];
   const int sy = blockIdx.x;
   double acc = 0.0;
@@ -489,6 +499,7 @@ constexpr double kAcc = 9.648533212e-3;   // (eV / (A amu)) -> A / fs^2
 
 __global__ void k_kick(int n, double* __restrict__ v, const float* __restrict__ F,
                        const double* __restrict__ mass, double hdt) {
+  ff_pdl();
   const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= 3LL * n) return;
   v[t] += hdt * kAcc * (double)F[t] / mass[t / 3];
@@ -496,6 +507,7 @@ __global__ void k_kick(int n, double* __restrict__ v, const float* __restrict__ 
 
 __global__ void k_drift(long long n3, double* __restrict__ x, const double* __restrict__ v,
                         double dt) {
+  ff_pdl();
   const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= n3) return;
   x[t] += dt * v[t];
@@ -503,6 +515,7 @@ __global__ void k_drift(long long n3, double* __restrict__ x, const double* __re
 
 __global__ void k_kinetic(const double* __restrict__ v, const double* __restrict__ mass,
                           const int* __restrict__ sys_ptr, double* __restrict__ E_kin) {
+  ff_pdl();
   __shared__ double sh[32];
   const int sy = blockIdx.x;
   double acc = 0.0;
@@ -517,6 +530,7 @@ __global__ void k_kinetic(const double* __restrict__ v, const double* __restrict
 // dst[r][col0 + c] = bf16(src[r][col0 + c]) for c < ncols
 __global__ void k_cvt_bf16(const float* __restrict__ src, int lds, __nv_bfloat16* __restrict__ dst,
                            int ldd, long long rows, int col0, int ncols) {
+  ff_pdl();
   const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= rows * ncols) return;
   const long long r = t / ncols;
@@ -529,6 +543,7 @@ __global__ void k_cvt_bf16(const float* __restrict__ src, int lds, __nv_bfloat16
 __global__ void k_nh_update(int n_sys, const int* __restrict__ sys_ptr,
                             const double* __restrict__ ke, double* __restrict__ thermo,
                             double* __restrict__ scale, double dt, double kT, double tau) {
+  ff_pdl();
   const int k = blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= n_sys) return;
   const double g = 3.0 * (sys_ptr[k + 1] - sys_ptr[k]);
@@ -546,6 +561,7 @@ __global__ void k_nh_update(int n_sys, const int* __restrict__ sys_ptr,
 
 __global__ void k_scale_v(long long n3, const int* __restrict__ sys_of,
                           const double* __restrict__ scale, double* __restrict__ v) {
+  ff_pdl();
   const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= n3) return;
   v[t] *= scale[sys_of[t / 3]];
@@ -556,6 +572,7 @@ __global__ void k_nh_energy(int n_sys, const int* __restrict__ sys_ptr,
                             const double* __restrict__ epot, const double* __restrict__ ke,
                             const double* __restrict__ thermo, double kT, double tau,
                             double* __restrict__ H) {
+  ff_pdl();
   const int k = blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= n_sys) return;
   const double g = 3.0 * (sys_ptr[k + 1] - sys_ptr[k]);
@@ -564,11 +581,13 @@ __global__ void k_nh_energy(int n_sys, const int* __restrict__ sys_ptr,
 }
 
 __global__ void k_fill_f32(float* __restrict__ p, long long n, float v) {
+  ff_pdl();
   const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (t < n) p[t] = v;
 }
 
 __global__ void k_check_finite(const float* __restrict__ F, long long n, int* __restrict__ err) {
+  ff_pdl();
   const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (t < n && !isfinite(F[t])) atomicOr(err, FF_FLAG_NONFINITE_F);
 }
@@ -587,8 +606,8 @@ void launch_edge_features(long long E, const int* src, const int* col, const int
   ProfScope ps_(PC_EDGE_FEAT, s);
   if (E <= 0) return;
   const int nt = edge_threads(E);
-  k_edge_features<<<ff_cdiv(E, nt), nt, 0, s>>>(E, src, col, shift, pos, L, Z, rc, n_basis, p,
-                                                 lmax, ef, zz, fenv);
+  ff_launch(k_edge_features, ff_cdiv(E, nt), nt, 0, s, E, src, col, shift, pos, L, Z, rc, n_basis,
+            p, lmax, ef, zz, fenv);
   ff_count_launch(1);
 }
 
@@ -602,11 +621,11 @@ void launch_twobody_in(long long E, int width, int n_basis, const float* ef, con
   if (E <= 0) return;
   const int epb = 256 / (width / 4);
   if (E >= kTwobodyWide)
-    k_twobody_in<4><<<ff_cdiv(E, 4 * epb), 256, 0, s>>>(E, width, n_basis, ef, zz, W0, alpha, pre,
-                                                        preb, out, ldo, outb, ldob, final_layer);
+    ff_launch(k_twobody_in<4>, ff_cdiv(E, 4 * epb), 256, 0, s, E, width, n_basis, ef, zz, W0,
+              alpha, pre, preb, out, ldo, outb, ldob, final_layer);
   else
-    k_twobody_in<1><<<ff_cdiv(E, epb), 256, 0, s>>>(E, width, n_basis, ef, zz, W0, alpha, pre, preb,
-                                                    out, ldo, outb, ldob, final_layer);
+    ff_launch(k_twobody_in<1>, ff_cdiv(E, epb), 256, 0, s, E, width, n_basis, ef, zz, W0, alpha,
+              pre, preb, out, ldo, outb, ldob, final_layer);
   ff_count_launch(1);
 }
 
@@ -614,7 +633,8 @@ void launch_energy(int n_atoms, const int* row_ptr, int e0, const float* X, int 
                    const float* w_eff, float* E_atom, cudaStream_t s) {
   ProfScope ps_(PC_ENERGY, s);
   if (n_atoms <= 0) return;
-  k_energy<<<ff_cdiv(n_atoms, 8), 256, 0, s>>>(n_atoms, row_ptr, e0, X, ldx, D, w_eff, E_atom);
+  ff_launch(k_energy, ff_cdiv(n_atoms, 8), 256, 0, s, n_atoms, row_ptr, e0, X, ldx, D, w_eff,
+            E_atom);
   ff_count_launch(1);
 }
 
@@ -622,8 +642,8 @@ void launch_energy_sum(int n_atoms, const int* row_ptr, int e0, const float* E_e
                        long long ld, float* E_atom, cudaStream_t s) {
   ProfScope ps_(PC_ENERGY, s);
   if (n_atoms <= 0) return;
-  k_energy_sum<<<ff_cdiv(n_atoms, 8), 256, 0, s>>>(n_atoms, row_ptr, e0, E_edge, nsl, ld,
-                                                   E_atom);
+  ff_launch(k_energy_sum, ff_cdiv(n_atoms, 8), 256, 0, s, n_atoms, row_ptr, e0, E_edge, nsl, ld,
+            E_atom);
   ff_count_launch(1);
 }
 
@@ -649,13 +669,11 @@ void launch_edge_grad(long long E, int w0, int n_basis, float rc, int p, int lma
   const int nt = edge_threads(E);
   const size_t smem = (size_t)n_basis * w0 * sizeof(float);
   if (gy_groups % 4 == 0)
-    k_edge_grad<true><<<ff_cdiv(E, nt), nt, smem, s>>>(E, w0, n_basis, rc, p, lmax, ef, gz0, ldg,
-                                                       WB, alpha0, gf, gfp, n_gfp, gfp_ld, gY,
-                                                       gy_groups, src, sys_of, seed, g);
+    ff_launch(k_edge_grad<true>, ff_cdiv(E, nt), nt, smem, s, E, w0, n_basis, rc, p, lmax, ef,
+              gz0, ldg, WB, alpha0, gf, gfp, n_gfp, gfp_ld, gY, gy_groups, src, sys_of, seed, g);
   else
-    k_edge_grad<false><<<ff_cdiv(E, nt), nt, smem, s>>>(E, w0, n_basis, rc, p, lmax, ef, gz0, ldg,
-                                                        WB, alpha0, gf, gfp, n_gfp, gfp_ld, gY,
-                                                        gy_groups, src, sys_of, seed, g);
+    ff_launch(k_edge_grad<false>, ff_cdiv(E, nt), nt, smem, s, E, w0, n_basis, rc, p, lmax, ef,
+              gz0, ldg, WB, alpha0, gf, gfp, n_gfp, gfp_ld, gY, gy_groups, src, sys_of, seed, g);
   ff_count_launch(1);
 }
 
@@ -663,7 +681,7 @@ void launch_force_gather(int n, const int* row_ptr, const int* rev, const float4
                          cudaStream_t s) {
   ProfScope ps_(PC_FORCE_GATHER, s);
   if (n <= 0) return;
-  k_force_gather<<<ff_cdiv(n, 8), 256, 0, s>>>(n, row_ptr, rev, g, F);
+  ff_launch(k_force_gather, ff_cdiv(n, 8), 256, 0, s, n, row_ptr, rev, g, F);
   ff_count_launch(1);
 }
 
@@ -672,9 +690,9 @@ void launch_virial(const int* sys_ptr, int n_sys, const int* row_ptr, const int*
                    const float4* g, double* part, double* W, cudaStream_t s) {
   ProfScope ps_(PC_MISC, s);
   if (n_sys <= 0) return;
-  k_virial_part<<<dim3(kVirBlocks, n_sys), 256, 0, s>>>(sys_ptr, row_ptr, src, col, shift, pos, L,
-                                                       g, part);
-  k_virial_final<<<ff_cdiv(n_sys * 9, 256), 256, 0, s>>>(part, n_sys, W);
+  ff_launch(k_virial_part, dim3(kVirBlocks, n_sys), 256, 0, s, sys_ptr, row_ptr, src, col, shift,
+            pos, L, g, part);
+  ff_launch(k_virial_final, ff_cdiv(n_sys * 9, 256), 256, 0, s, part, n_sys, W);
   ff_count_launch(2);
 }
 
@@ -682,7 +700,7 @@ void launch_esys(const float* E_atom, const int* sys_ptr, int n_sys, double* E_s
                  cudaStream_t s) {
   ProfScope ps_(PC_MISC, s);
   if (n_sys <= 0) return;
-  k_esys<<<n_sys, 256, 0, s>>>(E_atom, sys_ptr, E_sys);
+  ff_launch(k_esys, n_sys, 256, 0, s, E_atom, sys_ptr, E_sys);
   ff_count_launch(1);
 }
 
@@ -690,14 +708,14 @@ void launch_kick(int n, double* v, const float* F, const double* mass, double hd
                  cudaStream_t s) {
   ProfScope ps_(PC_MD, s);
   if (n <= 0) return;
-  k_kick<<<ff_cdiv(3LL * n, 256), 256, 0, s>>>(n, v, F, mass, hdt);
+  ff_launch(k_kick, ff_cdiv(3LL * n, 256), 256, 0, s, n, v, F, mass, hdt);
   ff_count_launch(1);
 }
 
 void launch_drift(int n, double* x, const double* v, double dt, cudaStream_t s) {
   ProfScope ps_(PC_MD, s);
   if (n <= 0) return;
-  k_drift<<<ff_cdiv(3LL * n, 256), 256, 0, s>>>(3LL * n, x, v, dt);
+  ff_launch(k_drift, ff_cdiv(3LL * n, 256), 256, 0, s, 3LL * n, x, v, dt);
   ff_count_launch(1);
 }
 
@@ -705,7 +723,7 @@ void launch_kinetic(const double* v, const double* mass, const int* sys_ptr, int
                     double* E_kin, cudaStream_t s) {
   ProfScope ps_(PC_MD, s);
   if (n_sys <= 0) return;
-  k_kinetic<<<n_sys, 256, 0, s>>>(v, mass, sys_ptr, E_kin);
+  ff_launch(k_kinetic, n_sys, 256, 0, s, v, mass, sys_ptr, E_kin);
   ff_count_launch(1);
 }
 
@@ -713,7 +731,8 @@ void launch_cvt_bf16(const float* src, int lds, __nv_bfloat16* dst, int ldd, lon
                      int col0, int ncols, cudaStream_t s) {
   ProfScope ps_(PC_MISC, s);
   if (rows <= 0 || ncols <= 0) return;
-  k_cvt_bf16<<<ff_cdiv(rows * ncols, 256), 256, 0, s>>>(src, lds, dst, ldd, rows, col0, ncols);
+  ff_launch(k_cvt_bf16, ff_cdiv(rows * ncols, 256), 256, 0, s, src, lds, dst, ldd, rows, col0,
+            ncols);
   ff_count_launch(1);
 }
 
@@ -723,8 +742,9 @@ void launch_nh_half(int n, int n_sys, const int* sys_ptr, const int* sys_of, dou
   if (n <= 0 || n_sys <= 0) return;
   launch_kinetic(v, mass, sys_ptr, n_sys, ke, s);
   ProfScope ps_(PC_MD, s);
-  k_nh_update<<<ff_cdiv(n_sys, 128), 128, 0, s>>>(n_sys, sys_ptr, ke, thermo, scale, dt, kT, tau);
-  k_scale_v<<<ff_cdiv(3LL * n, 256), 256, 0, s>>>(3LL * n, sys_of, scale, v);
+  ff_launch(k_nh_update, ff_cdiv(n_sys, 128), 128, 0, s, n_sys, sys_ptr, ke, thermo, scale, dt,
+            kT, tau);
+  ff_launch(k_scale_v, ff_cdiv(3LL * n, 256), 256, 0, s, 3LL * n, sys_of, scale, v);
   ff_count_launch(2);
 }
 
@@ -732,20 +752,21 @@ void launch_nh_energy(int n_sys, const int* sys_ptr, const double* epot, const d
                       const double* thermo, double kT, double tau, double* H, cudaStream_t s) {
   ProfScope ps_(PC_MD, s);
   if (n_sys <= 0) return;
-  k_nh_energy<<<ff_cdiv(n_sys, 128), 128, 0, s>>>(n_sys, sys_ptr, epot, ke, thermo, kT, tau, H);
+  ff_launch(k_nh_energy, ff_cdiv(n_sys, 128), 128, 0, s, n_sys, sys_ptr, epot, ke, thermo, kT,
+            tau, H);
   ff_count_launch(1);
 }
 
 void launch_fill_f32(float* p, long long n, float v, cudaStream_t s) {
   ProfScope ps_(PC_MISC, s);
   if (n <= 0) return;
-  k_fill_f32<<<ff_cdiv(n, 256), 256, 0, s>>>(p, n, v);
+  ff_launch(k_fill_f32, ff_cdiv(n, 256), 256, 0, s, p, n, v);
   ff_count_launch(1);
 }
 
 void launch_check_finite(const float* F, long long n, int* err, cudaStream_t s) {
   ProfScope ps_(PC_MISC, s);
   if (n <= 0) return;
-  k_check_finite<<<ff_cdiv(n, 256), 256, 0, s>>>(F, n, err);
+  ff_launch(k_check_finite, ff_cdiv(n, 256), 256, 0, s, F, n, err);
   ff_count_launch(1);
 }

@@ -63,6 +63,7 @@ __device__ int block_exclusive_scan(int x, int* sh, int& total) {
 __global__ void __launch_bounds__(1024) k_scan_block(const int* __restrict__ in,
                                                      int* __restrict__ out, int n,
                                                      int* __restrict__ bsum) {
+  ff_pdl();
   __shared__ int sh[96];
   const long long base = (long long)blockIdx.x * FF_SCAN_BLOCK + threadIdx.x * 4;
   int v[4], s = 0;
@@ -85,6 +86,7 @@ __global__ void __launch_bounds__(1024) k_scan_block(const int* __restrict__ in,
 __global__ void __launch_bounds__(1024) k_scan_one(const int* __restrict__ in,
                                                    int* __restrict__ out, int n,
                                                    int* __restrict__ total_out) {
+  ff_pdl();
   __shared__ int sh[96];
   const int base = threadIdx.x * 4;
   int v[4], s = 0;
@@ -110,6 +112,7 @@ __global__ void __launch_bounds__(1024) k_scan_add(int* __restrict__ out, int n,
                                                    const int* __restrict__ bex,
                                                    const int* __restrict__ bsum, int nb,
                                                    int* __restrict__ total) {
+  ff_pdl();
   const long long base = (long long)blockIdx.x * FF_SCAN_BLOCK + threadIdx.x * 4;
   const int add = bex[blockIdx.x];
 #pragma unroll
@@ -126,6 +129,7 @@ __global__ void __launch_bounds__(1024) k_scan_add(int* __restrict__ out, int n,
 __global__ void k_bin(const double* __restrict__ pos, int n, NbrGrid g, int* __restrict__ cell_of,
                       int4* __restrict__ img, float4* __restrict__ xf,
                       int* __restrict__ cell_count) {
+  ff_pdl();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   int c[3], im[3];
@@ -155,6 +159,7 @@ __global__ void k_bin(const double* __restrict__ pos, int n, NbrGrid g, int* __r
 }
 
 __global__ void k_pos_to_f32(const double* __restrict__ pos, int n, float4* __restrict__ xf) {
+  ff_pdl();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   xf[i] = make_float4((float)pos[3 * (long long)i], (float)pos[3 * (long long)i + 1],
@@ -164,6 +169,7 @@ __global__ void k_pos_to_f32(const double* __restrict__ pos, int n, float4* __re
 __global__ void k_cell_scatter(const int* __restrict__ cell_of, int n,
                                const int* __restrict__ cell_start, int* __restrict__ cell_fill,
                                int* __restrict__ cell_atoms) {
+  ff_pdl();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   const int c = cell_of[i];
@@ -245,6 +251,7 @@ k_verlet_cells(int n, NbrGrid g, const int* __restrict__ cell_of, const int4* __
                const float4* __restrict__ xf, const int* __restrict__ cell_start,
                const int* __restrict__ cell_atoms, float rl2, int vmax, int* __restrict__ vl_j,
                int* __restrict__ vl_s, int* __restrict__ vl_cnt, int* __restrict__ err) {
+  ff_pdl();
   extern __shared__ unsigned long long sh_keys[];
   const int wib = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int i = blockIdx.x * kWarpsPerBlockNbr + wib;
@@ -277,6 +284,7 @@ k_verlet_cells_split(int n, NbrGrid g, const int* __restrict__ cell_of,
                      const int* __restrict__ cell_start, const int* __restrict__ cell_atoms,
                      float rl2, int vmax, int* __restrict__ vl_j, int* __restrict__ vl_s,
                      int* __restrict__ vl_cnt, int* __restrict__ err) {
+  ff_pdl();
   extern __shared__ unsigned long long sh_keys[];
   __shared__ int s_cnt;
   const int lane = threadIdx.x & 31, i = blockIdx.x;
@@ -306,6 +314,7 @@ __global__ void k_verlet_allpairs(int n, const int* __restrict__ sys_of,
                                   const float4* __restrict__ xf, float rl2, int vmax,
                                   int* __restrict__ vl_j, int* __restrict__ vl_s,
                                   int* __restrict__ vl_cnt, int* __restrict__ err) {
+  ff_pdl();
   const int wib = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int i = blockIdx.x * (blockDim.x >> 5) + wib;
   if (i >= n) return;
@@ -336,6 +345,7 @@ __global__ void k_filter(int pass, int n, const float4* __restrict__ xf,
                          const int* __restrict__ vl_cnt, int* __restrict__ cnt_out,
                          const int* __restrict__ row_ptr, int* __restrict__ col,
                          int* __restrict__ shift, int* __restrict__ src) {
+  ff_pdl();
   const int wib = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int i = blockIdx.x * (blockDim.x >> 5) + wib;
   if (i >= n) return;
@@ -372,6 +382,7 @@ __global__ void k_rev_index(long long E, const int* __restrict__ row_ptr,
                             const int* __restrict__ col, const int* __restrict__ shift,
                             const int* __restrict__ src, int* __restrict__ rev,
                             int* __restrict__ err) {
+  ff_pdl();
   const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= E) return;
   const int i = src[e], j = col[e];
@@ -393,6 +404,7 @@ __global__ void k_rev_index(long long E, const int* __restrict__ row_ptr,
 
 __global__ void k_disp_check(const double* __restrict__ x, const double* __restrict__ xref,
                              int n, double lim2, int* __restrict__ flag) {
+  ff_pdl();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   const double dx = x[3 * (long long)i] - xref[3 * (long long)i];
@@ -403,11 +415,13 @@ __global__ void k_disp_check(const double* __restrict__ x, const double* __restr
 }
 
 __global__ void k_check_pos(const double* __restrict__ x, long long n3, int* __restrict__ err) {
+  ff_pdl();
   const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (t < n3 && !isfinite(x[t])) atomicOr(err, FF_FLAG_NONFINITE_POS);
 }
 
 __global__ void k_check_species(const int* __restrict__ Z, int n, int* __restrict__ err) {
+  ff_pdl();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   if (Z[i] < 1 || Z[i] > FF_N_SPECIES) atomicOr(err, FF_FLAG_SPECIES);
@@ -421,16 +435,16 @@ void launch_scan_i32(const int* in, int* out, int n, int* block_sums, int* total
   ProfScope ps_(PC_NEIGHBOR, s);
   const int nb = n > 0 ? ff_cdiv(n, FF_SCAN_BLOCK) : 1;
   if (nb == 1) {   // one block scans it all and writes the total: one launch instead of three
-    k_scan_one<<<1, 1024, 0, s>>>(in, out, n, total);
+    ff_launch(k_scan_one, 1, 1024, 0, s, in, out, n, total);
     ff_count_launch(1);
     return;
   }
   int* bsum = block_sums;
   int* bex = block_sums + FF_SCAN_BLOCK;
   int* tmp = block_sums + 2 * FF_SCAN_BLOCK;
-  k_scan_block<<<nb, 1024, 0, s>>>(in, out, n, bsum);
-  k_scan_block<<<1, 1024, 0, s>>>(bsum, bex, nb, tmp);
-  k_scan_add<<<nb, 1024, 0, s>>>(out, n, bex, bsum, nb, total);
+  ff_launch(k_scan_block, nb, 1024, 0, s, in, out, n, bsum);
+  ff_launch(k_scan_block, 1, 1024, 0, s, bsum, bex, nb, tmp);
+  ff_launch(k_scan_add, nb, 1024, 0, s, out, n, bex, bsum, nb, total);
   ff_count_launch(3);
 }
 
@@ -438,21 +452,21 @@ void launch_bin_atoms(const double* pos, int n, NbrGrid g, int* cell_of, int4* i
                       int* cell_count, cudaStream_t s) {
   ProfScope ps_(PC_NEIGHBOR, s);
   if (n <= 0) return;
-  k_bin<<<ff_cdiv(n, 256), 256, 0, s>>>(pos, n, g, cell_of, img, xf, cell_count);
+  ff_launch(k_bin, ff_cdiv(n, 256), 256, 0, s, pos, n, g, cell_of, img, xf, cell_count);
   ff_count_launch(1);
 }
 
 void launch_pos_to_f32(const double* pos, int n, float4* xf, cudaStream_t s) {
   ProfScope ps_(PC_NEIGHBOR, s);
   if (n <= 0) return;
-  k_pos_to_f32<<<ff_cdiv(n, 256), 256, 0, s>>>(pos, n, xf);
+  ff_launch(k_pos_to_f32, ff_cdiv(n, 256), 256, 0, s, pos, n, xf);
   ff_count_launch(1);
 }
 
 void launch_check_pos(const double* pos, int n, int* err, cudaStream_t s) {
   ProfScope ps_(PC_NEIGHBOR, s);
   if (n <= 0) return;
-  k_check_pos<<<ff_cdiv(3LL * n, 256), 256, 0, s>>>(pos, 3LL * n, err);
+  ff_launch(k_check_pos, ff_cdiv(3LL * n, 256), 256, 0, s, pos, 3LL * n, err);
   ff_count_launch(1);
 }
 
@@ -460,7 +474,8 @@ void launch_cell_scatter(const int* cell_of, int n, const int* cell_start, int* 
                          int* cell_atoms, cudaStream_t s) {
   ProfScope ps_(PC_NEIGHBOR, s);
   if (n <= 0) return;
-  k_cell_scatter<<<ff_cdiv(n, 256), 256, 0, s>>>(cell_of, n, cell_start, cell_fill, cell_atoms);
+  ff_launch(k_cell_scatter, ff_cdiv(n, 256), 256, 0, s, cell_of, n, cell_start, cell_fill,
+            cell_atoms);
   ff_count_launch(1);
 }
 
@@ -471,14 +486,14 @@ void launch_verlet_cells(int n, NbrGrid g, const int* cell_of, const int4* img, 
   if (n <= 0) return;
   const size_t key_bytes = (size_t)vmax * sizeof(unsigned long long);
   if (n <= 1024) {   // up to some seven blocks per SM
-    k_verlet_cells_split<<<n, 32 * kNbrSplit, key_bytes, s>>>(
-        n, g, cell_of, img, xf, cell_start, cell_atoms, rl2, vmax, vl_j, vl_s, vl_cnt, err);
+    ff_launch(k_verlet_cells_split, n, 32 * kNbrSplit, key_bytes, s, n, g, cell_of, img, xf,
+              cell_start, cell_atoms, rl2, vmax, vl_j, vl_s, vl_cnt, err);
     ff_count_launch(1);
     return;
   }
   const size_t smem = kWarpsPerBlockNbr * key_bytes;
-  k_verlet_cells<<<ff_cdiv(n, kWarpsPerBlockNbr), 32 * kWarpsPerBlockNbr, smem, s>>>(
-      n, g, cell_of, img, xf, cell_start, cell_atoms, rl2, vmax, vl_j, vl_s, vl_cnt, err);
+  ff_launch(k_verlet_cells, ff_cdiv(n, kWarpsPerBlockNbr), 32 * kWarpsPerBlockNbr, smem, s, n, g,
+            cell_of, img, xf, cell_start, cell_atoms, rl2, vmax, vl_j, vl_s, vl_cnt, err);
   ff_count_launch(1);
 }
 
@@ -487,8 +502,8 @@ void launch_verlet_allpairs(int n, const int* sys_of, const int* sys_ptr, const 
                             cudaStream_t s) {
   ProfScope ps_(PC_NEIGHBOR, s);
   if (n <= 0) return;
-  k_verlet_allpairs<<<ff_cdiv(n, 4), 128, 0, s>>>(n, sys_of, sys_ptr, xf, rl2, vmax, vl_j, vl_s,
-                                                 vl_cnt, err);
+  ff_launch(k_verlet_allpairs, ff_cdiv(n, 4), 128, 0, s, n, sys_of, sys_ptr, xf, rl2, vmax, vl_j,
+            vl_s, vl_cnt, err);
   ff_count_launch(1);
 }
 
@@ -497,8 +512,8 @@ void launch_filter(int pass, int n, const float4* xf, const float* Lf, float rc2
                    const int* row_ptr, int* col, int* shift, int* src, cudaStream_t s) {
   ProfScope ps_(PC_NEIGHBOR, s);
   if (n <= 0) return;
-  k_filter<<<ff_cdiv(n, 8), 256, 0, s>>>(pass, n, xf, Lf, rc2, vmax, vl_j, vl_s, vl_cnt, cnt,
-                                        row_ptr, col, shift, src);
+  ff_launch(k_filter, ff_cdiv(n, 8), 256, 0, s, pass, n, xf, Lf, rc2, vmax, vl_j, vl_s, vl_cnt,
+            cnt, row_ptr, col, shift, src);
   ff_count_launch(1);
 }
 
@@ -506,7 +521,7 @@ void launch_rev_index(long long E, const int* row_ptr, const int* col, const int
                       const int* src, int* rev, int* err, cudaStream_t s) {
   ProfScope ps_(PC_NEIGHBOR, s);
   if (E <= 0) return;
-  k_rev_index<<<ff_cdiv(E, 256), 256, 0, s>>>(E, row_ptr, col, shift, src, rev, err);
+  ff_launch(k_rev_index, ff_cdiv(E, 256), 256, 0, s, E, row_ptr, col, shift, src, rev, err);
   ff_count_launch(1);
 }
 
@@ -514,13 +529,13 @@ void launch_disp_check(const double* x, const double* xref, int n, double lim2, 
                        cudaStream_t s) {
   ProfScope ps_(PC_NEIGHBOR, s);
   if (n <= 0) return;
-  k_disp_check<<<ff_cdiv(n, 256), 256, 0, s>>>(x, xref, n, lim2, flag);
+  ff_launch(k_disp_check, ff_cdiv(n, 256), 256, 0, s, x, xref, n, lim2, flag);
   ff_count_launch(1);
 }
 
 void launch_check_species(const int* Z, int n, int* err, cudaStream_t s) {
   ProfScope ps_(PC_MISC, s);
   if (n <= 0) return;
-  k_check_species<<<ff_cdiv(n, 256), 256, 0, s>>>(Z, n, err);
+  ff_launch(k_check_species, ff_cdiv(n, 256), 256, 0, s, Z, n, err);
   ff_count_launch(1);
 }

@@ -7,10 +7,11 @@ template <int LMAX, int INK, int OUTK, int CT, bool WB, typename... A>
 void bwd_w(int n_atoms, int C, cudaStream_t s, A... args) {
   const long long teams = (long long)n_atoms * (C / CT);
   if (use_small(teams))
-    k_env_tp_bwd<LMAX, INK, OUTK, CT, WB, true><<<(int)teams, 128, 0, s>>>(n_atoms, C, args...);
+    ff_launch(k_env_tp_bwd<LMAX, INK, OUTK, CT, WB, true>, (int)teams, 128, 0, s, n_atoms, C,
+              args...);
   else
-    k_env_tp_bwd<LMAX, INK, OUTK, CT, WB, false><<<ff_cdiv(teams * CT, 128), 128, 0, s>>>(
-        n_atoms, C, args...);
+    ff_launch(k_env_tp_bwd<LMAX, INK, OUTK, CT, WB, false>, ff_cdiv(teams * CT, 128), 128, 0, s,
+              n_atoms, C, args...);
 }
 
 template <int LMAX, int INK, int OUTK, int CT>

@@ -269,6 +269,7 @@ k_env_tp_fwd(int n_atoms, int C, const int* __restrict__ row_ptr, int e0,
              const float* __restrict__ Vin, const float* __restrict__ thetaT,
              float* __restrict__ X, __nv_bfloat16* __restrict__ Xb, int ldx, int D,
              float* __restrict__ Vout, float* __restrict__ Gam, float inv_sqrt_nu) {
+  ff_pdl();
   using K = TPK<LMAX, INK, OUTK>;
   using R = EdgeRec<LMAX, INK, OUTK, CT, false, WB, SMALL>;
   constexpr bool LAST = R::LAST;
@@ -396,6 +397,7 @@ k_env_tp_bwd(int n_atoms, int C, const int* __restrict__ row_ptr, int e0,
              float* __restrict__ gVin, float* __restrict__ GW, __nv_bfloat16* __restrict__ GWb,
              float* __restrict__ gY_v0, float* __restrict__ gY_env, int gy_stride,
              const float* __restrict__ Gam, float inv_sqrt_nu) {
+  ff_pdl();
   using K = TPK<LMAX, INK, OUTK>;
   using R = EdgeRec<LMAX, INK, OUTK, CT, true, WB, SMALL>;
   constexpr bool LAST = R::LAST;
