@@ -23,6 +23,15 @@ namespace {
 // budget of this path is set by its bf16 operands, unit roundoff 2^-8).  exp(-z) = inf for
 // z < -88 gives 0, the correct limit.
 __device__ __forceinline__ float sigm_fast(float z) { return __fdividef(1.f, 1.f + __expf(-z)); }
+// sigm_fast as 1 / (1 + 2^(-z log2 e)) on the flush-to-zero units: the same bits for every input
+// (checked over all 2^32; the argument of the reciprocal is at least 1, and an exponential below
+// the normal range adds nothing to 1), in two thirds of the instructions
+__device__ __forceinline__ float sigm_ftz(float z) {
+  float e, r;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"(z * -1.4426950408889634f));
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(1.f + e));
+  return r;
+}
 __device__ __forceinline__ float silu_f(float z) { return z * sigm_fast(z); }
 __device__ __forceinline__ float dsilu_f(float z) {
   const float sg = sigm_fast(z);
@@ -130,7 +139,7 @@ __device__ __forceinline__ void epi_batch(const EpiParams& ep, const float4 (&ac
         float gz[4];
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-          const float sg = sigm_fast(z4[j]);
+          const float sg = sigm_ftz(z4[j]);
           gz[j] = ep.alpha2 * fr[i] * o[j] * (sg * (1.f + z4[j] * (1.f - sg)));
           racc[i][0] += o[j] * z4[j] * sg;
         }
@@ -539,15 +548,6 @@ __device__ __forceinline__ void tma_store_2d(const CUtensorMap* map, uint32_t sr
                : "memory");
 }
 
-// sigm_fast on the flush-to-zero units: the same bits for every input (the argument of the
-// reciprocal is at least 1, and an exponential below the normal range adds nothing to 1), in
-// two thirds of the instructions
-__device__ __forceinline__ float sigm_ftz(float z) {
-  float e, r;
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"(z * -1.4426950408889634f));
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(1.f + e));
-  return r;
-}
 __device__ __forceinline__ uint32_t pack_b16(float lo, float hi) {
   const __nv_bfloat162 p = __floats2bfloat162_rn(lo, hi);
   return *reinterpret_cast<const uint32_t*>(&p);
