@@ -127,7 +127,7 @@ int ff_neighbors(ff_ctx* ctx, const double* pos, const int32_t* Z, int n_atoms,
  * more than skin/2 since the last build.  Synchronises `stream` (edge count and flags in one
  * read, and the device error word after the evaluation).
  * Errors: FF_ERR_STATE (no ff_neighbors yet), FF_ERR_CAPACITY, FF_ERR_NONFINITE, FF_ERR_OOM,
- * FF_ERR_CUDA, FF_ERR_TIMEOUT (precision 1: a tensor-core pipeline wait ran out). */
+ * FF_ERR_CUDA, FF_ERR_TIMEOUT (a tensor-core pipeline wait ran out). */
 int ff_energy_forces(ff_ctx* ctx, const double* pos, double* E_sys, float* E_atom, float* F,
                      void* stream);
 

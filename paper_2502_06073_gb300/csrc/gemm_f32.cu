@@ -34,10 +34,10 @@
 // of the products alone measures, 107 us everything but the epilogue); the rest is latency of
 // the splitting and of the epilogue at 18 warps an SM.  The CUDA-core kernel that this one
 // replaced ran at 0.6 of the FP32 FMA peak: all 16 launches of an evaluation took 12.47 ms at
-// 358,000 edges and 67.2 ms at 1.97 million, now 4.50 and 23.8 ms; at 5,500 edges and widths
+// 358,000 edges and 67.2 ms at 1.97 million, now 4.35 and 22.7 ms; at 5,500 edges and widths
 // of 16 to 64, 0.170 and now 0.128 ms, so it serves every size.  Against 64 bits the forces
-// of those evaluations are off by 6.1e-7 and 1.3e-6 (relative, 2-norm), with FP32 FMAs by
-// 7.3e-7 and 1.5e-6.
+// of those evaluations are off by 6.4e-7 and 1.4e-6 (relative, 2-norm), with FP32 FMAs by
+// 7.2e-7 and 1.5e-6.
 #include "tc_ptx.cuh"
 
 namespace {
