@@ -182,7 +182,9 @@ struct ff_ctx {
   int* cell_count = nullptr; int* cell_start = nullptr; int* cell_fill = nullptr;
   int* cell_atoms = nullptr;
   double* xref = nullptr;
-  int* cnt = nullptr; int* row_ptr = nullptr;
+  // row_ptr belongs to the standing list; a list update scans into row_ptr_new, and the two are
+  // exchanged once the update is known to have succeeded
+  int* cnt = nullptr; int* row_ptr = nullptr; int* row_ptr_new = nullptr;
   int* col = nullptr; int* shift = nullptr; int* src = nullptr; int* rev = nullptr;
   long long ecap = 0, E = 0;
   std::vector<int> row_ptr_h;   // [0] and [n] always; all of it when row_ptr_full
@@ -819,17 +821,19 @@ int build_verlet(ff_ctx* c, const double* pos, cudaStream_t s) {
   return set_err(c, FF_ERR_CAPACITY, "neighbour capacity could not be established");
 }
 
-// Edges per atom at distance below the cutoff, their CSR offsets and their number (flags[2]).
+// Edges per atom at distance below the cutoff, their CSR offsets (row_ptr_new) and their number
+// (flags[2]).  Nothing of the standing list is written.
 void enqueue_count(ff_ctx* c, const double* pos, cudaStream_t s, float r2cut, bool have_xf) {
   if (!have_xf) launch_pos_to_f32(pos, c->n, c->xf, s);
   launch_filter(0, c->n, c->xf, c->Lf_d, r2cut, c->vmax, c->vl_j, c->vl_s, c->vl_cnt, c->cnt,
                 nullptr, nullptr, nullptr, nullptr, s);
-  launch_scan_i32(c->cnt, c->row_ptr, c->n, c->scan_tmp, c->flags + 2, s);
+  launch_scan_i32(c->cnt, c->row_ptr_new, c->n, c->scan_tmp, c->flags + 2, s);
 }
 
-// The model list from the counts read back (c->flags_h[2] edges).  The host keeps all CSR
-// offsets only when the list may need several chunks (fill_row_ptr).
-int fill_edges(ff_ctx* c, cudaStream_t s, float r2cut) {
+// The counts read back without an error (c->flags_h[2] edges) become the model list, and what
+// was computed on the one before is given up.  The host keeps all CSR offsets only when the list
+// may need several chunks (fill_row_ptr).
+int take_list(ff_ctx* c, cudaStream_t s, float r2cut) {
   if ((long long)c->n * c->vmax > INT32_MAX) {
     // the int32 CSR offsets wrap beyond 2^31 - 1 edges: count the edges in 64 bits first
     std::vector<int> cnt_h(c->n);
@@ -841,13 +845,15 @@ int fill_edges(ff_ctx* c, cudaStream_t s, float r2cut) {
       return set_err(c, FF_ERR_CAPACITY, "the model list has " + std::to_string(tot) +
                                              " edges (limit 2^31 - 1)");
   }
-  c->E = c->flags_h[2];
-  c->row_ptr_full = false;
-  c->row_ptr_h.resize(c->n + 1);
-  c->row_ptr_h[0] = 0;
-  c->row_ptr_h[c->n] = (int)c->E;
-  if (c->E > c->ecap) {
-    const long long cap = std::max(c->E + c->E / 8 + 1024, 2 * c->ecap);
+  std::swap(c->row_ptr, c->row_ptr_new);
+  c->state_valid = false;
+  c->g_pos = nullptr;
+  c->list_fixed = false;
+  c->E = 0;
+  const long long E = c->flags_h[2];
+  if (E > c->ecap) {
+    const long long cap = std::max(E + E / 8 + 1024, 2 * c->ecap);
+    c->ecap = 0;   // (until every buffer is there)
     FF_TRY(dalloc(c, &c->col, cap));
     FF_TRY(dalloc(c, &c->shift, cap));
     FF_TRY(dalloc(c, &c->src, cap));
@@ -855,6 +861,11 @@ int fill_edges(ff_ctx* c, cudaStream_t s, float r2cut) {
     FF_TRY(dalloc(c, &c->g, cap));
     c->ecap = cap;
   }
+  c->E = E;
+  c->row_ptr_full = false;
+  c->row_ptr_h.resize(c->n + 1);
+  c->row_ptr_h[0] = 0;
+  c->row_ptr_h[c->n] = (int)E;
   launch_filter(1, c->n, c->xf, c->Lf_d, r2cut, c->vmax, c->vl_j, c->vl_s, c->vl_cnt, c->cnt,
                 c->row_ptr, c->col, c->shift, c->src, s);
   launch_rev_index(c->E, c->row_ptr, c->col, c->shift, c->src, c->rev, c->flags, s);
@@ -865,7 +876,9 @@ int fill_edges(ff_ctx* c, cudaStream_t s, float r2cut) {
 // The model list at `r2cut` for positions `pos`, from the standing Verlet list or (build) from
 // a new one.  One read-back and wait in the usual case: the error word, the displacement flag
 // and the edge count together.  check_disp: also rebuild when an atom has moved more than
-// skin/2; the count made on the old list is then thrown away.
+// skin/2; the count made on the old list is then thrown away.  An update that fails leaves the
+// standing model list and the state computed on it as they were (a Verlet list that it had
+// begun to rebuild is built anew by the next update).
 int make_list(ff_ctx* c, const double* pos, cudaStream_t s, float r2cut, bool build,
               bool check_disp) {
   if (check_disp && !build) {
@@ -891,15 +904,13 @@ int make_list(ff_ctx* c, const double* pos, cudaStream_t s, float r2cut, bool bu
       continue;
     }
     if (build) FF_TRY(built_ok(c, pos, s));
-    return fill_edges(c, s, r2cut);
+    return take_list(c, s, r2cut);
   }
   return set_err(c, FF_ERR_CAPACITY, "neighbour capacity could not be established");
 }
 
 int update_neighbors(ff_ctx* c, const double* pos, cudaStream_t s) {
-  FF_TRY(make_list(c, pos, s, c->rc2, !c->built || c->hp.skin <= 0.f, true));
-  c->list_fixed = false;
-  return FF_OK;
+  return make_list(c, pos, s, c->rc2, !c->built || c->hp.skin <= 0.f, true);
 }
 
 // every CSR offset on the host
@@ -1412,7 +1423,8 @@ void ff_destroy(ff_ctx* c) {
   dfree(c->L_d); dfree(c->Lf_d);
   dfree(c->vl_j); dfree(c->vl_s); dfree(c->vl_cnt); dfree(c->cell_of); dfree(c->img); dfree(c->xf);
   dfree(c->cell_count); dfree(c->cell_start); dfree(c->cell_fill); dfree(c->cell_atoms);
-  dfree(c->xref); dfree(c->cnt); dfree(c->row_ptr); dfree(c->col); dfree(c->shift); dfree(c->src);
+  dfree(c->xref); dfree(c->cnt); dfree(c->row_ptr); dfree(c->row_ptr_new);
+  dfree(c->col); dfree(c->shift); dfree(c->src);
   dfree(c->rev); dfree(c->scan_tmp); dfree(c->flags); dfree(c->g); dfree(c->E_atom);
   dfree(c->F_int); dfree(c->esys_tmp); dfree(c->vir_part); dfree(c->nh_buf);
   if (c->flags_h) cudaFreeHost(c->flags_h);
@@ -1459,6 +1471,7 @@ int ff_neighbors(ff_ctx* c, const double* pos, const int32_t* Z, int n_atoms, co
     FF_TRY(dalloc(c, &c->xref, (size_t)n_atoms * 3));
     FF_TRY(dalloc(c, &c->cnt, n_atoms));
     FF_TRY(dalloc(c, &c->row_ptr, n_atoms + 1));
+    FF_TRY(dalloc(c, &c->row_ptr_new, n_atoms + 1));
     FF_TRY(dalloc(c, &c->E_atom, n_atoms));
     FF_TRY(dalloc(c, &c->F_int, (size_t)n_atoms * 3));
   }
