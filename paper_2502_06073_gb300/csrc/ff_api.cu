@@ -1358,6 +1358,15 @@ int graph_eval(ff_ctx* c, const double* pos, double* E_sys, float* E_atom, float
   return FF_OK;
 }
 
+// Waits for a stream at the end of its scope, unless done is set by then.
+struct WaitUnless {
+  cudaStream_t s;
+  bool done = false;
+  ~WaitUnless() {
+    if (!done) cudaStreamSynchronize(s);
+  }
+};
+
 // Rebuild the Verlet list when an atom moved more than skin/2 from its reference.
 int check_rebuild(ff_ctx* c, const double* x, cudaStream_t s) {
   const double lim = 0.5 * (double)c->hp.skin;
@@ -1452,6 +1461,12 @@ int ff_neighbors(ff_ctx* c, const double* pos, const int32_t* Z, int n_atoms, co
   const bool any_pbc = pbc[0] || pbc[1] || pbc[2];
   if (n_sys > 1 && any_pbc)
     return set_err(c, FF_ERR_ARG, "several systems need a fully non-periodic box");
+  // The host arrays that this call copies to the device (box is the caller's).  A copy from
+  // pageable memory may still be reading them when cudaMemcpyAsync returns: they outlive the
+  // wait of make_list, and a return that does not get there waits itself.
+  std::vector<int> sof;
+  const float Lf[3] = {(float)box[0], (float)box[1], (float)box[2]};
+  WaitUnless copied{s};
   const bool resized = n_atoms != c->n;
   c->n = n_atoms;
   c->n_sys = n_sys;
@@ -1495,12 +1510,11 @@ int ff_neighbors(ff_ctx* c, const double* pos, const int32_t* Z, int n_atoms, co
   c->vmax = vm;
   FF_TRY(dalloc_keep(c, &c->vl_j, &c->cap_vlj, (size_t)n_atoms * vm));
   FF_TRY(dalloc_keep(c, &c->vl_s, &c->cap_vls, (size_t)n_atoms * vm));
-  // (host arrays of this call: copies from pageable memory have been staged on return)
   FF_CK(c, cudaMemcpyAsync(c->Z, Z, (size_t)n_atoms * sizeof(int), cudaMemcpyDeviceToDevice, s));
   if (n_sys == 1) {
     FF_CK(c, cudaMemsetAsync(c->sys_of, 0, (size_t)n_atoms * sizeof(int), s));
   } else {
-    std::vector<int> sof(n_atoms);
+    sof.resize(n_atoms);
     for (int k = 0; k < n_sys; ++k)
       for (int i = sp[k]; i < sp[k + 1]; ++i) sof[i] = k;
     FF_CK(c, cudaMemcpyAsync(c->sys_of, sof.data(), (size_t)n_atoms * sizeof(int),
@@ -1508,7 +1522,6 @@ int ff_neighbors(ff_ctx* c, const double* pos, const int32_t* Z, int n_atoms, co
   }
   FF_CK(c, cudaMemcpyAsync(c->sys_ptr, sp.data(), (size_t)(n_sys + 1) * sizeof(int),
                            cudaMemcpyHostToDevice, s));
-  const float Lf[3] = {(float)box[0], (float)box[1], (float)box[2]};
   FF_CK(c, cudaMemcpyAsync(c->L_d, box, 3 * sizeof(double), cudaMemcpyHostToDevice, s));
   FF_CK(c, cudaMemcpyAsync(c->Lf_d, Lf, 3 * sizeof(float), cudaMemcpyHostToDevice, s));
   launch_check_species(c->Z, n_atoms, c->flags, s);
@@ -1521,6 +1534,7 @@ int ff_neighbors(ff_ctx* c, const double* pos, const int32_t* Z, int n_atoms, co
   c->list_fixed = false;
   const int r = make_list(c, pos, s, c->rc2, true, false);
   if (r == FF_ERR_SPECIES) c->bound = was_bound;
+  copied.done = r == FF_OK;
   return r;
 }
 
