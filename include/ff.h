@@ -111,8 +111,9 @@ void ff_destroy(ff_ctx* ctx);
  * membership test  ((x_j - x_i) + s*L)^2 < (rc+skin)^2  evaluated per component
  * without fused multiply-add) and the list at rc used by the model, sorted by
  * (i, j, s).  Synchronises `stream` (reads counts back).
- * Errors: FF_ERR_ARG, FF_ERR_SPECIES, FF_ERR_CAPACITY, FF_ERR_BOX, FF_ERR_OOM,
- * FF_ERR_CUDA. */
+ * Errors: FF_ERR_ARG (the system bound before stays bound); FF_ERR_SPECIES, FF_ERR_OOM,
+ * FF_ERR_CUDA (no system is bound any more); FF_ERR_NONFINITE, FF_ERR_CAPACITY, FF_ERR_BOX (the
+ * new system is bound but has no list yet: an evaluation at other positions builds it). */
 int ff_neighbors(ff_ctx* ctx, const double* pos, const int32_t* Z, int n_atoms,
                  const double box[3], const int pbc[3], const int32_t* sys_ptr, int n_sys,
                  void* stream);
@@ -126,7 +127,8 @@ int ff_neighbors(ff_ctx* ctx, const double* pos, const int32_t* Z, int n_atoms,
  * Re-filters the Verlet list at rc for `pos` and rebuilds it first when an atom moved
  * more than skin/2 since the last build.  Synchronises `stream` (edge count and flags in one
  * read, and the device error word after the evaluation).
- * Errors: FF_ERR_STATE (no ff_neighbors yet), FF_ERR_CAPACITY, FF_ERR_NONFINITE, FF_ERR_OOM,
+ * Errors: FF_ERR_STATE (no ff_neighbors yet), FF_ERR_CAPACITY, FF_ERR_NONFINITE, FF_ERR_BOX (the
+ * list at `pos` cannot be built: the list before and what was computed on it stay), FF_ERR_OOM,
  * FF_ERR_CUDA, FF_ERR_TIMEOUT (a tensor-core pipeline wait ran out). */
 int ff_energy_forces(ff_ctx* ctx, const double* pos, double* E_sys, float* E_atom, float* F,
                      void* stream);

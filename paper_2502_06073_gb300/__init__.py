@@ -188,8 +188,9 @@ class FFModel:
             self._sys_ptr_keep = arr
             sp, ns = ctypes.c_void_p(arr.ctypes.data), arr.shape[0] - 1
         rc = self.lib.ff_neighbors(self._h, _ptr(pos), _ptr(Z), n, b, p, sp, ns, _stream(torch))
+        if ERRORS.get(rc) != "FF_ERR_ARG":   # (refused arguments leave the system bound so far)
+            self.n, self.n_sys = n, ns
         self._check(rc)
-        self.n, self.n_sys = n, ns
         self._Z = Z
         return self
 

@@ -165,6 +165,7 @@ struct ff_ctx {
   bool gemm_fail = false;
   // system
   int n = 0, n_sys = 0, pbc[3] = {0, 0, 0};
+  int n_alloc = 0;            // atoms that the per-atom buffers are sized for
   double box[3] = {0, 0, 0};
   bool bound = false, allpairs = false, built = false;
   NbrGrid grid{};
@@ -182,11 +183,13 @@ struct ff_ctx {
   int* cell_count = nullptr; int* cell_start = nullptr; int* cell_fill = nullptr;
   int* cell_atoms = nullptr;
   double* xref = nullptr;
+  bool xref_set = false;      // xref holds positions of the bound system
   // row_ptr belongs to the standing list; a list update scans into row_ptr_new, and the two are
   // exchanged once the update is known to have succeeded
   int* cnt = nullptr; int* row_ptr = nullptr; int* row_ptr_new = nullptr;
   int* col = nullptr; int* shift = nullptr; int* src = nullptr; int* rev = nullptr;
   long long ecap = 0, E = 0;
+  bool listed = false;        // row_ptr .. rev and E are the model list of the bound system
   std::vector<int> row_ptr_h;   // [0] and [n] always; all of it when row_ptr_full
   bool row_ptr_full = false;
   int* scan_tmp = nullptr;
@@ -795,14 +798,18 @@ int grow_verlet(ff_ctx* c) {
                                            " neighbours within rc + skin (limit " +
                                            std::to_string(FF_MAX_NEIGHBORS) + ")");
   c->vmax = std::min(FF_MAX_NEIGHBORS, ((mx * 5 / 4) + 31) / 32 * 32);
+  c->bound = false;   // (until both buffers are there)
   FF_TRY(dalloc_keep(c, &c->vl_j, &c->cap_vlj, (size_t)c->n * c->vmax));
-  return dalloc_keep(c, &c->vl_s, &c->cap_vls, (size_t)c->n * c->vmax);
+  FF_TRY(dalloc_keep(c, &c->vl_s, &c->cap_vls, (size_t)c->n * c->vmax));
+  c->bound = true;
+  return FF_OK;
 }
 
 int built_ok(ff_ctx* c, const double* pos, cudaStream_t s) {
   if (pos != c->xref)
     FF_CK(c, cudaMemcpyAsync(c->xref, pos, (size_t)c->n * 3 * sizeof(double),
                              cudaMemcpyDeviceToDevice, s));
+  c->xref_set = true;
   c->built = true;
   c->list_gen++;
   return FF_OK;
@@ -849,7 +856,7 @@ int take_list(ff_ctx* c, cudaStream_t s, float r2cut) {
   c->state_valid = false;
   c->g_pos = nullptr;
   c->list_fixed = false;
-  c->E = 0;
+  c->listed = false;
   const long long E = c->flags_h[2];
   if (E > c->ecap) {
     const long long cap = std::max(E + E / 8 + 1024, 2 * c->ecap);
@@ -862,6 +869,7 @@ int take_list(ff_ctx* c, cudaStream_t s, float r2cut) {
     c->ecap = cap;
   }
   c->E = E;
+  c->listed = true;
   c->row_ptr_full = false;
   c->row_ptr_h.resize(c->n + 1);
   c->row_ptr_h[0] = 0;
@@ -1294,9 +1302,10 @@ void graph_reset(ff_ctx* c) {
 
 // The whole Verlet list (rc + skin, as built at the reference positions) becomes the model
 // list: edges beyond rc contribute exactly zero (the envelope and its derivative vanish),
-// so it stays valid while every atom is within skin/2 of its reference position.
-int prepare_fixed(ff_ctx* c, cudaStream_t s) {
-  FF_TRY(make_list(c, c->xref, s, c->rl2, !c->built, false));
+// so it stays valid while every atom is within skin/2 of its reference position (`pos`, when the
+// bound system has had no list yet).
+int prepare_fixed(ff_ctx* c, const double* pos, cudaStream_t s) {
+  FF_TRY(make_list(c, c->xref_set ? c->xref : pos, s, c->rl2, !c->built, false));
   FF_TRY(plan_and_reserve(c, c->fixed_starts, s));
   c->list_fixed = true;
   c->fixed_gen = c->list_gen;
@@ -1309,7 +1318,7 @@ int prepare_fixed(ff_ctx* c, cudaStream_t s) {
 // (and before) the caller's stream.
 int graph_eval(ff_ctx* c, const double* pos, double* E_sys, float* E_atom, float* F,
                cudaStream_t s) {
-  if (!c->list_fixed || c->fixed_gen != c->list_gen) FF_TRY(prepare_fixed(c, s));
+  if (!c->list_fixed || c->fixed_gen != c->list_gen) FF_TRY(prepare_fixed(c, pos, s));
   if (!c->gstream) {
     FF_CK(c, cudaStreamCreateWithFlags(&c->gstream, cudaStreamNonBlocking));
     FF_CK(c, cudaEventCreateWithFlags(&c->ev_a, cudaEventDisableTiming));
@@ -1467,7 +1476,15 @@ int ff_neighbors(ff_ctx* c, const double* pos, const int32_t* Z, int n_atoms, co
   std::vector<int> sof;
   const float Lf[3] = {(float)box[0], (float)box[1], (float)box[2]};
   WaitUnless copied{s};
-  const bool resized = n_atoms != c->n;
+  // the system bound so far is given up here; only a new one that is in place can be evaluated
+  c->bound = false;
+  c->listed = false;
+  c->xref_set = false;
+  c->built = false;
+  c->state_valid = false;
+  c->g_pos = nullptr;
+  c->md_force_pos = nullptr;
+  c->list_fixed = false;
   c->n = n_atoms;
   c->n_sys = n_sys;
   c->sys_ptr_h = sp;
@@ -1475,7 +1492,8 @@ int ff_neighbors(ff_ctx* c, const double* pos, const int32_t* Z, int n_atoms, co
   c->allpairs = n_sys > 1;
   setup_grid(c);
   const float rl = c->hp.rc + c->hp.skin;
-  if (resized || !c->Z) {
+  if (n_atoms != c->n_alloc) {
+    c->n_alloc = 0;   // (until every buffer is there)
     FF_TRY(dalloc(c, &c->Z, n_atoms));
     FF_TRY(dalloc(c, &c->sys_of, n_atoms));
     FF_TRY(dalloc(c, &c->vl_cnt, n_atoms));
@@ -1489,6 +1507,7 @@ int ff_neighbors(ff_ctx* c, const double* pos, const int32_t* Z, int n_atoms, co
     FF_TRY(dalloc(c, &c->row_ptr_new, n_atoms + 1));
     FF_TRY(dalloc(c, &c->E_atom, n_atoms));
     FF_TRY(dalloc(c, &c->F_int, (size_t)n_atoms * 3));
+    c->n_alloc = n_atoms;
   }
   FF_TRY(dalloc_keep(c, &c->sys_ptr, &c->cap_sys_ptr, n_sys + 1));
   FF_TRY(dalloc_keep(c, &c->esys_tmp, &c->cap_esys, n_sys));
@@ -1525,15 +1544,9 @@ int ff_neighbors(ff_ctx* c, const double* pos, const int32_t* Z, int n_atoms, co
   FF_CK(c, cudaMemcpyAsync(c->L_d, box, 3 * sizeof(double), cudaMemcpyHostToDevice, s));
   FF_CK(c, cudaMemcpyAsync(c->Lf_d, Lf, 3 * sizeof(float), cudaMemcpyHostToDevice, s));
   launch_check_species(c->Z, n_atoms, c->flags, s);
-  const bool was_bound = c->bound;
-  c->bound = true;
-  c->built = false;
-  c->state_valid = false;
-  c->g_pos = nullptr;
-  c->md_force_pos = nullptr;
-  c->list_fixed = false;
   const int r = make_list(c, pos, s, c->rc2, true, false);
-  if (r == FF_ERR_SPECIES) c->bound = was_bound;
+  // a list that cannot be built at these positions leaves a system that can be evaluated at others
+  c->bound = r != FF_ERR_SPECIES && r != FF_ERR_OOM && r != FF_ERR_CUDA;
   copied.done = r == FF_OK;
   return r;
 }
@@ -1763,7 +1776,7 @@ int ff_export_params(ff_ctx* c, double* host_buf, size_t cap, size_t* needed) {
 int ff_get_edges(ff_ctx* c, int64_t* n_edges, int32_t* row_ptr, int32_t* col, int32_t* shift,
                  int32_t* rev, size_t cap, void* stream) {
   if (!c) return FF_ERR_ARG;
-  if (!c->bound) return set_err(c, FF_ERR_STATE, "no system bound");
+  if (!c->bound || !c->listed) return set_err(c, FF_ERR_STATE, "no edge list");
   cudaStream_t s = (cudaStream_t)stream;
   if (n_edges) *n_edges = c->E;
   if (!row_ptr && !col && !shift && !rev) return FF_OK;

@@ -44,3 +44,59 @@ def test_batches_divided_differently(ff):
         Es, F = forces(m, step)
         Es_ref, F_ref = forces(ff.FFModel(hp, seed=42), step)
         assert torch.equal(Es, Es_ref) and torch.equal(F, F_ref)
+
+
+def _small(ff, s):
+    m = ff.FFModel(synth.preset("small", skin=0.7), seed=42)
+    m.bind(_dev(s.pos), _dev(s.Z, torch.int32), s.box, s.pbc)
+    return m
+
+
+def test_a_rejected_species_leaves_nothing_bound(ff):
+    """The list of the rejected system is not built, and neither that system nor the one before
+    it can be evaluated: an atomic number outside the table selects no row of it."""
+    s = synth.config1_system()
+    pos, Z = _dev(s.pos), _dev(s.Z, torch.int32)
+    m = _small(ff, s)
+    m.energy_forces(pos)
+    bad = Z.clone()
+    bad[3] = 95
+    with pytest.raises(ff.FFError, match="FF_ERR_SPECIES"):
+        m.bind(pos, bad, s.box, s.pbc)
+    v, mass = torch.zeros_like(pos), _dev(s.masses)
+    for call in (lambda: m.energy_forces(pos), lambda: m.energy_forces_graph(pos),
+                 lambda: m.forces_adjoint(), lambda: m.virial(), lambda: m.edges(),
+                 lambda: m.md(pos.clone(), v, mass, 1, 0.5), lambda: m.autotune(pos)):
+        with pytest.raises(ff.FFError, match="FF_ERR_STATE"):
+            call()
+    m.bind(pos, Z, s.box, s.pbc)
+    ref = _small(ff, s)
+    for a, b in zip(m.energy_forces(pos), ref.energy_forces(pos)):
+        assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("call", ["energy_forces", "energy_forces_graph"])
+def test_positions_rejected_at_the_bind_can_be_replaced(ff, call):
+    """A bind to a larger system at a non-finite position fails; its other data are in place, and
+    an evaluation at good positions is that of a context bound there."""
+    s0 = synth.config1_system()
+    s = synth.water_system(400, L=22.88, seed=7)
+    m = _small(ff, s0)
+    bad = s.pos.copy()
+    bad[17, 2] = np.inf
+    with pytest.raises(ff.FFError, match="FF_ERR_NONFINITE"):
+        m.bind(_dev(bad), _dev(s.Z, torch.int32), s.box, s.pbc)
+    with pytest.raises(ff.FFError, match="FF_ERR_STATE"):
+        m.edges()
+    ref = _small(ff, s)
+    out = []
+    for model in (m, ref):
+        pos = _dev(s.pos)
+        if call == "energy_forces":
+            out.append(model.energy_forces(pos))
+        else:
+            Ea = torch.empty(s.n, dtype=torch.float32, device="cuda")
+            F = torch.empty(s.n, 3, dtype=torch.float32, device="cuda")
+            out.append(model.energy_forces_graph(pos, None, Ea, F))
+    for a, b in zip(*out):
+        assert torch.equal(a, b)
