@@ -769,8 +769,8 @@ void setup_grid(ff_ctx* c) {
   c->ncells = (int)total;
 }
 
-// Enqueue the Verlet list at rc + skin.  A non-finite coordinate sets its error bit; it bins
-// into some cell (the index is clamped) and no pair passes the distance test with it.
+// Enqueue the Verlet list at rc + skin.  A non-finite coordinate sets its error bit; its atom is
+// in no cell and in no pair.
 void enqueue_build(ff_ctx* c, const double* pos, cudaStream_t s) {
   launch_check_pos(pos, c->n, c->flags, s);
   if (c->allpairs) {

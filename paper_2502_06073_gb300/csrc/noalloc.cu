@@ -145,8 +145,8 @@ extern "C" int ff_neighbors_noalloc(const double* pos, int n_atoms, const double
     cudaGetLastError();
     return fail(msg, msg_cap, FF_ERR_CUDA, "clearing the scratch failed");
   }
-  // positions are checked like ff_neighbors checks them; a non-finite coordinate is binned
-  // (clamped into a valid cell) but the call then reports it instead of a list
+  // positions are checked like ff_neighbors checks them; an atom with a non-finite coordinate
+  // falls into no cell, and the call then reports it instead of a list
   launch_check_pos(pos, n_atoms, flags, s);
   launch_bin_atoms(pos, n_atoms, g, cell_of, img, xf, cell_count, s);
   launch_scan_i32(cell_count, cell_start, ncells, scan_tmp, nullptr, s);

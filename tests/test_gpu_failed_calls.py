@@ -96,3 +96,32 @@ def test_graph_replay_after_a_failed_update(ff, kind):
     m.energy_forces_graph(pos, Es, Ea, F)
     for t, r in zip((Es, Ea, F), ref):
         assert torch.equal(t, r)
+
+
+def test_a_list_update_of_non_finite_positions_costs_no_more_than_a_good_one(ff):
+    """An MD run that has blown up: every coordinate is NaN.  The atoms fall into no cell (in one
+    cell together they would be tested pair by pair, 7e10 of them here); the call reports them
+    within three times the time of a good bind."""
+    g = np.arange(64) * 2.2
+    pos = np.stack(np.meshgrid(g, g, g, indexing="ij"), -1).reshape(-1, 3)
+    box, pbc = np.full(3, 64 * 2.2), np.array([True] * 3)
+    pos, Z = _dev(pos), torch.ones(64 ** 3, dtype=torch.int32, device="cuda")
+    bad = torch.full_like(pos, float("nan"))
+    m = ff.FFModel(synth.preset("small"), seed=42)
+
+    def timed(call):
+        a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        a.record()
+        call()
+        b.record()
+        b.synchronize()
+        return a.elapsed_time(b)
+
+    def rejected():
+        with pytest.raises(ff.FFError, match="FF_ERR_NONFINITE"):
+            m.bind(bad, Z, box, pbc)
+
+    m.bind(pos, Z, box, pbc)
+    good = min(timed(lambda: m.bind(pos, Z, box, pbc)) for _ in range(3))
+    t = min(timed(rejected) for _ in range(3))
+    assert t <= 3 * good, (t, good)
