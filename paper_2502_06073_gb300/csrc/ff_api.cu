@@ -168,6 +168,10 @@ struct ff_ctx {
   int n_alloc = 0;            // atoms that the per-atom buffers are sized for
   double box[3] = {0, 0, 0};
   bool bound = false, allpairs = false, built = false;
+  // the stream of the last call, and whether calls have used others since the device was last
+  // waited for (ff_neighbors)
+  cudaStream_t last_stream = nullptr;
+  bool used = false, mixed = false;
   NbrGrid grid{};
   float rl2 = 0.f, rc2 = 0.f;
   int vmax = 0;
@@ -1390,6 +1394,15 @@ int check_rebuild(ff_ctx* c, const double* x, cudaStream_t s) {
   return FF_OK;
 }
 
+// The stream of a call.
+cudaStream_t on_stream(ff_ctx* c, void* stream) {
+  const cudaStream_t s = (cudaStream_t)stream;
+  if (c->used && s != c->last_stream) c->mixed = true;
+  c->used = true;
+  c->last_stream = s;
+  return s;
+}
+
 }  // namespace
 
 // ============================================================================= C ABI
@@ -1452,7 +1465,7 @@ void ff_destroy(ff_ctx* c) {
 int ff_neighbors(ff_ctx* c, const double* pos, const int32_t* Z, int n_atoms, const double box[3],
                  const int pbc[3], const int32_t* sys_ptr, int n_sys, void* stream) {
   if (!c) return FF_ERR_ARG;
-  cudaStream_t s = (cudaStream_t)stream;
+  cudaStream_t s = on_stream(c, stream);
   if (!pos || !Z || !box || !pbc || n_atoms < 1 || n_atoms > (16 << 20))
     return set_err(c, FF_ERR_ARG, "pos, Z, box, pbc must be given and 1 <= n_atoms <= 16M");
   if (n_sys < 1) n_sys = 1;
@@ -1476,6 +1489,12 @@ int ff_neighbors(ff_ctx* c, const double* pos, const int32_t* Z, int n_atoms, co
   std::vector<int> sof;
   const float Lf[3] = {(float)box[0], (float)box[1], (float)box[2]};
   WaitUnless copied{s};
+  // Replays and other work of earlier calls on another stream may still be reading the buffers
+  // that this call writes: allocating them anew waited for the device, keeping them does not.
+  if (c->mixed) {
+    FF_CK(c, cudaDeviceSynchronize());
+    c->mixed = false;
+  }
   // the system bound so far is given up here; only a new one that is in place can be evaluated
   c->bound = false;
   c->listed = false;
@@ -1557,7 +1576,7 @@ int ff_energy_forces(ff_ctx* c, const double* pos, double* E_sys, float* E_atom,
   if (!c->bound) return set_err(c, FF_ERR_STATE, "ff_neighbors must be called first");
   if (!pos) return set_err(c, FF_ERR_ARG, "pos is null");
   c->md_force_pos = nullptr;
-  return evaluate(c, pos, E_sys, E_atom, F, nullptr, F != nullptr, (cudaStream_t)stream);
+  return evaluate(c, pos, E_sys, E_atom, F, nullptr, F != nullptr, on_stream(c, stream));
 }
 
 int ff_forces(ff_ctx* c, const double* grad_E, float* F, void* stream) {
@@ -1565,7 +1584,7 @@ int ff_forces(ff_ctx* c, const double* grad_E, float* F, void* stream) {
   if (!c->state_valid || !c->state_pos)
     return set_err(c, FF_ERR_STATE, "ff_forces needs a preceding ff_energy_forces");
   if (!F) return set_err(c, FF_ERR_ARG, "F is null");
-  cudaStream_t s = (cudaStream_t)stream;
+  cudaStream_t s = on_stream(c, stream);
   if (c->state_chunks == 1) {
     backward_chunk(c, 0, c->n, grad_E, s);
   } else {
@@ -1593,7 +1612,7 @@ int ff_virial(ff_ctx* c, double* W, void* stream) {
     return set_err(c, FF_ERR_STATE, "ff_virial needs a preceding force evaluation (unit seed)");
   FF_TRY(dalloc(c, &c->vir_part, (size_t)c->n_sys * 32 * 9));
   launch_virial(c->sys_ptr, c->n_sys, c->row_ptr, c->src, c->col, c->shift, c->g_pos, c->L_d,
-                c->g, c->vir_part, W, (cudaStream_t)stream);
+                c->g, c->vir_part, W, on_stream(c, stream));
   FF_CK(c, cudaGetLastError());
   return FF_OK;
 }
@@ -1603,7 +1622,7 @@ int ff_md_step(ff_ctx* c, double* x, double* v, const double* mass, int n_steps,
   if (!c) return FF_ERR_ARG;
   if (!c->bound) return set_err(c, FF_ERR_STATE, "ff_neighbors must be called first");
   if (!x || !v || !mass || n_steps < 0) return set_err(c, FF_ERR_ARG, "bad md arguments");
-  cudaStream_t s = (cudaStream_t)stream;
+  cudaStream_t s = on_stream(c, stream);
   if (c->graph_md) {
     // frozen Verlet list + graph replay; the list is rebuilt (and the graph recaptured)
     // when an atom has moved more than skin/2
@@ -1651,7 +1670,7 @@ int ff_energy_forces_graph(ff_ctx* c, const double* pos, double* E_sys, float* E
   if (!c->bound) return set_err(c, FF_ERR_STATE, "ff_neighbors must be called first");
   if (!pos) return set_err(c, FF_ERR_ARG, "pos is null");
   c->md_force_pos = nullptr;
-  return graph_eval(c, pos, E_sys, E_atom, F, (cudaStream_t)stream);
+  return graph_eval(c, pos, E_sys, E_atom, F, on_stream(c, stream));
 }
 
 int ff_autotune(ff_ctx* c, const double* pos, int* slice, int* stages, double* ms_best,
@@ -1659,7 +1678,7 @@ int ff_autotune(ff_ctx* c, const double* pos, int* slice, int* stages, double* m
   if (!c) return FF_ERR_ARG;
   if (!c->bound) return set_err(c, FF_ERR_STATE, "ff_neighbors must be called first");
   if (!pos) return set_err(c, FF_ERR_ARG, "pos is null");
-  cudaStream_t s = (cudaStream_t)stream;
+  cudaStream_t s = on_stream(c, stream);
   if (c->hp.precision == 1) {
     // stages 0 = the launcher's default (2 stages for 256-column slices; the persistent
     // kernel for narrower ones), 1..4 = the non-persistent kernel with that ring depth
@@ -1731,7 +1750,7 @@ int ff_md_nvt(ff_ctx* c, double* x, double* v, const double* mass, int n_steps, 
   if (!c->bound) return set_err(c, FF_ERR_STATE, "ff_neighbors must be called first");
   if (!x || !v || !mass || !thermo || n_steps < 0 || !(T_K > 0.0) || !(tau_fs > 0.0))
     return set_err(c, FF_ERR_ARG, "bad NVT arguments");
-  cudaStream_t s = (cudaStream_t)stream;
+  cudaStream_t s = on_stream(c, stream);
   const double kT = 8.617333262e-5 * T_K;
   FF_TRY(dalloc(c, &c->nh_buf, (size_t)c->n_sys * 2));
   double* ke = c->nh_buf;
@@ -1777,7 +1796,7 @@ int ff_get_edges(ff_ctx* c, int64_t* n_edges, int32_t* row_ptr, int32_t* col, in
                  int32_t* rev, size_t cap, void* stream) {
   if (!c) return FF_ERR_ARG;
   if (!c->bound || !c->listed) return set_err(c, FF_ERR_STATE, "no edge list");
-  cudaStream_t s = (cudaStream_t)stream;
+  cudaStream_t s = on_stream(c, stream);
   if (n_edges) *n_edges = c->E;
   if (!row_ptr && !col && !shift && !rev) return FF_OK;
   if (cap < (size_t)c->E) return set_err(c, FF_ERR_ARG, "buffer too small");

@@ -100,3 +100,36 @@ def test_positions_rejected_at_the_bind_can_be_replaced(ff, call):
             out.append(model.energy_forces_graph(pos, None, Ea, F))
     for a, b in zip(*out):
         assert torch.equal(a, b)
+
+
+def test_a_bind_on_another_stream_waits_for_the_replays_of_the_first(ff):
+    """The second system has the first one's size, so that its lists go into the same buffers,
+    while replays on the first system are still in flight on their own stream."""
+    a = synth.water_system(1365, L=34.44, seed=1001)
+    b = synth.water_system(1365, L=34.44, seed=1002)
+    hp = synth.preset("fm_water")
+    pos_a, Z_a, pos_b, Z_b = (_dev(a.pos), _dev(a.Z, torch.int32), _dev(b.pos),
+                              _dev(b.Z, torch.int32))
+    Ea = [torch.empty(a.n, dtype=torch.float32, device="cuda") for _ in range(2)]
+    F = [torch.empty(a.n, 3, dtype=torch.float32, device="cuda") for _ in range(2)]
+    ref = ff.FFModel(hp, seed=42, precision=1)
+    ref.bind(pos_a, Z_a, a.box, a.pbc)
+    ref.energy_forces_graph(pos_a, None, Ea[0], F[0])
+    ref_b = ff.FFModel(hp, seed=42, precision=1)
+    ref_b.bind(pos_b, Z_b, b.box, b.pbc)
+    out_ref = ref_b.energy_forces(pos_b)
+    m = ff.FFModel(hp, seed=42, precision=1)
+    Es = torch.empty(1, dtype=torch.float64, device="cuda")
+    s1, s2 = torch.cuda.Stream(), torch.cuda.Stream()
+    torch.cuda.synchronize()
+    with torch.cuda.stream(s1):
+        m.bind(pos_a, Z_a, a.box, a.pbc)
+        for _ in range(20):
+            m.energy_forces_graph(pos_a, Es, Ea[1], F[1])
+    with torch.cuda.stream(s2):
+        m.bind(pos_b, Z_b, b.box, b.pbc)
+        out = m.energy_forces(pos_b)
+    torch.cuda.synchronize()
+    assert torch.equal(Ea[0], Ea[1]) and torch.equal(F[0], F[1])
+    for x, y in zip(out, out_ref):
+        assert torch.equal(x, y)
