@@ -21,6 +21,22 @@ void ff_count_launch(int k) { g_launches.fetch_add(k, std::memory_order_relaxed)
 
 static thread_local std::string g_create_err;
 
+// ----------------------------------------------------------------------------- device
+const FfDevice* ff_device() {
+  static PerDevice<FfDevice> devices;
+  int dev = 0;
+  const FfDevice* d = nullptr;
+  if (cudaGetDevice(&dev) == cudaSuccess)
+    d = devices.get(dev, [dev](FfDevice& v) {
+      v.id = dev;
+      return cudaDeviceGetAttribute(&v.n_sm, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess &&
+             cudaDeviceGetAttribute(&v.smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) ==
+                 cudaSuccess;
+    });
+  if (!d) cudaGetLastError();
+  return d;
+}
+
 // ----------------------------------------------------------------------------- profiling
 namespace {
 const char* kProfNames[PC_COUNT] = {"gemm_f32",   "gemm_bf16",  "env_tp_fwd",   "env_tp_bwd",

@@ -9,6 +9,7 @@
 #include <vector>
 
 #include "../../include/ff.h"
+#include "ff_device.h"
 #include "ff_flags.h"
 
 #define FF_MAX_LAYERS 4
@@ -36,6 +37,11 @@ void ff_count_launch(int k);
 
 // ----------------------------------------------------------------------------- helpers
 __host__ __device__ inline int ff_cdiv(long long a, long long b) { return (int)((a + b - 1) / b); }
+
+// SMs of the current device and the largest dynamic + static shared memory of a block there (null
+// if they cannot be read).
+struct FfDevice { int id, n_sm, smem_optin; };
+const FfDevice* ff_device();
 
 // Small launches follow one another without draining the GPU in between: such a kernel may be
 // resident before the one ahead of it has finished.  Every kernel of the library waits in

@@ -997,13 +997,16 @@ template <int MODE, int NW>
 bool launch_nw(const CUtensorMap& ta, const CUtensorMap& ta2, const CUtensorMap& tb, int M, int N,
                int K, int k1c, int nslices, int nbw, int stages, const EpiParams& ep, int* err,
                cudaStream_t s) {
-  static bool attr_set = false;
-  if (!attr_set) {
-    if (cudaFuncSetAttribute(k_gemm_tc<MODE, NW>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             200 * 1024) != cudaSuccess)
-      return false;
-    attr_set = true;
-  }
+  static PerDevice<bool> limit;   // of dynamic shared memory, set on this device
+  const FfDevice* dev = ff_device();
+  if (!dev || !limit.get(dev->id, [](bool& set) {
+        set = cudaFuncSetAttribute(k_gemm_tc<MODE, NW>,
+                                   cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                   200 * 1024) == cudaSuccess;
+        if (!set) cudaGetLastError();
+        return set;
+      }))
+    return false;
   CUtensorMap tx = ta;
   int aux_tma = aux_map<MODE>(&tx, ep, M, N);
   const size_t base_bytes = gemm_pipe_bytes(MODE, NW, stages, nbw) + 1024 + 256;  // align + bars
@@ -1026,27 +1029,22 @@ template <int MODE, bool ROW>
 bool launch_pp(const CUtensorMap& ta, const CUtensorMap& ta2, const CUtensorMap& tb, int M,
                int N, int K, int k1c, int nslices, int nbw, const EpiParams& ep, int* err,
                cudaStream_t s) {
-  static int n_sm = 0;
-  static size_t kMaxSmem = 0;   // the opt-in per-block limit less the static shared memory
-  if (!kMaxSmem) {
-    int dev = 0, optin = 0;
+  // dynamic shared memory, its limit set on this device: the opt-in limit of a block less the
+  // static shared memory
+  static PerDevice<size_t> limit;
+  const FfDevice* dev = ff_device();
+  const size_t* smem = !dev ? nullptr : limit.get(dev->id, [dev](size_t& lim) {
     cudaFuncAttributes fa{};
-    if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) !=
-            cudaSuccess ||
-        cudaFuncGetAttributes(&fa, k_gemm_pp<MODE, ROW>) != cudaSuccess) {
-      cudaGetLastError();
-      return false;
+    if (cudaFuncGetAttributes(&fa, k_gemm_pp<MODE, ROW>) == cudaSuccess) {
+      lim = (size_t)dev->smem_optin - fa.sharedSizeBytes;
+      if (cudaFuncSetAttribute(k_gemm_pp<MODE, ROW>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               (int)lim) == cudaSuccess)
+        return true;
     }
-    const size_t lim = (size_t)optin - fa.sharedSizeBytes;
-    if (cudaFuncSetAttribute(k_gemm_pp<MODE, ROW>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)lim) != cudaSuccess) {
-      cudaGetLastError();
-      return false;
-    }
-    kMaxSmem = lim;
-  }
+    cudaGetLastError();
+    return false;
+  });
+  if (!smem) return false;
   CUtensorMap tx = ta, tx2 = ta, to = ta;
   int aux_tma = 0;
   if constexpr (ROW) {
@@ -1066,10 +1064,10 @@ bool launch_pp(const CUtensorMap& ta, const CUtensorMap& ta2, const CUtensorMap&
   const size_t fixed = (size_t)PP_EW * pp_warp_bytes<MODE, ROW>() + 1024 + 512;   // epilogue warps,
                                                                              // alignment, barriers
   int stages = 4;
-  while (stages > 1 && pp_ring_bytes(stages, nbw) + fixed > kMaxSmem) --stages;
-  if (pp_ring_bytes(stages, nbw) + fixed > kMaxSmem) return false;
+  while (stages > 1 && pp_ring_bytes(stages, nbw) + fixed > *smem) --stages;
+  if (pp_ring_bytes(stages, nbw) + fixed > *smem) return false;
   const int ntiles = ff_cdiv(M, TM) * nslices;
-  const int grid = ntiles < n_sm ? ntiles : n_sm;
+  const int grid = ntiles < dev->n_sm ? ntiles : dev->n_sm;
   ff_launch_work(ntiles, k_gemm_pp<MODE, ROW>, grid, pp_threads<MODE>(),
                  pp_ring_bytes(stages, nbw) + fixed, s, ta, ta2, tb, tx, tx2, to, M, N, K, k1c,
                  nslices, nbw, stages, aux_tma, ep, err);

@@ -615,24 +615,21 @@ template <int MODE>
 bool launch_fs(const CUtensorMap& tb, const float* A, int lda, const float* A2, int lda2, int M,
                int N, int K1, int K2, int nslices, int nbw, const EpiParams& ep, int* err,
                cudaStream_t s) {
-  static int n_sm = 0;
-  if (!n_sm) {
-    int dev = 0, sms = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-        cudaFuncSetAttribute(k_gemm_fs<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             226 * 1024) != cudaSuccess) {
-      cudaGetLastError();
-      return false;
-    }
-    n_sm = sms;
-  }
+  static PerDevice<bool> limit;   // of dynamic shared memory, set on this device
+  const FfDevice* dev = ff_device();
+  if (!dev || !limit.get(dev->id, [](bool& set) {
+        set = cudaFuncSetAttribute(k_gemm_fs<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                   226 * 1024) == cudaSuccess;
+        if (!set) cudaGetLastError();
+        return set;
+      }))
+    return false;
   // ring, tiles, epilogue inputs, alignment, barriers
   const size_t bytes = fs_stages<MODE>() * (3 * (size_t)FS_ASLICE + 3 * (size_t)nbw * FS_TK * 2) +
                        FS_EW * 32 * 16 * 4 + FS_EW * fs_auxn<MODE>() * fs_naux<MODE>() * 2048 +
                        1024 + 256;
   const int ntiles = ff_cdiv(M, TM) * nslices;
-  ff_launch_work(ntiles, k_gemm_fs<MODE>, ntiles < n_sm ? ntiles : n_sm, FS_THREADS, bytes, s, tb,
+  ff_launch_work(ntiles, k_gemm_fs<MODE>, ntiles < dev->n_sm ? ntiles : dev->n_sm, FS_THREADS, bytes, s, tb,
                  A, lda, A2, lda2, M, N, K1, K2, nslices, nbw, ep, err);
   return true;
 }

@@ -573,15 +573,8 @@ k_env_tp_bwd(int n_atoms, int C, const int* __restrict__ row_ptr, int e0,
 // 130 and 79, 512 teams 420 and 335, but 2,048 teams 451 and 492 (C = 32), 308 and 392 (C = 128),
 // 4,095 teams 1,738 and 2,129.
 inline bool use_small(long long teams) {
-  static int n_sm = 0;
-  if (!n_sm) {
-    int dev = 0, sms = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-      cudaGetLastError();
-    n_sm = sms > 0 ? sms : 1;
-  }
-  return teams <= 4LL * n_sm;
+  const FfDevice* dev = ff_device();
+  return dev && teams <= 4LL * dev->n_sm;
 }
 
 // (input kind, output kind) of every layer of a 1- to 4-layer model; see TPK above.
