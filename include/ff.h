@@ -88,8 +88,8 @@ typedef struct ff_ctx ff_ctx;
  * Model Training) in the documented tensor order, uploads them to the current device.
  * *out receives the handle (NULL on failure).  Environment read here: FF_WORKSPACE_MB
  * (per-chunk workspace budget in MiB; default 120 GB or 60 % of the free device memory)
- * and FF_TEST_STALL_ONCE (tests of the timeout path only: with precision 1 the context's
- * first tensor-core GEMM withholds a completion signal, so a bounded device wait runs out
+ * and FF_TEST_STALL_ONCE (tests of the timeout path only: the context's first
+ * tensor-core GEMM withholds a completion signal, so a bounded device wait runs out
  * and that evaluation returns FF_ERR_TIMEOUT).  Errors: FF_ERR_ARG, FF_ERR_OOM,
  * FF_ERR_CUDA. */
 int ff_create(ff_ctx** out, const ff_hparams* hp, uint64_t seed);

@@ -979,15 +979,15 @@ void plan_chunks(const ff_ctx* c, long long cap, std::vector<int>& starts) {
 void mlp_gemm(ff_ctx* c, int mode, long long M, int N, int K, const float* A32,
               const __nv_bfloat16* Ab, int lda, const __nv_bfloat16* Wt_s,
               const __nv_bfloat16* Wt_b, const EpiParams& ep, cudaStream_t s) {
-  if (c->hp.precision == 0) {
-    if (!launch_gemm_f32(mode, (int)M, N, K, A32, lda, Wt_s, K, ep, c->flags, s))
-      c->gemm_fail = true;
-    return;
-  }
   EpiParams e2 = ep;
   if (c->test_stall_pending) {
     e2.test_stall = 1;
     c->test_stall_pending = false;
+  }
+  if (c->hp.precision == 0) {
+    if (!launch_gemm_f32(mode, (int)M, N, K, A32, lda, Wt_s, K, e2, c->flags, s))
+      c->gemm_fail = true;
+    return;
   }
   if (!launch_gemm_bf16(mode, (int)M, N, K, Ab, lda, Wt_b, K, e2, c->flags, s, c->tune_slice,
                         c->tune_stages))
@@ -1434,7 +1434,7 @@ int ff_create(ff_ctx** out, const ff_hparams* hp, uint64_t seed) {
   ff_ctx* c = new ff_ctx();
   c->hp = *hp;
   c->seed = seed;
-  c->test_stall_pending = hp->precision == 1 && getenv("FF_TEST_STALL_ONCE") != nullptr;
+  c->test_stall_pending = getenv("FF_TEST_STALL_ONCE") != nullptr;
   build_structure(c);
   int r = upload_weights(c);
   if (r == FF_OK) r = dalloc(c, &c->flags, 4);
