@@ -15,23 +15,11 @@
 //                     columns at a time, fused element-wise op, stores.
 // Every mbarrier wait is bounded; a timeout sets FF_FLAG_TIMEOUT in the error word and the
 // CTA drains what it issued, frees its tensor memory and returns.
+#include "sigmoid.cuh"
 #include "tc_ptx.cuh"
 
 namespace {
 
-// Logistic sigmoid from the hardware exponential and fast division (a few ulp; the error
-// budget of this path is set by its bf16 operands, unit roundoff 2^-8).  exp(-z) = inf for
-// z < -88 gives 0, the correct limit.
-__device__ __forceinline__ float sigm_fast(float z) { return __fdividef(1.f, 1.f + __expf(-z)); }
-// sigm_fast as 1 / (1 + 2^(-z log2 e)) on the flush-to-zero units: the same bits for every input
-// (checked over all 2^32; the argument of the reciprocal is at least 1, and an exponential below
-// the normal range adds nothing to 1), in two thirds of the instructions
-__device__ __forceinline__ float sigm_ftz(float z) {
-  float e, r;
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"(z * -1.4426950408889634f));
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(1.f + e));
-  return r;
-}
 __device__ __forceinline__ float silu_f(float z) { return z * sigm_fast(z); }
 __device__ __forceinline__ float dsilu_f(float z) {
   const float sg = sigm_fast(z);

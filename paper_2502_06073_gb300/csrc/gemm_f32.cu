@@ -38,6 +38,7 @@
 // of 16 to 64, 0.170 and now 0.128 ms, so it serves every size.  Against 64 bits the forces
 // of those evaluations are off by 6.4e-7 and 1.4e-6 (relative, 2-norm), with FP32 FMAs by
 // 7.2e-7 and 1.5e-6.
+#include "sigmoid.cuh"
 #include "tc_ptx.cuh"
 
 namespace {
@@ -97,16 +98,6 @@ __device__ __forceinline__ void fs_cp16(uint32_t dst, const float* src) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
 }
 
-// Logistic sigmoid from expf and the hardware reciprocal with one Newton step,
-// r' = r + r (1 - d r): within about an ulp, and without the branch of the IEEE division,
-// which took a fifth of the SiLU epilogues' time.  The clamp keeps d finite (the sigmoid at
-// -80 is 2e-35).
-__device__ __forceinline__ float sigm_nr(float z) {
-  const float d = 1.f + expf(fminf(-z, 80.f));
-  float r;   // d in [1, 6e34]: no denormals either side
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(d));
-  return fmaf(r, fmaf(-d, r, 1.f), r);
-}
 __device__ __forceinline__ float silu_nr(float z) { return z * sigm_nr(z); }
 __device__ __forceinline__ float dsilu_nr(float z) {
   const float sg = sigm_nr(z);
