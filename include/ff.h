@@ -62,8 +62,11 @@ enum {
  *   latent[]          widths of the per-layer latent MLP (last must equal D)
  *   edge_eng[]        hidden widths of the linear edge-energy MLP (output width 1 implied)
  *   avg_num_neighbors nu, normalisation of the environment sum
- *   precision         0 = FP32 everywhere (the dense layers as tensor-core products of three
- *                     bf16 slices per operand, at least as accurate as FP32 FMAs); 1 = BF16 latent MLPs on the tensor cores with
+ *   precision         0 = FP32 everywhere.  The dense layers are tensor-core products of three
+ *                     bf16 slices per operand, with an error relative to the largest elements of
+ *                     a row's 32-element chunks; with these weights (uniform draws) energies and
+ *                     forces are no further from 64 bits than with FP32 FMAs.
+ *                     1 = BF16 latent MLPs on the tensor cores with
  *                     FP32 accumulation: GEMM operands, the residual stream x^L, the
  *                     stored pre-activations and the env-projection outputs (the
  *                     env weights w^L, widened to FP32 where the tensor product reads

@@ -52,3 +52,21 @@ extern "C" int shim_check_sigmoid(int which, unsigned* worst) {
   else k_check_sigmoid<2><<<1216, 256>>>(worst);
   return (int)cudaDeviceSynchronize();
 }
+
+// out [M][N] = [A | A2] B by the FP32 GEMM, B^T = [W1 | W2] given as FP32 rows (K2 = 0: A, W1
+// alone).  slices: 3 N split_ld(K1, K2) bf16 of device memory; err: the device error word.
+extern "C" int shim_gemm_f32(const float* A, const float* A2, const float* W1, const float* W2,
+                             int M, int N, int K1, int K2, __nv_bfloat16* slices, float* out,
+                             int* err) {
+  launch_split_weights(W1, N, K1, W2, K2, 1.0, slices, nullptr);
+  EpiParams ep{};
+  ep.alpha = 1.f;
+  ep.out = out;
+  ep.ldo = N;
+  if (!launch_gemm_f32(EPI_STORE, M, N, K1, A, K1, slices, split_ld(K1, K2), ep, err, nullptr,
+                       K2 > 0 ? A2 : nullptr, K2, K2))
+    return -1;
+  return (int)cudaDeviceSynchronize();
+}
+
+extern "C" int shim_split_ld(int K1, int K2) { return split_ld(K1, K2); }
