@@ -994,7 +994,7 @@ void mlp_gemm(ff_ctx* c, int mode, long long M, int N, int K, const float* A32,
     c->gemm_fail = true;
 }
 
-// Whether the GEMMs are the persistent ones, which write row sums per 128-column slice.
+// Whether all GEMMs are the persistent ones, with row sums per 128-column slice in gfp.
 bool slice_sums(const ff_ctx* c) {
   return c->hp.precision == 0 || (c->tune_stages == 0 && c->tune_slice == 128);
 }
@@ -1070,8 +1070,11 @@ void forward_chunk(ff_ctx* c, const double* pos, int a0, int a1, float* E_atom, 
         el.wv = c->w_eff;
         el.outb = c->GZL; el.ldob = c->D;
         el.out = c->GZLf; el.ldo = c->D;
+        // the envelope-gradient seed: slots of 128 columns, or, where the adjoint takes it from
+        // one array, that array.  The readout of D <= 128 with tiles (256, 0) is the persistent
+        // kernel too; its only slot is then the array.
         el.eout = c->E_edge; el.gfo = c->gfL;
-        el.gfp = c->gfp; el.gfp_ld = c->wcap;
+        el.gfp = slice_sums(c) ? c->gfp : c->gfL; el.gfp_ld = c->wcap;
         mlp_gemm(c, EPI_HEAD, Ec, wout, fan, A32, Ab, lda, c->WlatT_s[L][k],
                  c->WlatT_b[L][k], el, s);
         break;
