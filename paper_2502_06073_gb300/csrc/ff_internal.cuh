@@ -47,7 +47,7 @@ const FfDevice* ff_device();
 // resident before the one ahead of it has finished.  Every kernel of the library waits in
 // ff_pdl, before it touches memory, until that one is complete and its writes are visible (so
 // are, through it, all earlier ones), and then lets the next kernel in.
-// Small: at most two blocks (or tiles of a persistent kernel) per SM.  96 atoms, 33 launches a
+// Small: at most two blocks (or tiles of a persistent kernel) per SM of the 152.  96 atoms, 33 launches a
 // call: 320 -> 261 us.  For every launch it cost more than it gave: 68,000 edges 1,016 -> 1,202
 // us, 10.4 million 82.6 -> 86.3 ms (blocks let in early run under the shared-memory split of
 // the kernel ahead, with little L1).

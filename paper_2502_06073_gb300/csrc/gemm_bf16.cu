@@ -1135,9 +1135,6 @@ bool launch_gemm_bf16(int mode, int M, int N, int K, const __nv_bfloat16* A, int
   } else {
     ta2 = ta;
   }
-  // default: 2 stages for 256-column slices (<= 96 KB: two CTAs per SM), 1 for the 4-warp
-  // CTAs of narrower slices (<= 32 KB: four per SM, which overlap each other's loads);
-  // the autotuner may ask for 2..4
   // default: slices of up to 128 columns run the persistent kernel (stages 0: it picks the
   // deepest ring that fits), 256-column slices two stages (<= 96 KB: two CTAs per SM); the
   // autotuner may ask for the non-persistent kernel with 1..4 stages

@@ -285,6 +285,10 @@ k_verlet_cells(int n, NbrGrid g, const int* __restrict__ cell_of, const int4* __
 // them: for few atoms, where a warp walking 27 cells one after the other (a chain of three
 // dependent loads each) is all there is on an SM.  96 atoms: 25 -> 9 us.  The keys land in any
 // order; their ranks do not depend on it.
+// All list kernels of a bind, us, with a warp and with a block per atom, at rc + skin = 5 A and
+// at 7 A (0.09 atoms per A^3): 96 atoms 73 and 61, 85 and 65; 512 80 and 66, 97 and 75; 1,000
+// 84 and 71, 100 and 80; 2,197 88 and 81, 104 and 96; 4,096 104 and 101, 131 and 124.  The line
+// (launch_verlet_cells) lies at 1,024 atoms, well inside the range where it gains.
 constexpr int kNbrSplit = 8;
 __global__ void __launch_bounds__(32 * kNbrSplit)
 k_verlet_cells_split(int n, NbrGrid g, const int* __restrict__ cell_of,
@@ -493,7 +497,7 @@ void launch_verlet_cells(int n, NbrGrid g, const int* cell_of, const int4* img, 
   ProfScope ps_(PC_NEIGHBOR, s);
   if (n <= 0) return;
   const size_t key_bytes = (size_t)vmax * sizeof(unsigned long long);
-  if (n <= 1024) {   // up to some seven blocks per SM
+  if (n <= 1024) {   // up to some seven blocks per SM; figures at the kernel
     ff_launch(k_verlet_cells_split, n, 32 * kNbrSplit, key_bytes, s, n, g, cell_of, img, xf,
               cell_start, cell_atoms, rl2, vmax, vl_j, vl_s, vl_cnt, err);
     ff_count_launch(1);
