@@ -115,8 +115,9 @@ void ff_destroy(ff_ctx* ctx);
  * without fused multiply-add) and the list at rc used by the model, sorted by
  * (i, j, s).  Synchronises `stream` (reads counts back).
  * Errors: FF_ERR_ARG (the system bound before stays bound); FF_ERR_SPECIES, FF_ERR_OOM,
- * FF_ERR_CUDA (no system is bound any more); FF_ERR_NONFINITE, FF_ERR_CAPACITY, FF_ERR_BOX (the
- * new system is bound but has no list yet: an evaluation at other positions builds it). */
+ * FF_ERR_CUDA (no system is bound any more); FF_ERR_NONFINITE, FF_ERR_CAPACITY, FF_ERR_BOX, or
+ * FF_ERR_TIMEOUT of an earlier replay (the new system is bound but has no list yet: the next
+ * evaluation builds it, at positions where it can be built). */
 int ff_neighbors(ff_ctx* ctx, const double* pos, const int32_t* Z, int n_atoms,
                  const double box[3], const int pbc[3], const int32_t* sys_ptr, int n_sys,
                  void* stream);

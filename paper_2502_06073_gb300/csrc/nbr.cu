@@ -128,8 +128,7 @@ __global__ void __launch_bounds__(1024) k_scan_add(int* __restrict__ out, int n,
 // ------------------------------------------------------------------ binning
 // An atom with a non-finite coordinate falls into no cell (cell_of = -1): its list is empty and
 // no other atom looks at it.  The call reports it, and no cell fills up with such atoms, whose
-// pairs would all be tested (2.6e5 atoms, every coordinate NaN: 437 ms; now below a good bind's
-// 2.6 ms).
+// pairs would all be tested (2.6e5 atoms, every coordinate NaN: 437 ms; now 0.3, a good bind 2.6).
 __global__ void k_bin(const double* __restrict__ pos, int n, NbrGrid g, int* __restrict__ cell_of,
                       int4* __restrict__ img, float4* __restrict__ xf,
                       int* __restrict__ cell_count) {
