@@ -634,8 +634,9 @@ bool launch_fs(const CUtensorMap& tb, const float* A, int lda, const float* A2, 
                        FS_EW * 32 * 16 * 4 + FS_EW * fs_auxn<MODE>() * fs_naux<MODE>() * 2048 +
                        1024 + 256;
   const int ntiles = ff_cdiv(M, TM) * nslices;
-  ff_launch_work(ntiles, k_gemm_fs<MODE>, ntiles < dev->n_sm ? ntiles : dev->n_sm, FS_THREADS, bytes, s, tb,
-                 A, lda, A2, lda2, M, N, K1, K2, nslices, nbw, ep, err);
+  const int grid = ntiles < dev->n_sm ? ntiles : dev->n_sm;
+  ff_launch_work(ntiles, k_gemm_fs<MODE>, grid, FS_THREADS, bytes, s, tb, A, lda, A2, lda2, M, N,
+                 K1, K2, nslices, nbw, ep, err);
   return true;
 }
 
